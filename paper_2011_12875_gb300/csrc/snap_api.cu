@@ -77,6 +77,9 @@ struct snap_ctx {
   int nbparts = 0;
   void* d_root = nullptr;
   void* d_hscale = nullptr;
+  unsigned* d_pair_idx = nullptr;  // closed form of u (HostTables::pair_*)
+  void* d_pair_scale = nullptr;
+  void* d_pair_ab = nullptr;
   int* d_yslice = nullptr;
   int* d_ysched = nullptr;  // lane schedule of the warp-per-atom compute_Y
   int ysched_m = 0;
@@ -518,6 +521,9 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
   }
   a.rootpq = c->d_root;
   a.hscale = c->d_hscale;
+  a.pair_idx = c->d_pair_idx;
+  a.pair_scale = c->d_pair_scale;
+  a.pair_ab = c->d_pair_ab;
   return a;
 }
 
@@ -639,8 +645,7 @@ int enqueue(snap_ctx* c, int n, const double* pos, const double* box, const int*
   }
   SNAP_CUDA(c, mixed ? snap::launch_yi<float>(a, s) : snap::launch_yi<double>(a, s));
   SNAP_CUDA(c, mark());
-  SNAP_CUDA(c, colk ? (mixed ? snap::launch_de_col<float>(a, s) : snap::launch_de_col<double>(a, s))
-                    : (mixed ? snap::launch_de<float>(a, s) : snap::launch_de<double>(a, s)));
+  SNAP_CUDA(c, mixed ? snap::launch_de<float>(a, s) : snap::launch_de<double>(a, s));
   SNAP_CUDA(c, mark());
   a.hflags = c->d_hflags;  // the force kernel ends the evaluation
   SNAP_CUDA(c, mixed ? snap::launch_force<float>(a, s) : snap::launch_force<double>(a, s));
@@ -755,8 +760,7 @@ int launch_batch(snap_ctx* c, const double* pos, double* energy, double* forces,
     nl += 2;
   }
   SNAP_CUDA(c, mixed ? snap::launch_yi<float>(a, s) : snap::launch_yi<double>(a, s));
-  SNAP_CUDA(c, colk ? (mixed ? snap::launch_de_col<float>(a, s) : snap::launch_de_col<double>(a, s))
-                    : (mixed ? snap::launch_de<float>(a, s) : snap::launch_de<double>(a, s)));
+  SNAP_CUDA(c, mixed ? snap::launch_de<float>(a, s) : snap::launch_de<double>(a, s));
   a.hflags = c->d_hflags;  // the force kernel ends the evaluation (the virial sums use no flag)
   SNAP_CUDA(c, mixed ? snap::launch_force<float>(a, s) : snap::launch_force<double>(a, s));
   c->flags_dirty = false;
@@ -1070,6 +1074,13 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
   if (!rc) rc = upload(c, &c->d_ysched, c->tab.lane_outputs(32, &c->ysched_m));
   if (!rc) rc = upload_r(c, &c->d_root, c->tab.rootpq);
   if (!rc) rc = upload_r(c, &c->d_hscale, c->tab.half_scale);
+  if (!rc) rc = upload(c, &c->d_pair_idx, c->tab.pair_idx);
+  if (!rc) {
+    std::vector<double> w(c->tab.pair_norm);  // the weighted Y of the fused dE
+    for (size_t k = 0; k < w.size(); ++k) w[k] *= c->tab.pair_weight[k];
+    rc = upload_r(c, &c->d_pair_scale, w);
+  }
+  if (!rc) rc = upload_r(c, &c->d_pair_ab, c->tab.pair_ab);
   if (!rc) rc = upload_yrec(c);
   if (!rc) rc = upload_brec(c);
   if (!rc) rc = upload(c, &c->d_bchunk_term, c->tab.bchunk_term);
@@ -1658,6 +1669,9 @@ int snap_destroy(snap_ctx* c) {
   c->bpart_cache.clear();
   dfree(c->d_root);
   dfree(c->d_hscale);
+  dfree(c->d_pair_idx);
+  dfree(c->d_pair_scale);
+  dfree(c->d_pair_ab);
   for (auto& kv : c->yslice_cache) cudaFree(kv.second);
   c->yslice_cache.clear();
   c->d_yslice = nullptr;

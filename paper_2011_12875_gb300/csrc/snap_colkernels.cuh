@@ -41,27 +41,6 @@ __device__ __forceinline__ c2<R> mk(R re, R im) {
   return c;
 }
 
-// sqrt(k) for the small integers of the recursion, folded at compile time.
-template <typename R>
-__device__ __forceinline__ constexpr R sqrt_int(int k) {
-  return k == 0   ? R(0)
-         : k == 1 ? R(1)
-         : k == 2 ? R(1.4142135623730950488)
-         : k == 3 ? R(1.7320508075688772935)
-         : k == 4 ? R(2)
-         : k == 5 ? R(2.2360679774997896964)
-         : k == 6 ? R(2.4494897427831780982)
-         : k == 7 ? R(2.6457513110645905905)
-         : k == 8 ? R(2.8284271247461900976)
-         : k == 9 ? R(3)
-         : k == 10 ? R(3.1622776601683793320)
-         : k == 11 ? R(3.3166247903553998491)
-         : k == 12 ? R(3.4641016151377545871)
-         : k == 13 ? R(3.6055512754639892931)
-         : k == 14 ? R(3.7416573867739413856)
-                   : R(3.8729833462074168852);
-}
-
 // Compile-time loop B..E (inclusive): f(std::integral_constant<int, k>).
 template <int B, int E, typename F>
 __device__ __forceinline__ void static_for(F&& f) {
@@ -74,13 +53,6 @@ __device__ __forceinline__ void static_for(F&& f) {
 template <typename R>
 __device__ __forceinline__ R shfl_up(R v) {
   return __shfl_up_sync(kFull, v, 1);
-}
-
-// Weight of a half-layout element in a full-matrix contraction (see
-// snap_kernels.cu): 2 below the middle column, on it 2 / 1 / 0.
-__device__ __forceinline__ int hweight(int t, int ma, int mb) {
-  if (2 * mb < t) return 2;
-  return ma < mb ? 2 : (ma == mb ? 1 : 0);
 }
 
 // Lane layout: NC = J2/2 + 1 lanes per pair, P pairs per warp.
@@ -566,242 +538,6 @@ __global__ void __launch_bounds__(64, ui_min_ctas<R, J2>()) tan_col_kernel(WorkA
   }
 }
 
-template <typename R>
-constexpr int de_max_warps() { return sizeof(R) == 4 ? 16 : 8; }
-
-// --------------------------------------- fused dU + dE/dr, reverse mode
-// Same lane layout (P pairs a warp, a lane per column); the CTA's atoms have
-// their weighted Y_i in shared memory (launch shape below).
-// For one pair, S(a, b) = Re sum_t Y_t : conj(u_t) is a real function of the
-// Cayley-Klein parameters; its gradient comes from one
-// forward pass of the recursion (each lane stores its column of every layer
-// in shared memory) and one adjoint pass through the same recursion, with
-// the adjoint lambda_t of a column in registers:
-//   lambda_{t-1}[m][mb] = Yw_{t-1}[m][mb] + a A - b B,
-//   A = sqrt((t-m)/(t-mb)) lambda_t[m][mb],  B = sqrt((m+1)/(t-mb)) lambda_t[m+1][mb],
-//   g_a += conj(A) u_{t-1}[m][mb],           g_b -= conj(B) u_{t-1}[m][mb],
-// plus, for even t, the part of layer t's column t/2 that read the mirror of
-// column t/2-1 (its adjoint comes one lane down by shuffle).  Then
-//   dE_i/dr_ik = S grad f_c + f_c (<g_a, da/dr> + <g_b, db/dr>)   (Eq. snapforce2).
-template <typename R>
-__device__ __forceinline__ R shfl_down(R v) {
-  return __shfl_down_sync(kFull, v, 1);
-}
-
-// FP32: 128 registers (up to 16 warps a CTA); FP64 may use them all, up to 8
-// warps (its FP64 pipe saturates with few warps, and the columns are twice
-// the size).
-//
-// CTA = A consecutive atoms and NW warps (A is a launch parameter, planned
-// by launch_de_rev_col_t).  The CTA's pairs, atom after atom, are taken in
-// passes of P pairs; warp w takes passes w, w + NW, ...  Every pass but the
-// CTA's last is full whatever the atoms' counts, and with A below NW x
-// (passes per warp) x P / (pairs per atom) no warp takes more passes than
-// planned (the time of a CTA is that of its longest chain of passes).  A
-// pair's arithmetic does not depend on its pass or its warp.
-//
-// QUEUE: a persistent launch over a work queue -- a grid of resident CTAs,
-// each taking CTA-sized items (A consecutive atoms) from a device counter
-// (flags[6], zeroed with the flags by every evaluation) until they run out;
-// an item's arithmetic is that of the CTA it would have been.
-template <typename R, int J2, bool QUEUE>
-__global__ void __launch_bounds__(de_max_warps<R>() * 32, 1) de_rev_col_kernel(WorkArgs a, int A) {
-  using S_ = Shape<J2>;
-  constexpr int NC = S_::NC, P = S_::P;
-  const int NW = blockDim.x >> 5;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ long item_s;
-  const int H = a.H;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long nitems = (a.n + A - 1) / A;
-  for (long item = blockIdx.x;;) {
-  if (QUEUE) {
-    if (threadIdx.x == 0) item_s = atomicAdd(&a.flags[6], 1);
-    __syncthreads();
-    item = item_s;
-    if (item >= nitems) break;
-  }
-  const long i0 = item * A;  // the CTA's atoms i0 .. i0 + na - 1
-  const int na = (int)min((long)A, a.n - i0);
-  c2<R>* Ywa = reinterpret_cast<c2<R>*>(smem);                    // [A][H] weighted Y
-  c2<R>* ust = Ywa + (size_t)A * H;                              // [NW*P][H] forward columns
-  R* red = reinterpret_cast<R*>(ust + (size_t)NW * P * H);       // [NW][32][5]
-  int* coff = reinterpret_cast<int*>(red + (size_t)NW * 32 * 5);  // [A+1] first pair of each atom
-  const int g = lane / NC, mb = lane - g * NC;
-  const bool grp = g < P;
-  for (int al = warp; al < na; al += NW) {  // weighted Y of the CTA's atoms
-    const long i = i0 + al;
-    const c2<R>* Yg = reinterpret_cast<const c2<R>*>(a.Y);
-    const long blk = i >> 5;
-    const int li = (int)(i & 31);
-    c2<R>* Yw = Ywa + (size_t)al * H;
-    for (int e = lane; e < H; e += 32) {
-      const int p = a.half_tmm[e];
-      // the contraction weight times S of the scaled recursion (u = S v)
-      const R w = (R)hweight(tmm_t(p), tmm_ma(p), tmm_mb(p)) * reinterpret_cast<const R*>(a.hscale)[e];
-      const c2<R> y = Yg[(blk * H + e) * 32 + li];
-      Yw[e] = mk<R>(w * y.re, w * y.im);
-    }
-  }
-  if (warp == 0) {  // exclusive offsets of the atoms' pairs (inclusive scan, 32 at a time)
-    int carry = 0;
-    if (lane == 0) coff[0] = 0;
-    for (int b = 0; b < na; b += 32) {
-      int c = b + lane < na ? a.cnt[i0 + b + lane] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(kFull, c, o);
-        if (lane >= o) c += u;
-      }
-      if (b + lane < na) coff[b + lane + 1] = carry + c;
-      carry += __shfl_sync(kFull, c, 31);
-    }
-  }
-  __syncthreads();
-  const int total = coff[na];
-  c2<R>* my = ust + (warp * P + (grp ? g : 0)) * H;
-  R* myred = red + (warp * 32 + lane) * 5;
-  for (int s0 = warp * P; s0 < total; s0 += NW * P) {
-    const int f = s0 + g;
-    const bool ok = grp && f < total;
-    // the pair's atom: the last al with coff[al] <= f (empty atoms skipped)
-    const int fk = min(f, total - 1);
-    int lo = 0, hi = na - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (coff[mid] <= fk) lo = mid;
-      else hi = mid - 1;
-    }
-    const long i = i0 + lo;
-    const c2<R>* Yw = Ywa + (size_t)lo * H;
-    const long slot = i * a.K + (ok ? f - coff[lo] : 0);
-    const R* gm = reinterpret_cast<const R*>(a.geom) + slot * kGeomStride;
-    c2<R> ka = mk<R>(1, 0), kb = mk<R>(0, 0);  // a and b
-    if (ok) {
-      ka = mk<R>(gm[0], gm[1]);
-      kb = mk<R>(gm[2], gm[3]);
-    }
-    // ---- forward: the scaled columns v, stored per layer
-    c2<R> u[J2 + 1];
-#pragma unroll
-    for (int k = 0; k <= J2; ++k) u[k] = mk<R>(0, 0);
-    R Ssum = 0;
-    if (mb == 0) {
-      u[0] = mk<R>(1, 0);
-      Ssum = Yw[0].re;
-      if (grp) my[0] = u[0];  // lanes past the last pair group own no storage
-    }
-    // conj(a), conj(b)
-    const c2<R> ca = mk<R>(ka.re, -ka.im), cb = mk<R>(kb.re, -kb.im);
-    static_for<1, J2>([&](auto tc) {
-      constexpr int t = decltype(tc)::value;
-      if constexpr ((t & 1) == 0) v_seed<R, t>(u, mb == t / 2);
-      v_layer<R, t>(u, ca, cb);
-      if (grp && 2 * mb <= t) {
-        c2<R>* dst = my + half_base(t) + mb * (t + 1);
-        const c2<R>* yr = Yw + half_base(t) + mb * (t + 1);
-#pragma unroll
-        for (int ma = 0; ma <= t; ++ma) {
-          dst[ma] = u[ma];
-          Ssum = fm(yr[ma].im, u[ma].im, fm(yr[ma].re, u[ma].re, Ssum));
-        }
-      }
-    });
-    __syncwarp();
-    // ---- reverse: adjoint columns
-    c2<R> lam[J2 + 1];
-#pragma unroll
-    for (int k = 0; k <= J2; ++k) lam[k] = mk<R>(0, 0);
-    if (2 * mb <= J2) {
-      const c2<R>* yr = Yw + half_base(J2) + mb * (J2 + 1);
-#pragma unroll
-      for (int k = 0; k <= J2; ++k) lam[k] = yr[k];
-    }
-    c2<R> ga = mk<R>(0, 0), gb = mk<R>(0, 0);
-    static_for<1, J2>([&](auto tc) {
-      constexpr int t = J2 + 1 - decltype(tc)::value;  // J2 down to 1
-      constexpr int tp = t - 1;
-      constexpr int mc = t / 2;
-      constexpr bool even = (t & 1) == 0;
-      c2<R> recv[t + 1];
-      if constexpr (even) {
-#pragma unroll
-        for (int k = 0; k <= t; ++k) {
-          recv[k].re = shfl_down(lam[k].re);
-          recv[k].im = shfl_down(lam[k].im);
-        }
-      }
-      const bool act = grp && 2 * mb <= tp;
-      const bool mir = even && act && (mb == mc - 1);
-      const c2<R>* ucol = my + half_base(tp) + (act ? mb * (tp + 1) : 0);
-      const c2<R>* yr = Yw + half_base(tp) + (act ? mb * (tp + 1) : 0);
-      // the seed's factor 1 / sqrt(mc) (v_seed)
-      constexpr double qd = even ? 1.0 / c_sqrt(double(mc)) : 0.0;
-      const R qm = R(qd);
-#pragma unroll
-      for (int m = 0; m <= tp; ++m) {
-        const c2<R> uu = act ? ucol[m] : mk<R>(0, 0);
-        const c2<R> Av = lam[m];
-        const c2<R> Bv = lam[m + 1];
-        // g_a += conj(A) u ; g_b -= conj(B) u
-        ga.re = fm(Av.im, uu.im, fm(Av.re, uu.re, ga.re));
-        ga.im = fm(-Av.im, uu.re, fm(Av.re, uu.im, ga.im));
-        gb.re = fm(-Bv.im, uu.im, fm(-Bv.re, uu.re, gb.re));
-        gb.im = fm(Bv.im, uu.re, fm(-Bv.re, uu.im, gb.im));
-        // new adjoint: Yw + a A - b B
-        const c2<R> y = act ? yr[m] : mk<R>(0, 0);
-        c2<R> nl;
-        nl.re = fm(kb.im, Bv.im, fm(-kb.re, Bv.re, fm(-ka.im, Av.im, fm(ka.re, Av.re, y.re))));
-        nl.im = fm(-kb.im, Bv.re, fm(-kb.re, Bv.im, fm(ka.im, Av.re, fm(ka.re, Av.im, y.im))));
-        if constexpr (even) {
-          if (mir) {
-            const int mp = tp - m;
-            const R sg = ((m + mc - 1) & 1) ? -qm : qm;
-            const c2<R> v = mk<R>(sg * uu.re, -sg * uu.im);
-            const c2<R> A2 = recv[mp];
-            const c2<R> B2 = recv[mp + 1];
-            ga.re = fm(A2.im, v.im, fm(A2.re, v.re, ga.re));
-            ga.im = fm(-A2.im, v.re, fm(A2.re, v.im, ga.im));
-            gb.re = fm(-B2.im, v.im, fm(-B2.re, v.re, gb.re));
-            gb.im = fm(B2.im, v.re, fm(-B2.re, v.im, gb.im));
-            const R lr = fm(kb.im, B2.im, fm(-kb.re, B2.re, fm(-ka.im, A2.im, ka.re * A2.re)));
-            const R li = fm(-kb.im, B2.re, fm(-kb.re, B2.im, fm(ka.im, A2.re, ka.re * A2.im)));
-            nl.re = fm(sg, lr, nl.re);
-            nl.im = fm(-sg, li, nl.im);
-          }
-        }
-        lam[m] = nl;
-      }
-      lam[tp + 1] = mk<R>(0, 0);
-    });
-    myred[0] = Ssum;
-    myred[1] = ga.re;
-    myred[2] = ga.im;
-    myred[3] = gb.re;
-    myred[4] = gb.im;
-    __syncwarp();
-    if (ok && mb == 0) {
-      R q[5] = {0, 0, 0, 0, 0};
-      for (int c = 0; c < NC; ++c) {
-        const R* p = red + (warp * 32 + lane + c) * 5;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) q[k] += p[k];
-      }
-      const R fc = gm[4];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const R ds = q[1] * gm[8 + 2 * d] + q[2] * gm[9 + 2 * d] + q[3] * gm[14 + 2 * d] +
-                     q[4] * gm[15 + 2 * d];
-        a.dedr[slot * 3 + d] = (double)(gm[5 + d] * q[0] + fc * ds);
-      }
-    }
-    __syncwarp();
-  }
-  if (!QUEUE) break;
-  __syncthreads();  // the item's shared memory is reused by the next item
-  }
-}
-
 template <typename K>
 inline cudaError_t col_allow_smem(K kernel, size_t bytes) {
   // the default 48 KB limit covers static and dynamic shared memory together
@@ -810,13 +546,6 @@ inline cudaError_t col_allow_smem(K kernel, size_t bytes) {
   if (e != cudaSuccess) return e;
   if (bytes + fa.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-// Warps (= atoms) per CTA: the tunable, halved until the CTA's shared memory
-// (proportional to its warps) fits the 227 KB limit.
-inline int col_fit_warps(int nw, size_t per_warp) {
-  while (nw > 1 && per_warp * nw > (size_t)227 * 1024) nw >>= 1;
-  return nw;
 }
 
 template <typename R, int J2>
@@ -861,158 +590,6 @@ cudaError_t launch_tan_col_t(const WorkArgs& a, const double* g, void* dU, cudaS
   if (e != cudaSuccess) return e;
   return launch_k(tan_col_kernel<R, J2>, dim3((unsigned)((a.n + UP::A - 1) / UP::A)), dim3(UP::A * UP::Q * 32),
                   smem, s, a, g, dU);
-}
-
-// Launch plan of the fused dE kernel: warps per CTA (NW) and atoms per CTA
-// (A) for atoms of `maxcnt` pairs, from the kernel's registers, the shared
-// memory of a plan and the SM count.
-//  * A plan's cost is (waves of CTAs) x (passes of its longest warp); the
-//    search minimises it, ties going to fewer warps in all.
-//  * The reference shape is a warp per atom in CTAs of `nw0` warps.  In one or
-//    two waves its cost is counted the same way; over more waves its small
-//    CTAs even out and it costs about (all passes) / (resident warps).
-//  * The searched plan is taken when it costs 3% less than the reference
-//    (measured at 2J8 and 2J14 on 2000 atoms, a 64-configuration batch, and
-//    16000 atoms at 2J14, where the reference stays ahead).
-//  * pipe_bound (FP64, whose pipe runs at 1/64 of the FP32 rate and is busy
-//    all the time): the CTAs an SM holds share its pipe, so A is chosen first
-//    by ceil(ctas / SMs) x ceil(A x maxcnt / P), the most CTAs an SM takes
-//    times a CTA's passes, among the A whose best warp count (the search
-//    above) keeps at least 8 warps an SM resident; then the warp count for
-//    that A as above.  Measured at 2J8, 2000 atoms: A = 2 1.067 ms, 3 1.138,
-//    16 1.151, 8 1.166, 4 1.182, 1 1.194, 6 1.365, 12 1.704 (the model: 63,
-//    65, 70, 70, 72, 70, 78, 104).
-struct DePlan {
-  int nw, A;
-  size_t smem;
-};
-// force_A > 0 (the SNAP_KNOB_DE_ATOMS tunable) restricts the search to CTAs
-// of force_A atoms (the best warp count for it) and skips the reference.
-inline DePlan de_plan(int n, int maxcnt, int P, size_t per_warp, size_t per_atom, int regs, int nsm,
-                      int max_warps, int nw0, int force_A = 0, bool pipe_bound = false);
-
-// The pipe-bound choice of A (see de_plan), then the plan for it.
-inline DePlan de_plan_pipe(int n, int maxcnt, int P, size_t per_warp, size_t per_atom, int regs, int nsm,
-                           int max_warps, int nw0) {
-  const int ralloc = (regs + 7) / 8 * 8;
-  DePlan best{0, 0, 0};
-  long best_cost = -1;
-  for (int A = 1; A <= 64; ++A) {
-    const DePlan p = de_plan(n, maxcnt, P, per_warp, per_atom, regs, nsm, max_warps, nw0, A);
-    if (p.smem == 0) break;
-    const long ctas = (n + A - 1) / A;
-    const int cps = std::min({65536 / (ralloc * p.nw * 32), (int)((228 * 1024) / (p.smem + 1024)), 64 / p.nw, 32});
-    const long per_sm = (ctas + nsm - 1) / nsm;
-    if (std::min<long>(per_sm, cps) * p.nw < 8) continue;  // too few warps to keep the pipe busy
-    const long cost = per_sm * (((long)A * maxcnt + P - 1) / P);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = p;
-    }
-  }
-  if (best_cost < 0) return de_plan(n, maxcnt, P, per_warp, per_atom, regs, nsm, max_warps, nw0);
-  return best;
-}
-
-inline DePlan de_plan(int n, int maxcnt, int P, size_t per_warp, size_t per_atom, int regs, int nsm,
-                      int max_warps, int nw0, int force_A, bool pipe_bound) {
-  if (pipe_bound && force_A <= 0) return de_plan_pipe(n, maxcnt, P, per_warp, per_atom, regs, nsm, max_warps, nw0);
-  const int ralloc = (regs + 7) / 8 * 8;
-  auto shape = [&](int nw, int A, size_t* smem, long* waves, long* ppw) -> bool {
-    *smem = (size_t)A * per_atom + (size_t)nw * per_warp + sizeof(int) * (A + 1);
-    if (*smem > (size_t)227 * 1024) return false;
-    const int cps = std::min({65536 / (ralloc * nw * 32), (int)((228 * 1024) / (*smem + 1024)), 64 / nw, 32});
-    if (cps < 1) return false;
-    const long ctas = (n + A - 1) / A;
-    *waves = (ctas + (long)nsm * cps - 1) / ((long)nsm * cps);
-    *ppw = ((((long)A * maxcnt + P - 1) / P) + nw - 1) / nw;
-    return true;
-  };
-  DePlan ref{nw0, nw0, 0};
-  double ref_cost = 1e300;
-  {
-    long waves, ppw;
-    size_t smem;
-    if (shape(nw0, nw0, &smem, &waves, &ppw)) {
-      ref.smem = smem;
-      const long slots = (long)nsm * std::max(1, (int)std::min<long>(
-                                                  {65536L / (ralloc * nw0 * 32), (long)((228 * 1024) / (smem + 1024)),
-                                                   64L / nw0, 32L})) * nw0;
-      const long per_atom_passes = (maxcnt + P - 1) / P;
-      ref_cost = waves <= 2 ? (double)(waves * per_atom_passes)
-                            : (double)n * per_atom_passes / (double)slots;
-    }
-  }
-  DePlan best{0, 0, 0};
-  long best_cost = -1, best_warps = 0;
-  for (int nw = 2; nw <= max_warps; nw *= 2) {
-    for (int A = force_A > 0 ? force_A : 1; A <= (force_A > 0 ? force_A : 256); ++A) {
-      long waves, ppw;
-      size_t smem;
-      if (!shape(nw, A, &smem, &waves, &ppw)) break;
-      const long cost = waves * ppw;
-      const long warps = (long)((n + A - 1) / A) * nw;
-      if (best_cost < 0 || cost < best_cost || (cost == best_cost && warps < best_warps)) {
-        best_cost = cost;
-        best_warps = warps;
-        best = DePlan{nw, A, smem};
-      }
-    }
-  }
-  if (force_A > 0 && best_cost >= 0) return best;
-  if (best_cost < 0 || (ref.smem != 0 && (double)best_cost > 0.97 * ref_cost)) return ref;
-  return best;
-}
-
-template <typename R, int J2>
-cudaError_t launch_de_rev_col_t(const WorkArgs& a, cudaStream_t s) {
-  if (a.n <= 0) return cudaSuccess;
-  // per warp: forward columns [P][H], lane partials [32][5]; per atom: Yw [H] and its offset
-  const size_t per_warp = sizeof(c2<R>) * (size_t)Shape<J2>::P * a.H + sizeof(R) * 32 * 5;
-  const size_t per_atom = sizeof(c2<R>) * (size_t)a.H;
-  // the kernel's registers and the last plan, per instantiation (the plan
-  // search is a few hundred candidate shapes; repeated calls reuse it)
-  static std::mutex mu;
-  static int regs = 0;
-  static long long last_key[4] = {-1, -1, -1, -1};
-  static DePlan last_plan{0, 0, 0};
-  const int nw0 = std::min(col_fit_warps(a.col_warps, per_warp + per_atom), de_max_warps<R>());
-  const int maxcnt = std::max(1, a.de_maxcnt), nsm = std::max(1, a.nsm);
-  DePlan p;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (regs == 0) {
-      cudaFuncAttributes fa;
-      cudaError_t e = cudaFuncGetAttributes(&fa, de_rev_col_kernel<R, J2, false>);
-      if (e != cudaSuccess) return e;
-      regs = fa.numRegs;
-    }
-    const long long key[4] = {a.n, ((long long)a.de_atoms << 32) | maxcnt, ((long long)nsm << 32) | nw0, a.H};
-    if (std::equal(key, key + 4, last_key)) {
-      p = last_plan;
-    } else {
-      p = de_plan(a.n, maxcnt, Shape<J2>::P, per_warp, per_atom, regs, nsm, de_max_warps<R>(), nw0, a.de_atoms,
-                  sizeof(R) == 8);
-      std::copy(key, key + 4, last_key);
-      last_plan = p;
-    }
-  }
-  if (p.smem == 0) return cudaErrorInvalidConfiguration;  // no plan fits (not reached for 2J <= 14)
-  const long nitems = (a.n + p.A - 1) / p.A;
-  if (a.persist & 2) {
-    // persistent: as many CTAs as stay resident, items from the queue
-    auto kq = de_rev_col_kernel<R, J2, true>;
-    cudaError_t e = col_allow_smem(kq, p.smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kq, p.nw * 32, p.smem);
-    if (e != cudaSuccess) return e;
-    const long grid = std::min<long>(nitems, (long)nsm * std::max(1, occ));
-    return launch_k(kq, dim3((unsigned)grid), dim3(p.nw * 32), p.smem, s, a, p.A);
-  }
-  cudaError_t e = col_allow_smem(de_rev_col_kernel<R, J2, false>, p.smem);
-  if (e != cudaSuccess) return e;
-  return launch_k(de_rev_col_kernel<R, J2, false>, dim3((unsigned)nitems), dim3(p.nw * 32), p.smem, s, a, p.A);
 }
 
 }  // namespace col

@@ -176,7 +176,7 @@ struct WorkArgs {
   const int* ysched;      // [32][ysched_m] outputs of each lane (warp-per-atom layout)
   int ysched_m;
   int nsm;
-  int col_warps;  // warps per CTA of the column-chain kernels (tunable)
+  int col_warps;  // fused dE: an SM with fewer than 2 col_warps batches shares them (tunable)
   int de_maxcnt;  // neighbour count the fused dE launch is planned for (last seen maximum, else K)
   int yi_waves;   // compute_Y waves per SM (tunable)
   int persist;    // tunable: bit 0 persistent compute_Y, bit 1 persistent fused dE (work queues)
@@ -196,6 +196,10 @@ struct WorkArgs {
   double* B;              // [N][ncoeff]
   const void* rootpq;
   const void* hscale;  // R [H]: S_t(ma, mb) of the scaled recursion (u = S v)
+  // closed-form u of a pair (snap_pairs.cuh, HostTables::pair_*), per step
+  const unsigned* pair_idx;
+  const void* pair_scale;  // R
+  const void* pair_ab;     // R x 2
 };
 
 // Launchers (snap_neigh.cu)
@@ -245,7 +249,6 @@ cudaError_t launch_flags_out(int* flags, int* hflags, cudaStream_t s);
 // Per-configuration virial: sum of vatom over each configuration's atoms.
 cudaError_t launch_virial_conf(const double* vatom, const NeighConf* confs, int nconf, double* virial,
                                cudaStream_t s);
-template <typename R> cudaError_t launch_de(const WorkArgs& a, cudaStream_t s);
 template <typename R> cudaError_t launch_force(const WorkArgs& a, cudaStream_t s);
 template <typename R> cudaError_t launch_bi(const WorkArgs& a, cudaStream_t s);
 
@@ -271,7 +274,6 @@ bool bi_plane_fits(int rsize, int H);
 // Register column-chain kernels (snap_col_*.cu), for 1 <= twojmax <= 14;
 // cudaErrorInvalidValue when no instance exists for the precision/2J.
 template <typename R> cudaError_t launch_ui_col(const WorkArgs& a, cudaStream_t s);
-template <typename R> cudaError_t launch_de_col(const WorkArgs& a, cudaStream_t s);
 // Neighbour build fused with compute_U (FP32: 1 <= twojmax <= 14; FP64: up
 // to 8): one configuration (ncta = 0) or a batch of ncta CTAs (na.confs).
 template <typename R>
@@ -279,6 +281,9 @@ cudaError_t launch_neigh_u(const NeighArgs& na, const WorkArgs& a, int ncta, cud
 // Tangent of Ulisttot along the displacement field g ([N][3], device); 0..14.
 template <typename R>
 cudaError_t launch_tan_col(const WorkArgs& a, const double* g, void* dU, cudaStream_t s);
+
+// Fused dU + dE/dr in closed form (snap_pairs.cuh), 0 <= twojmax <= 14.
+template <typename R> cudaError_t launch_de(const WorkArgs& a, cudaStream_t s);
 
 // d B_l along the tangent dU (snap_kernels.cu) and the weighted force gather.
 template <typename R> cudaError_t launch_dbi(const WorkArgs& a, const void* dU, double* dB, cudaStream_t s);

@@ -942,151 +942,6 @@ __global__ void __launch_bounds__(256) force_weighted_kernel(WorkArgs a, const d
     for (int c = 0; c < 3; ++c) grad[3 * k + c] = -f[c];
 }
 
-// ------------------------------------------------------ fused dU + dE/dr
-// One CTA per atom i with Y_i (weighted by half_weight and by S of the
-// scaled recursion u = S v) staged in shared memory; one warp per pair.  For
-// a pair, S(a, b) = sum_t Re Y_t : conj(u_t) = sum_t Re (S Y_t) : conj(v_t)
-// is a real function of the Cayley-Klein parameters.  Its gradient follows
-// from one forward pass of the scaled layer recursion (all layers of v kept
-// in shared memory) and one reverse (adjoint) pass through the same
-// recursion, so neither dU nor its three Cartesian components is ever
-// formed, and neither pass applies a root factor.  Then
-//   dE_i/dr_ik = S df_c/dr + f_c (<g_a, da/dr> + <g_b, db/dr>),
-// <x, y> = Re(conj(x) y), which is Eq. (snapforce2) for this pair.
-template <typename R, int NW>
-__global__ void __launch_bounds__(NW * 32) de_kernel(WorkArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int H = a.H, L = a.lmax, J2 = a.twojmax;
-  R* root = reinterpret_cast<R*>(smem);
-  cx<R>* Yw = reinterpret_cast<cx<R>*>(root + kRootDim * kRootDim);
-  cx<R>* ubase = Yw + H;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x;
-  const R* rootg = reinterpret_cast<const R*>(a.rootpq);
-  for (int e = threadIdx.x; e < kRootDim * kRootDim; e += blockDim.x) root[e] = rootg[e];
-  {
-    const cx<R>* Yg = reinterpret_cast<const cx<R>*>(a.Y);
-    const long blk = i >> 5;
-    const int li = i & 31;
-    for (int e = threadIdx.x; e < H; e += blockDim.x) {
-      const int p = a.half_tmm[e];
-      const R w = (R)half_weight(tmm_t(p), tmm_ma(p), tmm_mb(p));
-      // the contraction weight times S of the scaled recursion (u = S v)
-      const R ws = w * reinterpret_cast<const R*>(a.hscale)[e];
-      const cx<R> y = Yg[(blk * H + e) * 32 + li];
-      Yw[e] = mk<R>(ws * y.re, ws * y.im);
-    }
-  }
-  __syncthreads();
-  cx<R>* ust = ubase + warp * (H + 2 * L);
-  cx<R>* lam0 = ust + H;
-  cx<R>* lam1 = lam0 + L;
-  const int cnt = a.cnt[i];
-  for (int s = warp; s < cnt; s += NW) {
-    const long slot = (long)i * a.K + s;
-    const R* g = reinterpret_cast<const R*>(a.geom) + slot * kGeomStride;
-    const cx<R> ca = mk<R>(g[0], g[1]);
-    const cx<R> cb = mk<R>(g[2], g[3]);
-    // forward: all layers of u (half layout) and S
-    R S = 0;
-    if (lane == 0) {
-      ust[0] = mk<R>(1, 0);
-      S = Yw[0].re;
-    }
-    __syncwarp();
-    for (int t = 1; t <= J2; ++t) {
-      const int size = half_layer_size(t), hb = half_base(t);
-      const cx<R>* pl = ust + half_base(t - 1);
-      const R qm = (t & 1) ? R(0) : root[kRootDim + t / 2];  // 1 / sqrt(t/2): the mirror's ratio
-      for (int e = lane; e < size; e += 32) {
-        const int mb = e / (t + 1), ma = e - mb * (t + 1);
-        cx<R> v = mk<R>(0, 0);
-        if (ma < t) {  // + conj(a) v_{t-1}[ma]
-          const cx<R> p = prev_elem_v(pl, t - 1, ma, mb, qm);
-          v.re = fmr(ca.im, p.im, ca.re * p.re);
-          v.im = fmr(-ca.im, p.re, ca.re * p.im);
-        }
-        if (ma > 0) {  // - conj(b) v_{t-1}[ma-1]
-          const cx<R> p = prev_elem_v(pl, t - 1, ma - 1, mb, qm);
-          v.re = fmr(-cb.im, p.im, fmr(-cb.re, p.re, v.re));
-          v.im = fmr(cb.im, p.re, fmr(-cb.re, p.im, v.im));
-        }
-        ust[hb + e] = v;
-        const cx<R> yw = Yw[hb + e];
-        S = fmr(yw.im, v.im, fmr(yw.re, v.re, S));
-      }
-      __syncwarp();
-    }
-    // reverse: lambda_t = adjoint of layer t, gathered from layer t+1
-    {
-      const int hb = half_base(J2);
-      for (int e = lane; e < half_layer_size(J2); e += 32) lam0[e] = Yw[hb + e];
-    }
-    __syncwarp();
-    cx<R> ga = mk<R>(0, 0), gb = mk<R>(0, 0);
-    cx<R>* lt = lam0;
-    cx<R>* ln = lam1;
-    for (int t = J2; t >= 1; --t) {
-      const int tp = t - 1;
-      const int sizep = half_layer_size(tp), hbp = half_base(tp);
-      const bool mirror = ((t & 1) == 0);
-      const int mc = t >> 1;  // the column of layer t that reads a mirrored column
-      const R qmc = mirror ? root[kRootDim + mc] : R(0);  // 1 / sqrt(mc)
-      for (int e = lane; e < sizep; e += 32) {
-        const int mb = e / (tp + 1), m = e - mb * (tp + 1);
-        const cx<R> u = ust[hbp + e];
-        // v_{t-1}[m][mb] feeds v_t[m][mb] (a-term) and v_t[m+1][mb] (b-term)
-        const cx<R> A = lt[mb * (t + 1) + m];
-        const cx<R> B = lt[mb * (t + 1) + m + 1];
-        // g_a += conj(A) u ; g_b -= conj(B) u ; new adjoint Yw + a A - b B
-        ga.re = fmr(A.im, u.im, fmr(A.re, u.re, ga.re));
-        ga.im = fmr(-A.im, u.re, fmr(A.re, u.im, ga.im));
-        gb.re = fmr(-B.im, u.im, fmr(-B.re, u.re, gb.re));
-        gb.im = fmr(B.im, u.re, fmr(-B.re, u.im, gb.im));
-        const cx<R> yw = Yw[hbp + e];
-        cx<R> nl;
-        nl.re = fmr(cb.im, B.im, fmr(-cb.re, B.re, fmr(-ca.im, A.im, fmr(ca.re, A.re, yw.re))));
-        nl.im = fmr(-cb.im, B.re, fmr(-cb.re, B.im, fmr(ca.im, A.re, fmr(ca.re, A.im, yw.im))));
-        if (mirror && mb == mc - 1) {
-          // v_t column mc reads sig qm conj(v_{t-1}[m][mc-1]) at row mp = tp - m
-          const int mp = tp - m;
-          const R sig = ((m + mc - 1) & 1) ? -qmc : qmc;
-          const cx<R> v = mk<R>(sig * u.re, -sig * u.im);
-          const cx<R> A2 = lt[mc * (t + 1) + mp];
-          const cx<R> B2 = lt[mc * (t + 1) + mp + 1];
-          ga.re = fmr(A2.im, v.im, fmr(A2.re, v.re, ga.re));
-          ga.im = fmr(-A2.im, v.re, fmr(A2.re, v.im, ga.im));
-          gb.re = fmr(-B2.im, v.im, fmr(-B2.re, v.re, gb.re));
-          gb.im = fmr(B2.im, v.re, fmr(-B2.re, v.im, gb.im));
-          const R lr = fmr(cb.im, B2.im, fmr(-cb.re, B2.re, fmr(-ca.im, A2.im, ca.re * A2.re)));
-          const R li = fmr(-cb.im, B2.re, fmr(-cb.re, B2.im, fmr(ca.im, A2.re, ca.re * A2.im)));
-          nl.re = fmr(sig, lr, nl.re);
-          nl.im = fmr(-sig, li, nl.im);
-        }
-        ln[e] = nl;
-      }
-      __syncwarp();
-      cx<R>* tmp = lt;
-      lt = ln;
-      ln = tmp;
-    }
-    S = warp_sum(S);
-    ga.re = warp_sum(ga.re);
-    ga.im = warp_sum(ga.im);
-    gb.re = warp_sum(gb.re);
-    gb.im = warp_sum(gb.im);
-    // lanes 0..2: component d of dE_i/dr_ik in the working precision; the
-    // per-atom force and virial sums over pairs are FP64 (force_kernel)
-    if (lane < 3) {
-      const int d = lane;
-      const R ds = ga.re * g[8 + 2 * d] + ga.im * g[9 + 2 * d] + gb.re * g[14 + 2 * d] +
-                   gb.im * g[15 + 2 * d];
-      a.dedr[slot * 3 + d] = (double)(g[5 + d] * S + g[4] * ds);
-    }
-    __syncwarp();
-  }
-}
-
 // --------------------------------------------- energy, forces and virial
 // CTA = kFAtoms consecutive atoms, kFThreads threads (a warp per two atoms).
 // FP64 runs at 1/64 of the FP32 rate on this part and a warp FP64
@@ -1311,15 +1166,10 @@ __global__ void __launch_bounds__(kFThreads) force_kernel(WorkArgs a) {
 }
 
 constexpr int kUiWarps = 4;
-constexpr int kDeWarps = 4;
 
 template <typename R>
 size_t ui_smem(int H, int L) {
   return sizeof(R) * kRootDim * kRootDim + sizeof(cx<R>) * (size_t)kUiWarps * (H + 2 * L);
-}
-template <typename R>
-size_t de_smem(int H, int L) {
-  return sizeof(R) * kRootDim * kRootDim + sizeof(cx<R>) * (H + (size_t)kDeWarps * (H + 2 * L));
 }
 
 template <typename K>
@@ -1460,15 +1310,6 @@ cudaError_t launch_yi(const WorkArgs& a, cudaStream_t s) {
 }
 
 template <typename R>
-cudaError_t launch_de(const WorkArgs& a, cudaStream_t s) {
-  if (a.n <= 0) return cudaSuccess;
-  const size_t sm = de_smem<R>(a.H, a.lmax);
-  cudaError_t e = allow_smem(de_kernel<R, kDeWarps>, sm);
-  if (e != cudaSuccess) return e;
-  return launch_k(de_kernel<R, kDeWarps>, dim3(a.n), dim3(kDeWarps * 32), sm, s, a);
-}
-
-template <typename R>
 cudaError_t launch_force(const WorkArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
   const size_t sm = force_smem(a.K, a.vatom != nullptr);
@@ -1593,8 +1434,6 @@ template cudaError_t launch_ui<float>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_ui<double>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_yi<float>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_yi<double>(const WorkArgs&, cudaStream_t);
-template cudaError_t launch_de<float>(const WorkArgs&, cudaStream_t);
-template cudaError_t launch_de<double>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_force<float>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_force<double>(const WorkArgs&, cudaStream_t);
 

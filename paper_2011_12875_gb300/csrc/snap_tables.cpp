@@ -466,6 +466,48 @@ void HostTables::build(int J2, bool size_runs) {
     for (int k = 2; k <= t - mb; ++k) f /= k;
     half_scale[e] = (double)std::sqrt(f);
   }
+  // closed form of u: see snap_pairs.cuh.  P_k^(q,p) monic has the recursion
+  // pi_{k+1} = (x - b_k) pi_k - g_k pi_{k-1} (Jacobi polynomials, alpha = q,
+  // beta = p); with pi_k = s_k P_k, s_{k+1} = g_k s_{k-1}, the last factor is 1.
+  pair_idx.clear();
+  pair_norm.clear();
+  pair_weight.clear();
+  pair_ab.clear();
+  std::array<long double, kMaxTwoJ + 2> fact;
+  for (int k = 0; k < (int)fact.size(); ++k) fact[k] = lfact(k);
+  for (int p = 0; p <= J2; ++p)
+    for (int q = J2 - p; q >= 0; --q) {
+      long double s0 = 1.0L, s1 = 1.0L, al = 0.0L, be = 0.0L;  // s_{k-1}, s_k and the coefficients to P_k
+      for (int k = 0; p + q + 2 * k <= J2; ++k) {
+        const int t = p + q + 2 * k, c = 2 * k + p + q;
+        if (k > 0) {  // s0 = s_{k-1}, s1 = s_k
+          const long double b = k == 1 ? (long double)(p - q) / (p + q + 2)
+                                       : (long double)(p * p - q * q) / ((long double)(c - 2) * c);
+          al = s0 / s1;
+          be = -al * b;
+        }
+        unsigned w;
+        if (2 * (k + q) <= t) w = (unsigned)(half_base(t) + (k + q) * (t + 1) + k);
+        else w = (unsigned)(half_base(t) + (t - k - q) * (t + 1) + (t - k)) | (1u << 10) | ((unsigned)(q & 1) << 11);
+        if (p > 0 && q > 0) w |= ((unsigned)(half_base(t) + k * (t + 1) + k + q) << 12) | (1u << 22);
+        pair_idx.push_back(w);
+        pair_norm.push_back((double)(fact[t] / std::pow(2.0L, k) /
+                                     std::sqrt(fact[t - k] * fact[k] * fact[t - k - q] * fact[k + q]) * s1));
+        pair_weight.push_back(p == 0 && q == 0 ? 1.0 : 2.0);
+        pair_ab.push_back((double)al);
+        pair_ab.push_back((double)be);
+        // s_{k+1}: s_1 = sqrt(g_1), s_{k+1} = g_k s_{k-1}
+        const auto g = [&](int m) -> long double {
+          const long double d = 2.0L * m + p + q;
+          if (m == 1) return 4.0L * (1 + p) * (1 + q) / (d * d * (d + 1));
+          return 4.0L * m * (m + p) * (m + q) * (m + p + q) / (d * d * (d + 1) * (d - 1));
+        };
+        const long double s2 = k == 0 ? std::sqrt(g(1)) : g(k) * s0;
+        s0 = s1;
+        s1 = s2;
+      }
+    }
+
   rootpq.assign(kRootDim * kRootDim, 0.0);
   for (int p = 0; p < kRootDim; ++p)
     for (int q = 1; q < kRootDim; ++q) rootpq[p * kRootDim + q] = std::sqrt((double)p / (double)q);

@@ -54,6 +54,19 @@ struct HostTables {
   // element, the factor between the scaled recursion's v and u
   std::vector<double> half_scale;
 
+  // The closed form of u (snap_pairs.cuh): the steps (p, q, k) of the classes
+  // (p, q), p + q <= 2J, in the order p rising, q falling, k rising.
+  // pair_idx: the half-layout elements of the step, bits 0-9 (ma, mb) = (k,
+  //   k + q), bit 10 conjugated and bit 11 negated when it is read through its
+  //   mirror, bits 12-21 (k + q, k) with bit 22 set when it is another element
+  //   (p, q > 0);
+  // pair_norm: n s_k, u = n s_k monomial P_k(x);
+  // pair_weight: the step's weight in a full-matrix contraction (2; 1 for p =
+  //   q = 0);
+  // pair_ab: alpha_{k-1}, beta_{k-1} of the recursion to P_k (0, 0 at k = 0).
+  std::vector<unsigned> pair_idx;
+  std::vector<double> pair_norm, pair_weight, pair_ab;
+
   // size_runs: order each output's term groups by length (the run layout of
   // the FP32 compute_Y); otherwise by first factor
   void build(int twojmax, bool size_runs = true);

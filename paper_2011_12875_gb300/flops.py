@@ -41,8 +41,10 @@ def ui_pair(twojmax: int) -> int:
 
 @lru_cache(maxsize=None)
 def de_pair(twojmax: int) -> int:
-    """Fused dU + dE, one pair, in the scaled form (S folded into the
-    weighted Y, so neither pass scales by roots).  Forward: the recursion and
+    """Fused dU + dE, one pair, as the scaled layer recursion and its adjoint
+    pass (S folded into the weighted Y, so neither pass scales by roots).  The
+    library evaluates u in closed form (csrc/snap_pairs.cuh), with fewer
+    operations; this count stays the unit of the roofline.  Forward: the recursion and
     the seeds as in compute_U (layer 0 is v = 1, S = Re Yw_0: no arithmetic)
     and the Re(Yw conj v) accumulation (4) per element.
     Reverse, per element of layer t-1: conj(A) v and conj(B) v accumulated

@@ -495,3 +495,22 @@ def test_bispectrum_partials_in_global_scratch(snapmod):
     err = rel_err(B[atoms], ref.B[atoms])
     print(f"ERRS-B-SCRATCH {err:.3e}")
     assert err <= MIXED_B_TOL
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("twojmax", list(range(0, 15)))
+def test_fused_de_batch_sharing_changes_no_bit(snapmod, twojmax, prec):
+    """The fused dE kernel's launch forms: few pairs (each 32-pair batch shared
+    by four warps, a part of the p range each), many pairs a CTA (a warp takes
+    all parts; 16 and 5 atoms a CTA, last batches partly empty) and a forced
+    CTA size that does not fit, at every 2J: the same bits."""
+    cfg = inputs.bcc(3, disp=0.2, seed=81)
+    s = snapmod.Snap(twojmax, inputs.beta(twojmax), precision=prec)
+    pos = torch.tensor(cfg.pos, device="cuda:0")
+    ref = [x.cpu().numpy().copy() for x in s.compute(pos, cfg.box)]
+    for cw, atoms in ((2, 16), (2, 5), (8, 16), (4, 256)):
+        s.set_knob(snapmod.KNOB_COL_WARPS, cw)
+        s.set_knob(snapmod.KNOB_DE_ATOMS, atoms)
+        for x, y in zip(s.compute(pos, cfg.box), ref):
+            assert np.array_equal(x.cpu().numpy(), y), (cw, atoms)
+    s.close()
