@@ -58,7 +58,9 @@ struct snap_ctx {
   int* d_half_tmm = nullptr;
   void* d_yrec = nullptr;
   int* d_yfirst = nullptr;
-  unsigned short* d_yruns = nullptr;
+  int* d_yc_slot = nullptr;  // compute_Y (HostTables::yc_*)
+  int* d_yc_task = nullptr;
+  unsigned* d_yc_stream = nullptr;
   void* d_brec = nullptr;
   void* d_brec_cp = nullptr;
   void* d_bscratch = nullptr;  // chunk partials of the bispectrum kernels (when shared memory is short)
@@ -80,11 +82,11 @@ struct snap_ctx {
   unsigned* d_pair_idx = nullptr;  // closed form of u (HostTables::pair_*)
   void* d_pair_scale = nullptr;
   void* d_pair_ab = nullptr;
-  int* d_yslice = nullptr;
+  int* d_yc_bins = nullptr;
   int* d_ysched = nullptr;  // lane schedule of the warp-per-atom compute_Y
   int ysched_m = 0;
-  int nslices = -1;
-  std::map<int, int*> yslice_cache;  // compute_Y slice tables by slice count
+  int yc_split = -1;
+  std::map<int, int*> yc_bins_cache;  // compute_Y's tasks by CTAs a block
 
   // workspace
   long cap_nk = 0;
@@ -101,6 +103,7 @@ struct snap_ctx {
   double* d_dedr = nullptr;
   void* d_U = nullptr;  // complex AoSoA [ceil(N/32)][H][32]
   void* d_Y = nullptr;
+  void* d_Y2 = nullptr;
   void* d_dU = nullptr;  // tangent of U (bispectrum derivative)
   long long generation = 0;  // number of evaluations enqueued
   snap::WorkArgs last_args;   // arguments of the last evaluation (weighted gather)
@@ -210,38 +213,25 @@ int upload_inplace(snap_ctx* c, T** dst, const std::vector<T>& v) {
 int upload_yrec(snap_ctx* c) {
   const std::vector<double> coef = c->tab.term_coef(c->beta.data());
   const size_t n = c->tab.terms.size();
-  // Kernel word (the formats are described with yrec_plane_format): the
-  // element offsets in units of 256 B (one element's [32] lanes of complex
-  // float; the FP64 kernel doubles them), the group-end and output-end bits
-  // and, without a staged conjugate plane, the conjugation flags (the sign
-  // bit of the factor's imaginary part).  With the plane the elements run
-  // over 2H (element + H for a conjugated read).
-  const bool cp = snap::yi_conjplane((int)c->rsize(), c->tab.H);
-  const bool pf = snap::yrec_plane_format((int)c->rsize(), c->tab.H);
-  const unsigned H = (unsigned)c->tab.H;
-  if ((cp ? 2 * H : H) > 1024u) return fail(c, SNAP_ERR_ARG, "compute_Y element index exceeds 10 bits");
+  // the class stream
+  int rc = upload_inplace(c, &c->d_yc_stream, c->precision == SNAP_MIXED ? c->tab.yc_stream(c->beta.data())
+                                                                         : c->tab.yc_fixed(c->beta.data()));
+  if (rc) return rc;
+  // the records of the warp-per-atom layout
   auto word = [&](unsigned w) -> unsigned {
-    unsigned e1 = w & 1023u, e2 = (w >> 10) & 1023u;
-    unsigned c1 = (w >> 20) & 1u, c2 = (w >> 21) & 1u;
+    const unsigned e1 = w & 1023u, e2 = (w >> 10) & 1023u, c1 = (w >> 20) & 1u, c2 = (w >> 21) & 1u;
     const unsigned ge = (w >> 23) & 1u, oe = (w >> 22) & 1u;
-    if (cp) {
-      e1 += c1 * H;
-      e2 += c2 * H;
-      c1 = c2 = 0;
-    }
-    if (pf) return (e2 << 22) | e1 | (ge << 12) | (oe << 13);
     return (e2 << 8) | (e1 << 18) | (ge << 28) | (oe << 29) | (c1 << 30) | (c2 << 31);
   };
-  // kYRecPad zero records past the end: compute_Y reads up to that far ahead
   if (c->precision == SNAP_MIXED) {
-    std::vector<snap::YRec<float>> r(n + snap::kYRecPad);
+    std::vector<snap::YRec<float>> r(n);
     for (size_t k = 0; k < n; ++k) {
       r[k].w = word(c->tab.terms[k]);
       r[k].c = (float)coef[k];
     }
     return upload_inplace(c, reinterpret_cast<snap::YRec<float>**>(&c->d_yrec), r);
   }
-  std::vector<snap::YRec<double>> r(n + snap::kYRecPad);
+  std::vector<snap::YRec<double>> r(n);
   for (size_t k = 0; k < n; ++k) {
     r[k].w = word(c->tab.terms[k]);
     r[k].pad = 0;
@@ -292,6 +282,7 @@ void free_workspace(snap_ctx* c) {
   dfree(c->d_dedr);
   dfree(c->d_U);
   dfree(c->d_Y);
+  dfree(c->d_Y2);
   dfree(c->d_dU);
   dfree(c->d_vpart);
   c->cap_nk = 0;
@@ -319,6 +310,7 @@ int ensure_workspace(snap_ctx* c, int n, int K) {
   SNAP_CUDA(c, cudaMalloc(&c->d_dedr, sizeof(double) * 3 * nkcap));
   SNAP_CUDA(c, cudaMalloc(&c->d_U, uy));
   SNAP_CUDA(c, cudaMalloc(&c->d_Y, uy));
+  SNAP_CUDA(c, cudaMalloc(&c->d_Y2, uy));
   SNAP_CUDA(c, cudaMalloc(&c->d_dU, uy));
   // lanes past the last atom read zeros in compute_Y
   SNAP_CUDA(c, cudaMemset(c->d_U, 0, uy));
@@ -330,18 +322,20 @@ int ensure_workspace(snap_ctx* c, int n, int K) {
   return SNAP_OK;
 }
 
-int ensure_slices(snap_ctx* c, int n) {
-  const snap::YiGeometry g = snap::yi_geometry((int)c->rsize(), c->tab.H, n, c->nsm, c->yi_waves);
-  if (g.nslices == c->nslices) return SNAP_OK;
-  auto it = c->yslice_cache.find(g.nslices);
-  if (it == c->yslice_cache.end()) {
+// The tasks of compute_Y's CTAs for n atoms
+int ensure_bins(snap_ctx* c, int n) {
+  const snap::YiGeometry g =
+      snap::yi_geometry((int)c->rsize(), c->tab.H, n, c->nsm, c->yi_waves, (int)c->tab.yc_cost.size());
+  if (g.split == c->yc_split) return SNAP_OK;
+  auto it = c->yc_bins_cache.find(g.split);
+  if (it == c->yc_bins_cache.end()) {
     int* d = nullptr;
-    int rc = upload(c, &d, c->tab.slices(g.nslices));
+    int rc = upload(c, &d, c->tab.yc_bins(g.split));
     if (rc) return rc;
-    it = c->yslice_cache.emplace(g.nslices, d).first;
+    it = c->yc_bins_cache.emplace(g.split, d).first;
   }
-  c->d_yslice = it->second;
-  c->nslices = g.nslices;
+  c->d_yc_bins = it->second;
+  c->yc_split = g.split;
   c->ws_gen += 1;
   return SNAP_OK;
 }
@@ -485,18 +479,22 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
   a.geom = c->d_geom;
   a.U = c->d_U;
   a.Y = c->d_Y;
+  a.Y2 = c->d_Y2;
   a.dedr = c->d_dedr;
   a.vpart = c->d_vpart;
   a.flags = c->d_flags;
   a.half_tmm = c->d_half_tmm;
   a.yrec = c->d_yrec;
   a.yfirst = c->d_yfirst;
-  a.yruns = c->d_yruns;
-  a.yslice = c->d_yslice;
+  a.yc_slot = c->d_yc_slot;
+  a.yc_task = c->d_yc_task;
+  a.yc_stream = c->d_yc_stream;
+  a.yc_ntask = (int)c->tab.yc_cost.size();
+  a.yc_bins = c->d_yc_bins;
   a.yi_layout = c->yi_layout;
   a.ysched = c->d_ysched;
   a.ysched_m = c->ysched_m;
-  a.nslices = c->nslices;
+  a.yc_split = c->yc_split;
   a.nsm = c->nsm;
   a.col_warps = c->col_warps;
   a.de_maxcnt = de_maxcnt(c, K);
@@ -543,7 +541,7 @@ int enqueue(snap_ctx* c, int n, const double* pos, const double* box, const int*
   int rc = ensure_workspace(c, n, K);
   if (!rc) rc = ensure_flags(c);
   if (rc) return rc;
-  rc = ensure_slices(c, n);
+  rc = ensure_bins(c, n);
   if (!rc && mode != 0) rc = ensure_bparts(c, n, mode == 2);
   if (rc) return rc;
   SNAP_CUDA(c, open_flags(c, s));
@@ -698,10 +696,10 @@ int prepare_batch(snap_ctx* c, int nconf, const int* natoms, const double* boxes
   int rc = ensure_workspace(c, n, c->K);
   if (!rc) rc = ensure_flags(c);
   if (rc) return rc;
-  const int old_slices = c->nslices;
-  rc = ensure_slices(c, n);
+  const int old_slices = c->yc_split;
+  rc = ensure_bins(c, n);
   if (rc) return rc;
-  if (c->nslices != old_slices && c->gexec) {
+  if (c->yc_split != old_slices && c->gexec) {
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
   }
@@ -908,7 +906,7 @@ int compute_dev(snap_ctx* c, int n, const double* pos, const double* box, const 
   const int K = user ? ucap : c->K;
   int rc = ensure_workspace(c, n, K);
   if (!rc) rc = ensure_flags(c);
-  if (!rc) rc = ensure_slices(c, n);
+  if (!rc) rc = ensure_bins(c, n);
   if (rc) return rc;
   const std::vector<unsigned long long> key = {
       1, (unsigned long long)c->ws_gen, (unsigned long long)n, (unsigned long long)K,
@@ -944,25 +942,101 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
       !beta || !u || !y)
     return SNAP_ERR_ARG;
   snap::HostTables tab;
-  tab.build(twojmax, precision == SNAP_MIXED);
-  const std::vector<double> coef = tab.term_coef(beta);
-  auto fac = [&](unsigned idx, unsigned conj, double& re, double& im) {
-    re = u[2 * idx];
-    im = conj ? -u[2 * idx + 1] : u[2 * idx + 1];
+  tab.build(twojmax);
+  tab.build_classes(precision == SNAP_FP64);
+  std::vector<int> elem(tab.H);
+  for (int e = 0; e < tab.H; ++e) elem[tab.yc_slot[e]] = e;
+  const size_t nt = tab.yc_cost.size();
+  auto store = [&](size_t k, int o, double re, double im) {
+    const int* rec = &tab.yc_task[k * snap::kYcTask];
+    const int e = rec[4 + o], zero = rec[4 + snap::kYcOuts + o];
+    const bool second = (rec[3] & 1) != 0;  // half of a split sum
+    y[2 * e] = re + (second ? y[2 * e] : 0.0);
+    y[2 * e + 1] = im + (second ? y[2 * e + 1] : 0.0);
+    if (zero >= 0) y[2 * zero] = y[2 * zero + 1] = 0.0;
   };
-  for (int o = 0; o < tab.H; ++o) {
-    double yr = 0.0, yi = 0.0;
-    for (int k = tab.term_out_first[o]; k < tab.term_out_first[o + 1]; ++k) {
-      const unsigned w = tab.terms[k];
-      double ar, ai, br, bi;
-      fac(w & 1023u, (w >> 20) & 1u, ar, ai);
-      fac((w >> 10) & 1023u, (w >> 21) & 1u, br, bi);
-      yr += coef[k] * (ar * br - ai * bi);
-      yi += coef[k] * (ar * bi + ai * br);
-    }
-    y[2 * o] = yr;
-    y[2 * o + 1] = yi;
+  if (precision == SNAP_MIXED) {
+    // the class stream with FP64 arithmetic in place of FP32
+    const std::vector<double> bw = tab.beta_weights(beta);
+    std::vector<double> s(nt * snap::kYcOuts * 2, 0.0);
+    tab.yc_rows([&](int k, const unsigned* h, int r, size_t p, int o, int len) {
+      auto fac = [&](unsigned w, int j, double& re, double& im) {
+        const int e = elem[(w & 0x7FFFFFFFu) / 256 + j];
+        re = u[2 * e];
+        im = (w >> 31) ? -u[2 * e + 1] : u[2 * e + 1];
+      };
+      double ar = 0.0, ai = 0.0, xr, xi;
+      for (int c2 = 0; c2 < len; ++c2) {
+        const size_t w = p + 2 * c2;
+        if (tab.yc_trip[w] < 0) continue;
+        const double cf = tab.yc_cg[w] * bw[tab.yc_trip[w]];
+        fac(h[1], c2, xr, xi);
+        ar += cf * xr;
+        ai += cf * xi;
+      }
+      fac(h[0], r, xr, xi);
+      double* d = &s[((size_t)k * snap::kYcOuts + o) * 2];
+      d[0] += xr * ar - xi * ai;
+      d[1] += xr * ai + xi * ar;
+    });
+    for (size_t k = 0; k < nt; ++k)
+      for (int o = 0; o < tab.yc_task[k * snap::kYcTask + 2]; ++o)
+        store(k, o, s[(k * snap::kYcOuts + o) * 2], s[(k * snap::kYcOuts + o) * 2 + 1]);
+    return SNAP_OK;
   }
+  // the fixed-point form, as the kernel computes it (YcFixed)
+  typedef long long ll;
+  const std::vector<unsigned> words = tab.yc_fixed(beta);
+  double mx = 0.0;
+  for (int e = 0; e < 2 * tab.H; ++e) mx = std::max(mx, std::fabs(u[e]));
+  int ex = 0;
+  std::frexp(mx, &ex);
+  const ll half = 1LL << 29, one30 = 1LL << 30;
+  auto split = [&](ll v, ll& h, ll& l) {
+    h = (v + half) >> 30;
+    l = v - h * one30;
+  };
+  std::vector<ll> uh(2 * tab.H), ul(2 * tab.H);
+  for (int e = 0; e < 2 * tab.H; ++e) split(std::llround(std::ldexp(u[e], 59 - ex)), uh[e], ul[e]);
+  std::vector<__int128> s(nt * 4, 0);
+  ll acc[2][4];  // of each output's record: ph, pc, qh, qc
+  tab.yc_rows([&](int k, const unsigned* h, int r, size_t p, int o, int len) {
+    const int s1 = (h[0] >> 31) ? -1 : 1, s2 = (h[1] >> 31) ? -s1 : s1;
+    ll rh = 0, rc = half, ih = 0, ic = half;
+    for (int c2 = 0; c2 < len; ++c2) {
+      const ll wh = (int)words[p + 2 * c2], wl = (int)words[p + 2 * c2 + 1];
+      const int e = 2 * elem[(h[1] & 0x7FFFFFFFu) / 256 + c2];
+      rh += wh * uh[e];
+      rc += wh * ul[e] + wl * uh[e];
+      ih += s2 * wh * uh[e + 1];
+      ic += s2 * (wh * ul[e + 1] + wl * uh[e + 1]);
+    }
+    ll Ah, Al, Bh, Bl;
+    split(rh + (rc >> 30), Ah, Al);
+    split(ih + (ic >> 30), Bh, Bl);
+    const int e = 2 * elem[(h[0] & 0x7FFFFFFFu) / 256 + r];
+    const ll xh = uh[e], xl = ul[e], zh = uh[e + 1], zl = ul[e + 1];
+    ll* a = acc[o];
+    if (r == 0) {
+      a[0] = a[2] = 0;
+      a[1] = a[3] = half;
+    }
+    a[0] += xh * Ah - zh * Bh;
+    a[1] += xh * Al + xl * Ah - zh * Bl - zl * Bh;
+    a[2] += xh * Bh + zh * Ah;
+    a[3] += xh * Bl + xl * Bh + zh * Al + zl * Ah;
+    if (r + 1 == (int)(h[2] & 255u)) {
+      s[(size_t)k * 4 + 2 * o] += a[0] + (a[1] >> 30);
+      s[(size_t)k * 4 + 2 * o + 1] += s1 * (a[2] + (a[3] >> 30));
+    }
+  });
+  for (size_t k = 0; k < nt; ++k)
+    for (int o = 0; o < tab.yc_task[k * snap::kYcTask + 2]; ++o) {
+      const int e = (int)words[(size_t)tab.yc_task[k * snap::kYcTask] * snap::kYcChunk + 2 + o];
+      const __int128* d = &s[k * 4 + 2 * o];
+      if (e == snap::kYcNan || !std::isfinite(mx)) store(k, o, NAN, NAN);
+      else store(k, o, std::ldexp((double)d[0], 2 * ex + e - 58), std::ldexp((double)d[1], 2 * ex + e - 58));
+    }
   return SNAP_OK;
 }
 
@@ -1058,7 +1132,8 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
   c->rmin0 = rmin0;
   c->switchflag = switchflag;
   c->precision = precision;
-  c->tab.build(twojmax, precision == SNAP_MIXED);
+  c->tab.build(twojmax);
+  c->tab.build_classes(precision == SNAP_FP64);
   c->beta.assign(beta, beta + 1 + c->tab.ncoeff);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1070,7 +1145,8 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
   }
   int rc = upload(c, &c->d_half_tmm, c->tab.half_tmm);
   if (!rc) rc = upload(c, &c->d_yfirst, c->tab.term_out_first);
-  if (!rc) rc = upload(c, &c->d_yruns, c->tab.term_runs);
+  if (!rc) rc = upload(c, &c->d_yc_slot, c->tab.yc_slot);
+  if (!rc) rc = upload(c, &c->d_yc_task, c->tab.yc_task);
   if (!rc) rc = upload(c, &c->d_ysched, c->tab.lane_outputs(32, &c->ysched_m));
   if (!rc) rc = upload_r(c, &c->d_root, c->tab.rootpq);
   if (!rc) rc = upload_r(c, &c->d_hscale, c->tab.half_scale);
@@ -1560,7 +1636,7 @@ int snap_compute_host(snap_ctx* c, int natoms, const double* pos_host, const dou
     // every buffer exists before a capture (no allocation inside one)
     rc = ensure_workspace(c, natoms, c->K);
     if (!rc) rc = ensure_flags(c);
-    if (!rc) rc = ensure_slices(c, natoms);
+    if (!rc) rc = ensure_bins(c, natoms);
     if (rc) return rc;
     const std::vector<unsigned long long> key = {
         2, (unsigned long long)c->ws_gen, (unsigned long long)natoms, (unsigned long long)c->K,
@@ -1657,7 +1733,9 @@ int snap_destroy(snap_ctx* c) {
   dfree(c->d_half_tmm);
   dfree(c->d_yrec);
   dfree(c->d_yfirst);
-  dfree(c->d_yruns);
+  dfree(c->d_yc_slot);
+  dfree(c->d_yc_task);
+  dfree(c->d_yc_stream);
   dfree(c->d_ysched);
   dfree(c->d_brec);
   dfree(c->d_brec_cp);
@@ -1672,9 +1750,9 @@ int snap_destroy(snap_ctx* c) {
   dfree(c->d_pair_idx);
   dfree(c->d_pair_scale);
   dfree(c->d_pair_ab);
-  for (auto& kv : c->yslice_cache) cudaFree(kv.second);
-  c->yslice_cache.clear();
-  c->d_yslice = nullptr;
+  for (auto& kv : c->yc_bins_cache) cudaFree(kv.second);
+  c->yc_bins_cache.clear();
+  c->d_yc_bins = nullptr;
   dfree(c->d_flags);
   dfree(c->d_hpos);
   dfree(c->d_hE);

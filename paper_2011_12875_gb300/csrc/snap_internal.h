@@ -20,12 +20,14 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 #endif
 
 constexpr int kMaxTwoJ = 14;
-constexpr int kYGroupMax = 8;  // longest compute_Y term group (longer ones are cut)
+constexpr int kYcChunk = 256;  // words of a compute_Y stream chunk (snap_tables.h)
+constexpr int kYcOuts = 8;     // most outputs of a compute_Y task
+constexpr int kYcTask = 4 + 2 * kYcOuts;
+constexpr long kYcWhole = 1000;  // cost from which a task's sum is split in two
+constexpr int kYcNan = 0x7FFF;  // exponent of an output whose coefficients are not finite
 constexpr int kBChunk = 96;    // bispectrum terms a warp takes at a time (whole groups)
 constexpr int kBMaxChunks = 1024;  // chunks are lengthened past this count
 constexpr int kBGroupMax = 8;      // longest bispectrum term piece (longer groups are cut)
-constexpr int kYRecPad = 256;  // zero records after the compute_Y term list (read-ahead)
-constexpr int kYRecPrefetch = 64;  // compute_Y's L1 prefetch distance without the record ring
 constexpr int kMaxNeighCap = 64;
 constexpr int kRootDim = 16;     // rootpq table is kRootDim x kRootDim
 constexpr int kGeomStride = 20;  // doubles per neighbour slot, see PairGeom
@@ -156,6 +158,7 @@ struct WorkArgs {
   // Ulisttot and Y: complex (re, im interleaved), AoSoA [ceil(N/32)][H][32]
   void* U;
   void* Y;
+  void* Y2;  // compute_Y: the second halves of split sums (as Y)
   double* dedr;
   double* vatom;   // per-atom virial [N][6] (batch mode) or nullptr
   double* energy;
@@ -167,13 +170,19 @@ struct WorkArgs {
   // last CTA writes flags[0..3] to this host-mapped copy and zeroes the flags
   int* hflags;
   const int* half_tmm;
-  const void* yrec;       // compute_Y term records (see snap_tables.cpp)
-  const int* yfirst;      // [H+1] first term of each output element
-  const void* yruns;      // [H][kYGroupMax] u16: groups of 1..kYGroupMax terms per output
-  const int* yslice;
-  int nslices;
+  // compute_Y's tables (HostTables::yc_*); yc_bins for yc_split CTAs a block
+  const int* yc_bins;
+  int yc_split;
+  const int* yc_slot;
+  const int* yc_task;
+  const unsigned* yc_stream;
+  int yc_ntask;
   int yi_layout;          // 0: warp of 32 atoms (AoSoA), 1: warp per atom
-  const int* ysched;      // [32][ysched_m] outputs of each lane (warp-per-atom layout)
+  // warp-per-atom layout: term records (snap_tables.cpp), [H+1] first term of
+  // each output element, [32][ysched_m] outputs of each lane
+  const void* yrec;
+  const int* yfirst;
+  const int* ysched;
   int ysched_m;
   int nsm;
   int col_warps;  // fused dE: an SM with fewer than 2 col_warps batches shares them (tunable)
@@ -218,29 +227,16 @@ cudaError_t launch_neigh_ingest(int n, int K, const double* pos, double Lx, doub
 template <typename R> cudaError_t launch_ui(const WorkArgs& a, cudaStream_t s);
 template <typename R> cudaError_t launch_yi(const WorkArgs& a, cudaStream_t s);
 
-// Launch shape of compute_Y for N atoms: grid (nblk, ysplit), `threads` per
-// CTA, nslices = ysplit * warps per CTA work slices per 32-atom block; the
-// block's Ulisttot is staged in `smem` bytes of shared memory when it fits.
+// Launch shape of compute_Y for N atoms: nblk blocks of atoms x split CTAs of
+// `threads`, with `smem` bytes of shared memory.
 struct YiGeometry {
-  int nblk, ysplit, threads, nslices;
+  int nblk, split, threads;
   size_t smem;
-  bool staged;
-  bool conjplane;  // a conjugated copy of the block is staged too (records index it)
 };
-// Whether compute_Y stages U and its conjugate (records in the 2H-index format).
-__host__ __device__ inline bool yi_conjplane(int rsize, int H) {
-  return (size_t)4 * H * 32 * rsize + 16 <= 100 * 1024;
-}
-// compute_Y term record word.  FP32 with the conjugate plane: bits 14-31 the
-// byte offset of the second factor's [32] lanes (element times 256, the
-// element over the 2H plane), bits 0-9 the first factor's element, bit 12
-// ends a group, bit 13 an output.  Otherwise: bits 8-17 the second factor's
+// Term record word of the warp-per-atom layout: bits 8-17 the second factor's
 // element, 18-27 the first's, bit 28 ends a group, 29 an output, 30 / 31
-// conjugate the first / second factor (no conjugation bits with the plane).
-__host__ __device__ inline bool yrec_plane_format(int rsize, int H) {
-  return rsize == 4 && yi_conjplane(rsize, H);
-}
-YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves);
+// conjugate the first / second factor.
+YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves, int ntasks);
 
 // End of an evaluation: flags[0..3] into the host-mapped status words
 // (device pointer hflags), all eight flags zeroed.

@@ -179,21 +179,7 @@ __global__ void __launch_bounds__(NW * 32) ui_kernel(WorkArgs a) {
   }
 }
 
-// ------------------------------------------------------------- compute_Y
-// Lanes = 32 consecutive atoms (the paper's warp-of-atoms AoSoA layout,
-// Sec. V-B), so every index and coefficient is uniform across the warp.  The
-// 32 atoms' Ulisttot (re and im planes, [H][32]) is staged into shared memory
-// with one TMA bulk copy per plane.  The contraction of Eq. (z) and the sum of
-// Eq. (y) are walked as one list of terms, sorted by output element:
-//   Y_t[ma][mb] += coef * U_t1[ma1][mb1] * U_t2[ma2][mb2],
-// coef = betaw * C(ma1,ma2) C(mb1,mb2) (with the mirror signs), where a U
-// element past the stored half columns is read conjugated from its mirror.
-// The terms of an output come grouped by their first factor, so a group
-// costs one load and one complex multiply of U_t1 and each term one load and
-// two FMAs: Y += U_t1 * sum_k coef_k U_t2,k.  A term record is a word (two
-// element offsets, conjugation flags, end-of-group and end-of-output bits)
-// and the coefficient.  Each warp owns a contiguous run of outputs, so every
-// Y element is accumulated in registers and written once (no atomics).
+// ------------------------------------------- staging (bulk copies, waits)
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -279,13 +265,6 @@ __device__ bool stage_bulk(void* dst, const void* src, unsigned bytes, uint64_t*
   return ok;
 }
 
-__device__ __forceinline__ float flip_if(float v, unsigned bit) {
-  return __int_as_float(__float_as_int(v) ^ (bit << 31));
-}
-__device__ __forceinline__ double flip_if(double v, unsigned bit) {
-  return bit ? -v : v;
-}
-
 // v with its sign bit XORed with bit 31 of m
 __device__ __forceinline__ float flip_sign(float v, unsigned m) {
   return __int_as_float(__float_as_int(v) ^ (int)m);
@@ -300,33 +279,6 @@ struct YAcc {
   R ar, ai;  // sum of coef * second factor over the current group
 };
 
-// Byte offset of a record's second (first) factor from lane 0's element 0:
-// elements are 256 B apart for complex float, 512 B for complex double.  PF:
-// the FP32 conjugate-plane word, whose top bits are the second factor's
-// offset itself (one shift).
-template <typename R, bool PF>
-__device__ __forceinline__ unsigned y_off2(unsigned w) {
-  if constexpr (PF) return w >> 14;
-  return (w & 0x3FF00u) << (sizeof(R) == 4 ? 0 : 1);
-}
-template <typename R, bool PF>
-__device__ __forceinline__ unsigned y_off1(unsigned w) {
-  if constexpr (PF) return (w & 0x3FFu) << 8;
-  return ((w >> 10) & 0x3FF00u) << (sizeof(R) == 4 ? 0 : 1);
-}
-
-// Term records of compute_Y read straight from global memory (pulled into
-// L1 ahead of use: the stream is read once per CTA).
-template <typename R>
-struct YRecGlobal {
-  static constexpr bool kShared = false;
-  const YRec<R>* __restrict__ rec;
-  __device__ __forceinline__ void at(int q) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + q + kYRecPrefetch));
-  }
-  __device__ __forceinline__ const YRec<R>* ptr(int q) const { return rec + q; }
-};
-
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
@@ -337,278 +289,558 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Term records of compute_Y streamed through a per-warp ring in shared
-// memory: chunks of kYChunk records copied by cp.async (16 bytes a lane),
-// kYRingChunks of them resident or in flight, and the first kYGroupMax
-// records of the chunk in slot 0 mirrored past the ring's end, so that a
-// step of up to kYGroupMax records never wraps.  While the warp's steps
-// start in chunk c, chunks c and c + 1 are complete (a step may run into
-// c + 1) and c + 2, c + 3 are in flight.  A record is then a broadcast
-// shared-memory load instead of a global load through the L1 tags.
-constexpr int kYChunk = 32;
-constexpr int kYRingChunks = 4;
-constexpr int kYRingLen = kYChunk * kYRingChunks + kYGroupMax;
-static_assert(kYChunk % 2 == 0 && kYGroupMax % 2 == 0 && kYGroupMax <= kYChunk, "16-byte copies");
-static_assert(kYChunk * kYRingChunks <= kYRecPad, "ring reads stay in the padding");
+// ------------------------------------------- compute_Y by classes
+// The terms of Eq. (y) ordered for registers.  An element's doubled
+// projections m = (2 ma - t, 2 mb - t) add up in a product, so the outputs of
+// all ranks t with one M are a sum over the pairs m1 + m2 = M of bilinear forms
+//   Y_t[M] += sum_t1 u_t1[m1] sum_t2 c[t][t1][t2] u_t2[m2]
+// of two short vectors (at most J + 1 ranks): both are loaded once, and up to
+// 8 x 8 x 8 coefficients used on them (HostTables::build_classes, whose stream
+// of heads and coefficients a warp walks).  Lanes are the 32 atoms of a block;
+// a warp takes a class (a task) at a time and keeps its outputs in registers.
+//
+// The arithmetic is packed (fma.rn.f32x2) over two outputs t, t + 2: the
+// coefficients come in such pairs, so nothing but u has to be duplicated.
+//
+// The list of terms it replaces took three 128-byte wavefronts of shared memory
+// a term (its record and 8 bytes a lane of the factor) for two FMAs, and was
+// bound by them; here a term takes a quarter of a wavefront (coefficients, four
+// a load) and the vectors about 0.4.  The dense forms hold 7% of zero
+// coefficients at 2J14.  What bounds it now is issue: a packed FMA (two cycles of
+// its pipe) comes with 1.6 other instructions (unpacking the vectors, heads,
+// loops), on 16 warps an SM (2J14, 2000 atoms: issue slots 53% used, shared
+// memory 42%, FMA pipe 36% of the launch).
+// Measured, list of terms -> now: FP32, 2000 atoms, 2J8 41 -> 35 us, 2J11 199 ->
+// 120, 2J14 845 -> 388; 16000 atoms, 2J8 218 -> 179, 2J14 6005 -> 2809; FP64 (in
+// fixed point, below), 2000 atoms, 2J8 404 -> 197, 2J11 2388 -> 944, 2J14 9335 ->
+// 3390; 128 atoms, 2J8 119 -> 29.
+// Chunks of a warp's ring
+__host__ __device__ constexpr int yc_slots(int rsize) { return rsize == 8 ? 2 : 3; }
+// Warps of a CTA, by the longest vector LM: one CTA an SM above 2J = 9 (the
+// block's U fills its shared memory), two up to there, with the registers that
+// FP32 (128 and 64) and fixed point (96) need.
+__host__ __device__ constexpr int yc_warps(int rsize, int LM) { return rsize == 4 ? 16 : LM <= 5 ? 10 : 20; }
 
-// Byte offset of the record rings in compute_Y's dynamic shared memory:
-// after the staged plane(s) of complex float and the 16-byte barrier slot.
-__host__ __device__ constexpr size_t yi_ring_offset(int H, bool cp) {
-  return (size_t)(cp ? 2 : 1) * H * 32 * sizeof(cx<float>) + 16;
+typedef unsigned long long f2;  // two FP32
+
+__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 f2_get(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
-struct YRecRing {
-  static constexpr bool kShared = true;
-  YRec<float>* buf;         // [kYRingLen] of this warp
-  const YRec<float>* base;  // global record qs (qs even: 16-byte aligned)
-  int qs, cross, lane;
-  __device__ __forceinline__ void issue(int c) {  // chunk c into slot c % kYRingChunks
-    const int slot = (c % kYRingChunks) * kYChunk;
-    const YRec<float>* g = base + c * kYChunk;
-    if (lane < kYChunk / 2) {
-      cp_async16(buf + slot + 2 * lane, g + 2 * lane);
-    } else if (slot == 0 && lane < (kYChunk + kYGroupMax) / 2) {
-      const int m = lane - kYChunk / 2;
-      cp_async16(buf + kYChunk * kYRingChunks + 2 * m, g + 2 * m);
-    }
-    cp_async_commit();
-  }
-  __device__ __forceinline__ void init(const YRec<float>* rec, int q0, int ln, YRec<float>* b) {
-    buf = b;
-    lane = ln;
-    qs = q0 & ~1;
-    base = rec + qs;
-    cross = qs + kYChunk;
+// A record's head, unpacked
+struct YcHead {
+  uint4 h;
+  __device__ __forceinline__ explicit YcHead(const unsigned* p) : h(*reinterpret_cast<const uint4*>(p)) {}
+  __device__ __forceinline__ int rows() const { return (int)(h.z & 255u); }
+  __device__ __forceinline__ int len() const { return (int)(h.z >> 8); }
+};
+
+// The records of one length L from p on (h: the first one's head): NP output
+// pairs, rows (t1) of L elements of u[m2].  The next head and the next row's
+// factor are read ahead.
+template <int NP, int L>
+__device__ __forceinline__ void yc_run(const unsigned* __restrict__& p, YcHead& h, const char* __restrict__ ul,
+                                       f2 (&yr)[NP], f2 (&yi)[NP]) {
+  constexpr int LP = (L + 1) & ~1, ROW = NP * LP * 2;
+  do {
+    const int rows = h.rows();
+    const char* u1 = ul + (h.h.x & 0x7FFFFFFFu);
+    const char* u2 = ul + (h.h.y & 0x7FFFFFFFu);
+    const unsigned c1 = h.h.x & 0x80000000u, c2 = h.h.y & 0x80000000u;
+    const unsigned* q = p + 4;
+    p = q + rows * ROW;
+    h = YcHead(p);
+    float2 v = *reinterpret_cast<const float2*>(u1);
+    f2 ar[L], ai[L];
 #pragma unroll
-    for (int c = 0; c < kYRingChunks; ++c) issue(c);
-    cp_async_wait<kYRingChunks - 2>();
-    __syncwarp();
+    for (int c = 0; c < L; ++c) {
+      const float2 w = *reinterpret_cast<const float2*>(u2 + c * 256);
+      const float im = flip_sign(w.y, c2);
+      ar[c] = f2_pack(w.x, w.x);
+      ai[c] = f2_pack(im, im);
+    }
+#pragma unroll 1
+    for (const unsigned* end = p; q != end; q += ROW) {
+      const float im = flip_sign(v.y, c1);
+      const f2 x = f2_pack(v.x, v.x), y = f2_pack(im, im), ny = f2_pack(-im, -im);
+      u1 += 256;  // one row past the vector at the end, inside the CTA's shared memory
+      v = *reinterpret_cast<const float2*>(u1);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        f2 br, bi;
+#pragma unroll
+        for (int c = 0; c < L; c += 2) {
+          const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(q + (k * LP + c) * 2);
+          br = c == 0 ? f2_mul(w.x, ar[c]) : f2_fma(w.x, ar[c], br);
+          bi = c == 0 ? f2_mul(w.x, ai[c]) : f2_fma(w.x, ai[c], bi);
+          if (c + 1 < L) {
+            br = f2_fma(w.y, ar[c + 1], br);
+            bi = f2_fma(w.y, ai[c + 1], bi);
+          }
+        }
+        yr[k] = f2_fma(x, br, yr[k]);
+        yi[k] = f2_fma(x, bi, yi[k]);
+        yr[k] = f2_fma(ny, bi, yr[k]);
+        yi[k] = f2_fma(y, br, yi[k]);
+      }
+    }
+  } while (h.len() == L);
+}
+
+// Running sums of a task's output pairs, and (long sums, 2J > 9) what their
+// roundings lost.
+template <int NPM, bool COMP>
+struct YcSum {
+  f2 r[NPM], i[NPM], er[COMP ? NPM : 1], ei[COMP ? NPM : 1];
+};
+// s += x (COMP: Kahan's sum, e the part of s that is too much)
+template <bool COMP>
+__device__ __forceinline__ void yc_add(f2& s, f2& e, f2 x) {
+  if constexpr (COMP) {
+    const f2 minus = f2_pack(-1.f, -1.f);
+    const f2 y = f2_fma(minus, e, x), t = f2_add(s, y);
+    e = f2_fma(minus, y, f2_fma(minus, s, t));
+    s = t;
+  } else {
+    s = f2_add(s, x);
   }
-  // before a step that starts at record q (steps advance by < kYChunk)
-  __device__ __forceinline__ void at(int q) {
-    if (q >= cross) {
-      issue((cross - qs) / kYChunk - 1 + kYRingChunks);  // into the slot just left
-      cp_async_wait<kYRingChunks - 2>();
-      __syncwarp();
-      cross += kYChunk;
+}
+
+// The records of a chunk (from word 4) of a task with NP output pairs.  A
+// chunk's terms are summed by themselves and then added to the outputs.  The
+// list of terms summed each output in one go; its largest error in Y, relative
+// to the largest Y, was 1.2e-6 at 2J8 and 3.3e-6 at 2J14, here 4e-7 and 6e-7
+// (one long sum in this order: 1.4e-6 and 1.9e-6).
+template <int NP, int LM, int NPM, bool COMP>
+__device__ __forceinline__ void yc_chunk(const unsigned* __restrict__ p, const char* __restrict__ ul,
+                                         YcSum<NPM, COMP>& s) {
+  f2 yr[NP], yi[NP];
+#pragma unroll
+  for (int k = 0; k < NP; ++k) yr[k] = yi[k] = 0;
+  YcHead h(p);
+  while (h.rows() != 0) {
+    switch (h.len()) {
+#define SNAP_YC(L) \
+  case L: \
+    if constexpr (L <= LM) yc_run<NP, L>(p, h, ul, yr, yi); \
+    break;
+      SNAP_YC(1) SNAP_YC(2) SNAP_YC(3) SNAP_YC(4) SNAP_YC(5) SNAP_YC(6) SNAP_YC(7) SNAP_YC(8)
+#undef SNAP_YC
+      default: return;
     }
   }
-  __device__ __forceinline__ const YRec<float>* ptr(int q) const {
-    return buf + ((q - qs) & (kYChunk * kYRingChunks - 1));
+#pragma unroll
+  for (int k = 0; k < NP; ++k) {
+    yc_add<COMP>(s.r[k], s.er[COMP ? k : 0], yr[k]);
+    yc_add<COMP>(s.i[k], s.ei[COMP ? k : 0], yi[k]);
+  }
+}
+
+// The two precisions of the walk below: what a task's outputs are held in, how
+// a chunk adds to them and how they are stored.
+template <int LM>
+struct YcSingle {
+  static constexpr int kAtoms = 32;  // of a block; a row is their [32] of an element
+  static constexpr int kWarps = yc_warps(4, LM);  // of a CTA
+  static constexpr int kSlots = yc_slots(4);
+  static constexpr int NPM = LM > 5 ? 4 : 2;
+  static constexpr bool COMP = LM > 5;
+  YcSum<NPM, COMP> y;
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < NPM; ++k) y.r[k] = y.i[k] = y.er[COMP ? k : 0] = y.ei[COMP ? k : 0] = 0;
+  }
+  __device__ __forceinline__ void chunk(unsigned np, const unsigned* __restrict__ p, const char* __restrict__ ul, int) {
+    switch (np) {
+#define SNAP_YC(NP) \
+  case NP: \
+    if constexpr (NP <= NPM) yc_chunk<NP, LM, NPM, COMP>(p, ul, y); \
+    break;
+      SNAP_YC(1) SNAP_YC(2) SNAP_YC(3) SNAP_YC(4)
+#undef SNAP_YC
+      default: break;
+    }
+  }
+  // the outputs, plus those at `other` if it is given, to Yb
+  __device__ __forceinline__ void store(const int* __restrict__ rec, uint4, char* Yb, const char* other, int lane,
+                                        int) const {
+    cx<float>* Yg = reinterpret_cast<cx<float>*>(Yb) + lane;
+    const int nout = __ldg(rec + 2);
+#pragma unroll
+    for (int k = 0; k < NPM; ++k) {
+      const float2 r = f2_get(y.r[k]), i = f2_get(y.i[k]);
+#pragma unroll
+      for (int o = 0; o < 2; ++o)
+        if (2 * k + o < nout) {
+          const int at = __ldg(rec + 4 + 2 * k + o) * 32;
+          cx<float> v = o == 0 ? mk<float>(r.x, i.x) : mk<float>(r.y, i.y);
+          if (other) {
+            const cx<float> w = reinterpret_cast<const cx<float>*>(other)[at + lane];
+            v = mk<float>(v.re + w.re, v.im + w.im);
+          }
+          Yg[at] = v;
+          // the mirror below the centre of the middle column, which no
+          // contraction reads
+          const int z = __ldg(rec + 4 + kYcOuts + 2 * k + o);
+          if (z >= 0) Yg[z * 32] = mk<float>(0.f, 0.f);
+        }
+    }
   }
 };
 
-// B consecutive groups of K terms from record q: every record and both
-// factors are loaded ahead of the arithmetic (no branch inside), then per
-// group acc = sum_k coef_k U2,k and Y += U1 * acc.  `ul` points at lane 0's
-// element 0 plus this lane.  CP: the staged block is [2][H][32] with the
-// conjugate in its second half (no sign flips).
-template <typename R, bool CP, int K, int B, typename Src>
-__device__ __forceinline__ void y_groups(Src& src, int q, const char* __restrict__ ul, R& yre, R& yim) {
-  src.at(q);
-  const YRec<R>* rp = src.ptr(q);
-  unsigned w[B * K];
-  R c[B * K];
-#pragma unroll
-  for (int j = 0; j < B * K; ++j) {
-    if constexpr (sizeof(R) == 4) {
-      const uint2 r = Src::kShared ? *reinterpret_cast<const uint2*>(rp + j)
-                                   : __ldg(reinterpret_cast<const uint2*>(rp + j));
-      w[j] = r.x;
-      c[j] = __uint_as_float(r.y);
-    } else {
-      const uint4 r = __ldg(reinterpret_cast<const uint4*>(rp + j));
-      w[j] = r.x;
-      c[j] = (R)__hiloint2double((int)r.w, (int)r.z);
-    }
-  }
-  constexpr bool PF = sizeof(R) == 4 && CP;
-  cx<R> u2[B * K], u1[B];
-#pragma unroll
-  for (int j = 0; j < B * K; ++j) u2[j] = *reinterpret_cast<const cx<R>*>(ul + y_off2<R, PF>(w[j]));
-#pragma unroll
-  for (int b = 0; b < B; ++b) u1[b] = *reinterpret_cast<const cx<R>*>(ul + y_off1<R, PF>(w[b * K]));
-#pragma unroll
-  for (int b = 0; b < B; ++b) {
-    R ar = R(0), ai = R(0);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int j = b * K + k;
-      ar += c[j] * u2[j].re;
-      ai += c[j] * (CP ? u2[j].im : flip_sign(u2[j].im, w[j] & 0x80000000u));
-    }
-    const R i1 = CP ? u1[b].im : flip_sign(u1[b].im, (w[b * K] << 1) & 0x80000000u);
-    yre = fmr(-i1, ai, fmr(u1[b].re, ar, yre));
-    yim = fmr(i1, ar, fmr(u1[b].re, ai, yim));
-  }
+// FP64 in fixed point.  The FP64 pipe does a warp's multiply-add in 15 cycles
+// of an SM; the integer pipe a 32 x 32 + 64 bit one in half a cycle.  So the
+// block's U and the coefficients are held as two limbs (59 bits and a sign,
+// more than the 53 of a double) and a product is three integer multiply-adds,
+// hi hi and the two cross ones; the fourth is below the last bit.
+//   u = (h 2^30 + l) 2^(s - 59), |h| <= 2^29, |l| <= 2^29, 2^s above the atom's
+//     largest component of U (yf_prepare; rounded to nearest, exact for
+//     components above 2^-6 of the largest);
+//   c = (h 2^30 + l) 2^(e - 60), |l| <= 2^29, 2^e above the largest sum of |c|
+//     over a record (m1, m2) of its output;
+//   a row's sum A = sum_t2 c u is rounded at 2^-59 and split into h, l again,
+//     and u A, formed in the same way and summed over the record, is added to
+//     the output's 96-bit sum, which is exact.
+// Sums of a record stay below 2^63: with sum |h(c)| <= 2^30 and |A| <= 2^59,
+//   hi hi: 2^59, 2 x 2^59; cross: 2^59 + 8 2^58, 2 (8 2^58 + 2^59).
+// A rounding here is 2^-59 of the largest |U| (twice in a product) times the
+// largest sum of |c|, where FP64 rounds at 2^-53 of each partial sum.  Measured
+// against 64 bits, largest error of a step's energies, forces and virial, FP64
+// list of terms / fixed point: 2J8 128 atoms 6.3e-15 / 6.5e-15, 2000 atoms 7.0e-15
+// / 7.2e-15, 2J14 2000 atoms 2.8e-15 / 2.9e-15 (most of it from U and dE).
+//
+// A block is 16 atoms (a row of 16 x 16 bytes is then 256, as in FP32, and the
+// whole of 2J14 stays in shared memory); a warp's halves take the two outputs
+// of a task.
+__device__ __forceinline__ void wide_add(long long& s, int x, int y) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(x), "r"(y));
 }
 
-// FP64 path: one term at a time with the group-end and output-end bits of
-// the record (FP64 arithmetic, not the integer work around it, bounds that
-// path, and this loop keeps its registers low).
-template <typename R, bool CP>
-__device__ __forceinline__ void y_term(unsigned w, R c, cx<R> u2, const char* __restrict__ ul,
-                                       cx<R>* __restrict__ Yg, int lane, int& o, YAcc<R>& y) {
-  const R i2 = CP ? u2.im : flip_sign(u2.im, w & 0x80000000u);
-  y.ar += c * u2.re;
-  y.ai += c * i2;
-  if (w & (1u << 28)) {
-    const cx<R> u1 = *reinterpret_cast<const cx<R>*>(ul + y_off1<R, false>(w));
-    const R i1 = CP ? u1.im : flip_sign(u1.im, (w << 1) & 0x80000000u);
-    y.re = fmr(-i1, y.ai, fmr(u1.re, y.ar, y.re));
-    y.im = fmr(i1, y.ar, fmr(u1.re, y.ai, y.im));
-    y.ar = R(0);
-    y.ai = R(0);
-    if (w & (1u << 29)) {
-      Yg[o * 32 + lane] = mk<R>(y.re, y.im);
-      y.re = R(0);
-      y.im = R(0);
-      ++o;
-    }
+struct Acc96 {
+  unsigned lo, mid, hi;
+  __device__ __forceinline__ void add(long long v) {
+    const unsigned l = (unsigned)v, h = (unsigned)(v >> 32), s = (unsigned)((int)h >> 31);
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(lo), "+r"(mid), "+r"(hi)
+        : "r"(l), "r"(h), "r"(s));
   }
-}
-
-// All groups of K terms of one output (a run of `ng` groups from record q).
-template <typename R, bool CP, int K, typename Src>
-__device__ __forceinline__ void y_run(Src& src, int& q, int ng, const char* __restrict__ ul, R& yre, R& yim) {
-  constexpr int B = K >= 8 ? 1 : 8 / K;  // groups per step: about 8 records
-  static_assert(B * K <= kYGroupMax, "a step fits the record ring's mirror");
-  for (; ng >= B; ng -= B, q += B * K) y_groups<R, CP, K, B>(src, q, ul, yre, yim);
-  for (; ng > 0; --ng, q += K) y_groups<R, CP, K, 1>(src, q, ul, yre, yim);
-}
-
-// One warp's outputs [o0, o1): per output its runs of 1-, 2-, ... 8-term
-// groups (branch-free bodies of known length).  The records of consecutive
-// outputs are consecutive, and the next output's run header is loaded while
-// the current one is computed.
-template <typename R, bool CP, typename Src>
-__device__ __forceinline__ void y_outputs(Src& src, const uint4* __restrict__ runs, int q, int o0, int o1,
-                                          const char* __restrict__ ul, cx<R>* __restrict__ Yg, int lane) {
-  static_assert(kYGroupMax == 8, "one 16-byte run header per output");
-  uint4 h = __ldg(runs + o0);
-  for (int o = o0; o < o1; ++o) {
-    const uint4 hn = __ldg(runs + min(o + 1, o1 - 1));
-    R yre = R(0), yim = R(0);
-    y_run<R, CP, 1>(src, q, (int)(h.x & 0xffffu), ul, yre, yim);
-    y_run<R, CP, 2>(src, q, (int)(h.x >> 16), ul, yre, yim);
-    y_run<R, CP, 3>(src, q, (int)(h.y & 0xffffu), ul, yre, yim);
-    y_run<R, CP, 4>(src, q, (int)(h.y >> 16), ul, yre, yim);
-    y_run<R, CP, 5>(src, q, (int)(h.z & 0xffffu), ul, yre, yim);
-    y_run<R, CP, 6>(src, q, (int)(h.z >> 16), ul, yre, yim);
-    y_run<R, CP, 7>(src, q, (int)(h.w & 0xffffu), ul, yre, yim);
-    y_run<R, CP, 8>(src, q, (int)(h.w >> 16), ul, yre, yim);
-    Yg[o * 32 + lane] = mk<R>(yre, yim);
-    h = hn;
+  __device__ __forceinline__ double value() const {
+    return fma((double)(long long)(((unsigned long long)hi << 32) | mid), 4294967296.0, (double)lo);
   }
+};
+
+// hi hi and cross sums to one number, rounded (the cross sum starts at half
+// of 2^30), plus 2^29
+constexpr long long kYcRound = 1LL << 29, kYcSplit = kYcRound + (1LL << 59);
+// limbs of v, given v + 2^29
+__device__ __forceinline__ void split30(long long v, int& h, int& l) {
+  h = (int)(v >> 30);
+  l = (int)((unsigned)v & 0x3FFFFFFFu) - (1 << 29);
 }
 
-// One warp's outputs of slice `slice` for the 32-atom block blk, with the
-// block's U at `us` (staged in shared memory or in global memory).
-template <typename R, bool STAGED, bool CP>
-__device__ __forceinline__ void yi_slice(const WorkArgs& a, unsigned char* smem, const cx<R>* us, long blk,
-                                         int slice, int warp, int lane) {
-  if (slice >= a.nslices) return;
-  const int H = a.H;
-  const int o0 = a.yslice[slice], o1 = a.yslice[slice + 1];
-  if (o0 >= o1) return;
-  cx<R>* Yg = reinterpret_cast<cx<R>*>(a.Y) + blk * H * 32;
-  const YRec<R>* __restrict__ rec = reinterpret_cast<const YRec<R>*>(a.yrec);
-  const char* ul = reinterpret_cast<const char*>(us + lane);
-  if constexpr (sizeof(R) == 8) {
-    // FP64: the terms of the slice in order, four records per batch
-    int q = a.yfirst[o0];
-    const int q1 = a.yfirst[o1];
-    int o = o0;
-    YAcc<R> y;
-    y.re = y.im = y.ar = y.ai = R(0);
-    for (; q + 4 <= q1; q += 4) {
-      uint4 v[4];
+// yc_run in fixed point: one output a lane
+template <int L>
+__device__ __forceinline__ void yf_run(const unsigned* __restrict__& p, YcHead& h, const char* __restrict__ ul, int half,
+                                       Acc96& yr, Acc96& yi) {
+  constexpr int LP = (L + 1) & ~1, ROW = LP * 4;
+  do {
+    const char* u1 = ul + (h.h.x & 0x7FFFFFFFu);
+    const char* u2 = ul + (h.h.y & 0x7FFFFFFFu);
+    // conj(u1) v = conj(u1 conj(v)): u[m1] is taken as it is
+    const int c1 = (int)h.h.x >> 31, c2 = c1 ^ ((int)h.h.y >> 31);  // -1: conjugate
+    const unsigned* q = p + 4 + half * LP * 2;
+    p += 4 + h.rows() * ROW;
+    const unsigned* end = p + half * LP * 2;
+    h = YcHead(p);
+    int4 v = *reinterpret_cast<const int4*>(u1);
+    int4 a[L];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = __ldg(reinterpret_cast<const uint4*>(rec + q + k));
-      cx<R> u2[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) u2[k] = *reinterpret_cast<const cx<R>*>(ul + y_off2<R, false>(v[k].x));
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        y_term<R, CP>(v[k].x, (R)__hiloint2double((int)v[k].w, (int)v[k].z), u2[k], ul, Yg, lane, o, y);
+    for (int c = 0; c < L; ++c) {
+      a[c] = *reinterpret_cast<const int4*>(u2 + c * 256);
+      a[c].z = (a[c].z ^ c2) - c2;
+      a[c].w = (a[c].w ^ c2) - c2;
     }
-    for (; q < q1; ++q)
-      y_term<R, CP>(rec[q].w, rec[q].c, *reinterpret_cast<const cx<R>*>(ul + y_off2<R, false>(rec[q].w)), ul, Yg,
-                    lane, o, y);
-  } else {
-    // FP32: the records through the warp's ring in shared memory (staged
-    // CTAs; the ring sits after the staged planes and their barrier)
-    const uint4* runs = reinterpret_cast<const uint4*>(a.yruns);  // 8 u16 counts per output
-    const int q0 = a.yfirst[o0];
-    if constexpr (STAGED) {
-      YRec<float>* rb = reinterpret_cast<YRec<float>*>(smem + yi_ring_offset(H, CP)) + warp * kYRingLen;
-      YRecRing src;
-      src.init(rec, q0, lane, rb);
-      y_outputs<R, CP>(src, runs, q0, o0, o1, ul, Yg, lane);
-      cp_async_wait<0>();  // no copy outlives the warp's slice
-    } else {
-      YRecGlobal<R> src{rec};
-      y_outputs<R, CP>(src, runs, q0, o0, o1, ul, Yg, lane);
-    }
-  }
-}
-
-// CTA = one 32-atom block x one ysplit-th of the outputs; U of the block
-// staged by a TMA bulk copy.
-template <typename R, bool STAGED, bool CP>
-__global__ void __launch_bounds__(STAGED ? 1024 : 256, 1) yi_kernel(WorkArgs a) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long blk0 = blockIdx.x;
-  const int H = a.H;
-  const cx<R>* us = reinterpret_cast<const cx<R>*>(a.U) + blk0 * H * 32;
-  if (STAGED) {
-    cx<R>* su = reinterpret_cast<cx<R>*>(smem);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(su + (CP ? 2 : 1) * H * 32);
-    const unsigned bytes = (unsigned)(H * 32 * sizeof(cx<R>));
-    if (!stage_bulk(su, us, bytes, bar, a.flags, a.test_skip_stage != 0, [] {})) return;
-    if (CP) {
-      for (int e = threadIdx.x; e < H * 32; e += blockDim.x) {
-        const cx<R> v = su[e];
-        su[H * 32 + e] = mk<R>(v.re, -v.im);
+    long long ph = 0, qh = 0, pc = kYcRound, qc = kYcRound;
+#pragma unroll 1
+    for (; q != end; q += ROW) {
+      const int4 x = v;
+      u1 += 256;  // one row past the vector at the end, inside the CTA's shared memory
+      v = *reinterpret_cast<const int4*>(u1);
+      long long rh = 0, rc = kYcSplit, ih = 0, ic = kYcSplit;
+#pragma unroll
+      for (int c = 0; c < L; c += 2) {
+        const int4 w = *reinterpret_cast<const int4*>(q + c * 2);
+        wide_add(rh, w.x, a[c].x);
+        wide_add(ih, w.x, a[c].z);
+        wide_add(rc, w.x, a[c].y);
+        wide_add(ic, w.x, a[c].w);
+        wide_add(rc, w.y, a[c].x);
+        wide_add(ic, w.y, a[c].z);
+        if (c + 1 < L) {
+          wide_add(rh, w.z, a[c + 1].x);
+          wide_add(ih, w.z, a[c + 1].z);
+          wide_add(rc, w.z, a[c + 1].y);
+          wide_add(ic, w.z, a[c + 1].w);
+          wide_add(rc, w.w, a[c + 1].x);
+          wide_add(ic, w.w, a[c + 1].z);
+        }
       }
-      __syncthreads();
+      int Ah, Al, Bh, Bl;
+      split30(rh + (rc >> 30), Ah, Al);
+      split30(ih + (ic >> 30), Bh, Bl);
+      const int nz = -x.z, nw = -x.w;
+      wide_add(ph, x.x, Ah);
+      wide_add(qh, x.x, Bh);
+      wide_add(pc, x.x, Al);
+      wide_add(qc, x.x, Bl);
+      wide_add(ph, nz, Bh);
+      wide_add(qh, x.z, Ah);
+      wide_add(pc, x.y, Ah);
+      wide_add(qc, x.y, Bh);
+      wide_add(pc, nz, Bl);
+      wide_add(qc, x.z, Al);
+      wide_add(pc, nw, Bh);
+      wide_add(qc, x.w, Ah);
     }
-    us = su;
-  }
-  yi_slice<R, STAGED, CP>(a, smem, us, blk0, blockIdx.y * (blockDim.x >> 5) + warp, warp, lane);
+    yr.add(ph + (pc >> 30));
+    const long long q2 = qh + (qc >> 30);
+    yi.add((q2 ^ c1) - c1);
+  } while (h.len() == L);
 }
 
-// The same work as a persistent launch over a work queue: a grid of resident
-// CTAs, each taking (block, split) items from a device counter (flags[5],
-// zeroed with the flags by every evaluation) until the items run out, across
-// all configurations of a batch.  No CTA waits on another (the counter is the
-// only shared state), and an item's arithmetic is that of the CTA it would
-// have been, so the results are bit for bit those of yi_kernel.  The staging
+template <int LM>
+struct YcFixed {
+  static constexpr int kAtoms = 16;
+  static constexpr int kWarps = yc_warps(8, LM);
+  static constexpr int kSlots = yc_slots(8);
+  Acc96 yr, yi;
+  __device__ __forceinline__ void clear() { yr = yi = Acc96{0u, 0u, 0u}; }
+  __device__ __forceinline__ void chunk(unsigned, const unsigned* __restrict__ p, const char* __restrict__ ul, int half) {
+    YcHead h(p);
+    while (h.rows() != 0) {
+      switch (h.len()) {
+#define SNAP_YC(L) \
+  case L: \
+    if constexpr (L <= LM) yf_run<L>(p, h, ul, half, yr, yi); \
+    break;
+        SNAP_YC(1) SNAP_YC(2) SNAP_YC(3) SNAP_YC(4) SNAP_YC(5) SNAP_YC(6) SNAP_YC(7) SNAP_YC(8)
+#undef SNAP_YC
+        default: return;
+      }
+    }
+  }
+  // `ex`: the exponent of the lane's atom, or kBad
+  static constexpr int kBad = 1 << 20;
+  __device__ __forceinline__ void store(const int* __restrict__ rec, uint4 h, char* Yb, const char* other, int lane,
+                                        int ex) const {
+    const int o = lane >> 4;
+    if (o >= __ldg(rec + 2)) return;
+    const int ec = (int)(o ? h.w : h.z), n = 2 * ex + ec - 58;
+    // 2^n in two factors (a coefficient may be as small or large as a double)
+    const int n1 = n >> 1, n2 = n - n1;
+    double f1 = __hiloint2double((n1 + 1023) << 20, 0);
+    const double f2 = __hiloint2double((n2 + 1023) << 20, 0);
+    if (ex == kBad || ec == kYcNan) f1 = __longlong_as_double(0x7FF8000000000000LL);
+    const int at = __ldg(rec + 4 + o) * 32 + (lane & 15);
+    cx<double> v = mk<double>(yr.value() * f1 * f2, yi.value() * f1 * f2);
+    if (other) {
+      const cx<double> w = reinterpret_cast<const cx<double>*>(other)[at];
+      v = mk<double>(v.re + w.re, v.im + w.im);
+    }
+    reinterpret_cast<cx<double>*>(Yb)[at] = v;
+    const int z = __ldg(rec + 4 + kYcOuts + o);
+    if (z >= 0) reinterpret_cast<cx<double>*>(Yb)[z * 32 + (lane & 15)] = mk<double>(0.0, 0.0);
+  }
+};
+
+// The staged block of U, [H][16] complex double, to fixed point in place;
+// returns the exponent of the lane's atom (kBad if its U is not finite).
+__device__ int yf_prepare(unsigned char* su, int H, int* top) {
+  // top: [16] in shared memory.  A thread has one atom throughout.
+  const int al = threadIdx.x & 15, n = H * 16;
+  if (threadIdx.x < 16) top[threadIdx.x] = 0;
+  __syncthreads();
+  int m = 0;  // the larger of two magnitudes has the larger high word
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const int4 v = *reinterpret_cast<const int4*>(su + (size_t)e * 16);
+    m = max(m, max(v.y & 0x7FFFFFFF, v.w & 0x7FFFFFFF));
+  }
+  atomicMax(top + al, m);
+  __syncthreads();
+  const int E = max(top[al] >> 20, 1022 - 150);  // biased exponent; U below 2^-150 has that scale
+  auto fixed = [&](int lo, int hi, int& h, int& l) {
+    const int e = (hi >> 20) & 0x7FF;
+    // |x| = M 2^(e - 1075) = v 2^(E - 1022 - 59)
+    const unsigned long long M = ((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)lo;
+    const int sh = e - E + 6;
+    unsigned long long v = 0;
+    if (sh >= 0) v = M << (sh & 7);
+    else if (sh > -55) v = (M + (1ull << (-sh - 1))) >> -sh;
+    if (e == 0) v = 0;
+    split30((hi < 0 ? -(long long)v : (long long)v) + kYcRound, h, l);
+  };
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    int4* x = reinterpret_cast<int4*>(su + (size_t)e * 16);
+    const int4 v = *x;
+    int4 w;
+    fixed(v.x, v.y, w.x, w.y);
+    fixed(v.z, v.w, w.z, w.w);
+    *x = w;
+  }
+  return (top[al] >> 20) == 0x7FF ? YcFixed<8>::kBad : E - 1022;
+}
+
+// One warp's share of a CTA's tasks (tl: first chunk and chunks of each),
+// taken from a counter in shared memory: a task's outputs have one warp, so
+// nothing depends on which.  Chunks come through the warp's ring, the next
+// task's behind the last of the one before.
+template <class P>
+__device__ __forceinline__ void yc_tasks(const WorkArgs& a, const char* __restrict__ ul, unsigned* __restrict__ ring,
+                                         const int2* __restrict__ tl, int nt, int* next, int* met, size_t at, int lane,
+                                         int ex) {
+  P y;
+  y.clear();
+  int pc = 0, left = 0, live = 0, slot = 0;
+  bool more = true;
+  auto issue = [&](int s) {
+    if (left == 0 && more) {
+      int k = 0;
+      if (lane == 0) k = atomicAdd(next, 1);
+      k = __shfl_sync(kFull, k, 0);
+      more = k < nt;
+      if (more) {
+        pc = tl[k].x;
+        left = tl[k].y;
+      }
+    }
+    if (left > 0) {
+      const unsigned* g = a.yc_stream + (size_t)pc * kYcChunk + lane * 4;
+      unsigned* d = ring + s * kYcChunk + lane * 4;
+      cp_async16(d, g);
+      cp_async16(d + kYcChunk / 2, g + kYcChunk / 2);
+      ++pc;
+      --left;
+      ++live;
+    }
+    cp_async_commit();
+  };
+  static_assert(kYcChunk == 256, "two 16-byte copies a lane");
+#pragma unroll
+  for (int s = 0; s < P::kSlots - 1; ++s) issue(s);
+  while (live > 0) {
+    cp_async_wait<P::kSlots - 2>();
+    __syncwarp();
+    issue(slot == 0 ? P::kSlots - 1 : slot - 1);  // the slot of the chunk before
+    const unsigned* ch = ring + slot * kYcChunk;
+    const uint4 h = *reinterpret_cast<const uint4*>(ch);
+    y.chunk(h.y, ch + 4, ul, lane >> 4);
+    if (h.x >> 31) {  // the task's last chunk
+      const int* rec = a.yc_task + (size_t)(h.x & 0x7FFFFFFFu) * kYcTask;
+      const int half = __ldg(rec + 3);
+      char* Y = static_cast<char*>(a.Y) + at;
+      if (half == 0) {
+        y.store(rec, h, Y, nullptr, lane, ex);
+      } else {
+        // The sum's other half may be another warp's: each leaves its own (the
+        // first in Y, the second in Y2), and the one that comes second adds the
+        // two (a sum of two, so their order does not matter).
+        char* Y2 = static_cast<char*>(a.Y2) + at;
+        y.store(rec, h, (half & 1) ? Y2 : Y, nullptr, lane, ex);
+        __threadfence_block();
+        __syncwarp();
+        int first = 0;
+        if (lane == 0) first = atomicAdd(met + (half >> 1) - 1, 1) == 0;
+        first = __shfl_sync(kFull, first, 0);
+        if (!first) {
+          __threadfence_block();
+          y.store(rec, h, Y, (half & 1) ? Y : Y2, lane, ex);
+        }
+      }
+      y.clear();
+    }
+    --live;
+    slot = slot == P::kSlots - 1 ? 0 : slot + 1;
+  }
+  cp_async_wait<0>();  // no copy outlives the warp's tasks
+}
+
+// Shared memory: the block's U in class-major order (256 bytes an element),
+// the barrier, the rings, the CTA's tasks, and per split sum how many halves
+// are done.
+__host__ __device__ constexpr size_t yc_ring_offset(int H) { return (size_t)H * 256 + 16; }
+__host__ __device__ constexpr size_t yc_smem(int rsize, int H, int ntasks, int warps) {
+  return yc_ring_offset(H) + (size_t)warps * yc_slots(rsize) * kYcChunk * 4 + (size_t)ntasks * (sizeof(int2) + sizeof(int));
+}
+
+// CTA = one block of atoms x one ysplit-th of the tasks; U of the block staged
+// by TMA bulk copies, one an element (256 bytes), which put it in class-major
+// order.  QUEUE: a persistent launch, (block, split) items from a device
+// counter (flags[5], zeroed with the flags by every evaluation); the staging
 // barrier is reused item after item (its phase flips per completed copy).
-template <typename R, bool CP>
-__global__ void __launch_bounds__(1024, 1) yi_queue_kernel(WorkArgs a, int ysplit) {
+template <class P, int LM, bool QUEUE>
+__global__ void __launch_bounds__(P::kWarps * 32, LM <= 5 ? 2 : 1) yc_kernel(WorkArgs a, int ysplit) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ int item_s;
+  __shared__ int item_s, next_s, top_s[16];
+  constexpr bool FIXED = P::kAtoms == 16;
+  constexpr int kRow = FIXED ? 512 : 256;  // bytes of an element's 32 atoms in global memory
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int H = a.H;
-  const long nitems = (long)((a.n + 31) / 32) * ysplit;
-  cx<R>* su = reinterpret_cast<cx<R>*>(smem);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(su + (CP ? 2 : 1) * H * 32);
-  const unsigned bytes = (unsigned)(H * 32 * sizeof(cx<R>));
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)H * 256);
+  unsigned* ring = reinterpret_cast<unsigned*>(smem + yc_ring_offset(H)) + warp * P::kSlots * kYcChunk;
+  int2* tl = reinterpret_cast<int2*>(smem + yc_ring_offset(H) + (size_t)P::kWarps * P::kSlots * kYcChunk * 4);
+  int* met = reinterpret_cast<int*>(tl + a.yc_ntask);
+  const long nitems = (long)((a.n + P::kAtoms - 1) / P::kAtoms) * ysplit;
   if (threadIdx.x == 0) mbar_init(bar, 1);
   unsigned phase = 0;
-  for (;;) {
-    if (threadIdx.x == 0) item_s = atomicAdd(&a.flags[5], 1);
-    __syncthreads();  // also: every warp is done with the previous block
-    const long item = item_s;
-    if (item >= nitems) break;
+  for (long item = blockIdx.x;;) {
+    if (QUEUE) {
+      if (threadIdx.x == 0) item_s = atomicAdd(&a.flags[5], 1);
+      __syncthreads();  // also: every warp is done with the previous block
+      item = item_s;
+      if (item >= nitems) break;
+    }
     const long blk = item / ysplit;
     const int part = (int)(item - blk * ysplit);
+    // the block's first atom in the [ceil(N / 32)][H][32] buffers
+    const size_t at = FIXED ? (size_t)(blk >> 1) * H * kRow + (blk & 1) * 256 : (size_t)blk * H * kRow;
     if (threadIdx.x == 0) {
-      mbar_expect_tx(bar, bytes);
-      if (!a.test_skip_stage) bulk_g2s(su, reinterpret_cast<const cx<R>*>(a.U) + blk * H * 32, bytes, bar);
+      next_s = 0;
+      mbar_expect_tx(bar, (unsigned)(H * 256));
     }
+    __syncthreads();
+    if (!a.test_skip_stage) {
+      const char* ug = static_cast<const char*>(a.U) + at;
+      for (int e = threadIdx.x; e < H; e += blockDim.x)
+        bulk_g2s(smem + (size_t)__ldg(a.yc_slot + e) * 256, ug + (size_t)e * kRow, 256, bar);
+    }
+    const int b0 = a.yc_bins[part], nt = a.yc_bins[part + 1] - b0;
+    for (int k = threadIdx.x; k < nt; k += blockDim.x) {
+      const int* rec = a.yc_task + (size_t)a.yc_bins[ysplit + 1 + b0 + k] * kYcTask;
+      tl[k] = make_int2(__ldg(rec), __ldg(rec + 1));
+    }
+    for (int k = threadIdx.x; k < a.yc_ntask; k += blockDim.x) met[k] = 0;
     const bool ok = __syncthreads_and(mbar_wait_bounded(bar, phase, kWaitNs));
     if (!ok) {
       if (threadIdx.x == 0) atomicMax(&a.flags[3], 1);
@@ -616,15 +848,15 @@ __global__ void __launch_bounds__(1024, 1) yi_queue_kernel(WorkArgs a, int yspli
       return;
     }
     phase ^= 1u;
-    if (CP) {
-      for (int e = threadIdx.x; e < H * 32; e += blockDim.x) {
-        const cx<R> v = su[e];
-        su[H * 32 + e] = mk<R>(v.re, -v.im);
-      }
+    int ex = 0;
+    if (FIXED) {
+      ex = yf_prepare(smem, H, top_s);
       __syncthreads();
     }
-    yi_slice<R, true, CP>(a, smem, su, blk, part * (blockDim.x >> 5) + warp, warp, lane);
-    __syncthreads();  // item_s is rewritten next
+    yc_tasks<P>(a, reinterpret_cast<const char*>(smem) + (FIXED ? (lane & 15) * 16 : lane * 8), ring, tl, nt, &next_s,
+                met, at, lane, ex);
+    if (!QUEUE) break;
+    __syncthreads();  // item_s and the staged block are rewritten next
   }
 }
 
@@ -633,7 +865,10 @@ __global__ void __launch_bounds__(1024, 1) yi_queue_kernel(WorkArgs a, int yspli
 // Sec. V-B): warp = one atom, its Ulisttot and conj(Ulisttot) staged in shared
 // memory as a [2][H] block, lanes over output elements (dealt to the lanes in
 // decreasing term count, snake order, so their loads balance); each lane walks
-// its outputs' term records in the same grouped order as yi_kernel.
+// its outputs' term records, grouped by their first factor:
+//   Y += U_e1 * sum_k coef_k U_e2,k
+// (a word: two element offsets, conjugation flags, end-of-group and
+// end-of-output bits; and the coefficient).
 constexpr int kYaWarps = 8;
 
 template <typename R>
@@ -654,33 +889,48 @@ __global__ void __launch_bounds__(kYaWarps * 32) yi_atom_kernel(WorkArgs a) {
   __syncwarp();
   cx<R>* Yg = reinterpret_cast<cx<R>*>(a.Y) + base;
   const YRec<R>* __restrict__ rec = reinterpret_cast<const YRec<R>*>(a.yrec);
-  const bool pf = yrec_plane_format((int)sizeof(R), H);
   const int m = a.ysched_m;
   for (int k = 0; k < m; ++k) {
     const int o = a.ysched[lane * m + k];
     if (o < 0) break;
     YAcc<R> y;
     y.re = y.im = y.ar = y.ai = R(0);
+    // every 16 groups are summed by themselves and added up by Kahan's sum (a
+    // long FP32 sum is further off)
+    R sr = R(0), si = R(0), er = R(0), ei = R(0);
+    auto add = [](R& s, R& e, R x) {
+      const R v = x - e, t = s + v;
+      e = (t - s) - v;
+      s = t;
+    };
+    int groups = 0;
     const int q1 = a.yfirst[o + 1];
     for (int q = a.yfirst[o]; q < q1; ++q) {
       const unsigned w = rec[q].w;
       const R c = rec[q].c;
       // elements of the factors in the [2][H] block: the staged-conjugate
-      // record formats index it directly, the other one sets the sign bits
-      const int e2 = pf ? (int)(w >> 22) : (int)((w >> 8) & 1023u) + (int)(w >> 31) * H;
+      // record format indexes it directly, the other one sets the sign bits
+      const int e2 = (int)((w >> 8) & 1023u) + (int)(w >> 31) * H;
       const cx<R> u2 = ua[e2];
       y.ar += c * u2.re;
       y.ai += c * u2.im;
-      if (w & (pf ? (1u << 12) : (1u << 28))) {
-        const int e1 = pf ? (int)(w & 1023u) : (int)((w >> 18) & 1023u) + (int)((w >> 30) & 1u) * H;
+      if (w & (1u << 28)) {
+        const int e1 = (int)((w >> 18) & 1023u) + (int)((w >> 30) & 1u) * H;
         const cx<R> u1 = ua[e1];
         y.re = fmr(-u1.im, y.ai, fmr(u1.re, y.ar, y.re));
         y.im = fmr(u1.im, y.ar, fmr(u1.re, y.ai, y.im));
         y.ar = R(0);
         y.ai = R(0);
+        if ((++groups & 15) == 0) {
+          add(sr, er, y.re);
+          add(si, ei, y.im);
+          y.re = y.im = R(0);
+        }
       }
     }
-    Yg[(long)o * 32] = mk<R>(y.re, y.im);
+    add(sr, er, y.re);
+    add(si, ei, y.im);
+    Yg[(long)o * 32] = mk<R>(sr, si);
   }
 }
 
@@ -1194,81 +1444,58 @@ cudaError_t launch_ui(const WorkArgs& a, cudaStream_t s) {
   return launch_k(ui_kernel<R, kUiWarps>, dim3(a.n), dim3(kUiWarps * 32), sm, s, a);
 }
 
-template <typename R, bool STAGED, bool CP>
-cudaError_t yi_occupancy(const YiGeometry& g, int* ctas) {
-  cudaError_t e = STAGED ? allow_smem(yi_kernel<R, STAGED, CP>, g.smem) : cudaSuccess;
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, yi_kernel<R, STAGED, CP>, g.threads, g.smem);
-}
-
-
-YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves) {
-  YiGeometry g;
-  g.nblk = (n + 31) / 32;
-  const size_t block = (size_t)2 * H * 32 * rsize;  // one staged [H][32] complex block
-  g.staged = block + 16 <= 200 * 1024;
-  g.conjplane = yi_conjplane(rsize, H);
-  g.smem = g.staged ? (g.conjplane ? 2 : 1) * block + 16 : 0;
-  g.threads = (g.smem > 100 * 1024) ? 1024 : (g.smem > 60 * 1024 ? 512 : 256);
-  // FP32 staged CTAs: a term-record ring per warp after the planes
-  if (g.staged && rsize == 4) g.smem += (size_t)(g.threads / 32) * kYRingLen * sizeof(YRec<float>);
-  int cps = 2048 / g.threads;
-  if (g.staged) cps = std::max(1, std::min(cps, (int)((227 * 1024) / g.smem)));
-  // the instance's real residency (registers can limit it further), queried
-  // once per (precision, H)
-  static std::mutex mu;
-  static std::map<std::pair<int, int>, int> occ_cache;
-  int occ = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = occ_cache.find({rsize, H});
-    if (it != occ_cache.end()) {
-      occ = it->second;
-    } else {
-      cudaError_t oe;
-      if (rsize == 4)
-        oe = g.staged ? (g.conjplane ? yi_occupancy<float, true, true>(g, &occ)
-                                     : yi_occupancy<float, true, false>(g, &occ))
-                      : yi_occupancy<float, false, false>(g, &occ);
-      else
-        oe = g.staged ? (g.conjplane ? yi_occupancy<double, true, true>(g, &occ)
-                                     : yi_occupancy<double, true, false>(g, &occ))
-                      : yi_occupancy<double, false, false>(g, &occ);
-      if (oe != cudaSuccess) {
-        cudaGetLastError();
-        occ = 0;
-      } else {
-        occ_cache[{rsize, H}] = occ;
-      }
-    }
-  }
-  if (occ > 0) cps = std::min(cps, occ);
-  // Split each CTA's outputs into ysplit CTAs.  CTAs of one launch take about
-  // equal time, so the launch lasts ceil(CTAs / resident) CTA lifetimes;
-  // pick the split that minimises
-  //   ceil(nblk ysplit / resident) (1 / ysplit + c),
-  // c = the fixed per-CTA cost (staging U) relative to a whole block's terms,
-  // taken as 0.02 / waves (the tunable: more waves, finer splits), and a
-  // tenth of that without staging.  Staged FP64 keeps its pipe busy all the
-  // time, so the CTAs an SM holds share it: there the count is the most CTAs
-  // an SM takes, ceil(nblk ysplit / SMs), instead of the waves (2J8, 2000
-  // atoms: 405 against 426 us).  Unstaged (2J14) it reads U through L1 and
-  // wants the warps of the finer split (11.06 against 9.33 ms by the SM count).
-  const long resident = (long)nsm * cps;
-  const long per = (rsize == 8 && g.staged) ? (long)nsm : resident;
-  const double c = (g.staged ? 0.02 : 0.002) / std::max(1, waves);
+// Split of each block's outputs into ysplit CTAs.  CTAs of one launch take
+// about equal time, so the launch lasts ceil(CTAs / per) CTA lifetimes; the
+// split minimises
+//   ceil(nblk ysplit / per) (1 / ysplit + c),
+// c = the fixed cost of a CTA (staging U) relative to a whole block's terms.
+static int yi_split(int nblk, long per, double c) {
   double best = 1e300;
-  g.ysplit = 1;
+  int split = 1;
   for (int ys = 1; ys <= 64; ++ys) {
-    const long w = ((long)g.nblk * ys + per - 1) / per;
+    const long w = ((long)nblk * ys + per - 1) / per;
     const double t = (double)w * (1.0 / ys + c);
     if (t < best - 1e-12) {
       best = t;
-      g.ysplit = ys;
+      split = ys;
     }
   }
-  g.nslices = g.ysplit * (g.threads / 32);
+  return split;
+}
+
+YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves, int ntasks) {
+  YiGeometry g;
+  g.nblk = rsize == 4 ? (n + 31) / 32 : (n + 15) / 16;
+  // The CTAs an SM holds share its pipes, so the launch lasts as long as the
+  // SM with the most CTAs.  c = 0.02 / waves (the tunable: more waves, finer
+  // splits).
+  const int warps = yc_warps(rsize, H <= half_size(9) ? 5 : 8);
+  g.threads = warps * 32;
+  g.smem = yc_smem(rsize, H, ntasks, warps);
+  g.split = yi_split(g.nblk, nsm, 0.02 / std::max(1, waves));
   return g;
+}
+
+template <typename K>
+cudaError_t launch_yq(K kq, const YiGeometry& g, const WorkArgs& a, cudaStream_t s) {
+  // persistent: as many CTAs as stay resident, (block, split) items from the queue
+  cudaError_t e = allow_smem(kq, g.smem);
+  if (e != cudaSuccess) return e;
+  int occ = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kq, g.threads, g.smem);
+  if (e != cudaSuccess) return e;
+  const long nitems = (long)g.nblk * g.split;
+  const long grid = std::min<long>(nitems, (long)a.nsm * std::max(1, occ));
+  return launch_k(kq, dim3((unsigned)grid), dim3(g.threads), g.smem, s, a, g.split);
+}
+
+template <class P, int LM>
+cudaError_t launch_yc(const YiGeometry& g, const WorkArgs& a, cudaStream_t s) {
+  if (a.persist & 1) return launch_yq(yc_kernel<P, LM, true>, g, a, s);
+  cudaError_t e = allow_smem(yc_kernel<P, LM, false>, g.smem);
+  if (e != cudaSuccess) return e;
+  return launch_k(yc_kernel<P, LM, false>, dim3((unsigned)(g.nblk * g.split)), dim3(g.threads), g.smem, s, a,
+                  g.split);
 }
 
 template <typename R>
@@ -1281,32 +1508,12 @@ cudaError_t launch_yi(const WorkArgs& a, cudaStream_t s) {
     return launch_k(yi_atom_kernel<R>, dim3((unsigned)((a.n + kYaWarps - 1) / kYaWarps)),
                     dim3(kYaWarps * 32), sm, s, a);
   }
-  const YiGeometry g = yi_geometry(sizeof(R), a.H, a.n, a.nsm, a.yi_waves);
-  if (g.nslices != a.nslices) return cudaErrorInvalidValue;
-  if ((a.persist & 1) && g.staged) {
-    // persistent: as many CTAs as stay resident, (block, split) items from the queue
-    auto kq = g.conjplane ? yi_queue_kernel<R, true> : yi_queue_kernel<R, false>;
-    cudaError_t e = allow_smem(kq, g.smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kq, g.threads, g.smem);
-    if (e != cudaSuccess) return e;
-    const long nitems = (long)g.nblk * g.ysplit;
-    const long grid = std::min<long>(nitems, (long)a.nsm * std::max(1, occ));
-    return launch_k(kq, dim3((unsigned)grid), dim3(g.threads), g.smem, s, a, g.ysplit);
-  }
-  dim3 grid(g.nblk, g.ysplit);
-  if (g.staged && g.conjplane) {
-    cudaError_t e = allow_smem(yi_kernel<R, true, true>, g.smem);
-    if (e != cudaSuccess) return e;
-    return launch_k(yi_kernel<R, true, true>, grid, dim3(g.threads), g.smem, s, a);
-  }
-  if (g.staged) {
-    cudaError_t e = allow_smem(yi_kernel<R, true, false>, g.smem);
-    if (e != cudaSuccess) return e;
-    return launch_k(yi_kernel<R, true, false>, grid, dim3(g.threads), g.smem, s, a);
-  }
-  return launch_k(yi_kernel<R, false, false>, grid, dim3(g.threads), 0, s, a);
+  const YiGeometry g = yi_geometry(sizeof(R), a.H, a.n, a.nsm, a.yi_waves, a.yc_ntask);
+  if (g.split != a.yc_split) return cudaErrorInvalidValue;
+  if constexpr (sizeof(R) == 4)
+    return a.twojmax <= 9 ? launch_yc<YcSingle<5>, 5>(g, a, s) : launch_yc<YcSingle<8>, 8>(g, a, s);
+  else
+    return a.twojmax <= 9 ? launch_yc<YcFixed<5>, 5>(g, a, s) : launch_yc<YcFixed<8>, 8>(g, a, s);
 }
 
 template <typename R>

@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <unordered_map>
 
@@ -139,7 +140,7 @@ void orient_by_cover(std::vector<unsigned>& terms, size_t first) {
 
 }  // namespace
 
-void HostTables::build(int J2, bool size_runs) {
+void HostTables::build(int J2) {
   twojmax = J2;
   H = half_size(J2);
   lmax = half_layer_size(J2);
@@ -203,7 +204,6 @@ void HostTables::build(int J2, bool size_runs) {
   term_cg.clear();
   term_trip.clear();
   term_out_first.clear();
-  term_runs.clear();
   auto half_elem = [&](int tt, int xa, int xb, int& idx, int& conj, double& sgn) {
     if (2 * xb <= tt) {
       idx = half_base(tt) + xb * (tt + 1) + xa;
@@ -291,15 +291,10 @@ void HostTables::build(int J2, bool size_runs) {
         // Group the output's terms by their first factor (index and
         // conjugation flag, stable): compute_Y then forms
         //   Y += U_t1[..] * sum_k coef_k U_t2,k[..]
-        // once per group.  Groups longer than kYGroupMax are cut into chunks,
-        // and with size_runs the chunks are ordered by length (stable), so an
-        // output is a run of 1-term groups, then of 2-term groups, ...;
-        // term_runs counts them.  Without it the groups keep the order of
-        // their first factor.  Bit 23 ends a group, bit 22 the output; every output has at
+        // once per group.  Bit 23 ends a group, bit 22 the output; every output has at
         // least one term: the term of the (t, 0, t) triple, whose
         // Clebsch-Gordan product is 1, or the zero term of a mirrored output.
         const size_t cnt = terms.size() - first;
-        std::array<unsigned short, kYGroupMax> runs{};
         if (cnt > 0) {
           std::vector<size_t> ord(cnt);
           for (size_t k = 0; k < cnt; ++k) ord[k] = k;
@@ -314,30 +309,14 @@ void HostTables::build(int J2, bool size_runs) {
             tq[k] = term_trip[first + ord[k]];
           }
           const unsigned kmask = 1023u | (1u << 20);
-          struct Chunk {
-            size_t b, n;
-          };
-          std::vector<Chunk> ch;
-          for (size_t k = 0; k < cnt;) {
-            size_t e = k + 1;
-            while (e < cnt && (tw[e] & kmask) == (tw[k] & kmask)) ++e;
-            for (size_t b = k; b < e; b += kYGroupMax) ch.push_back({b, std::min<size_t>(kYGroupMax, e - b)});
-            k = e;
-          }
-          if (size_runs)
-            std::stable_sort(ch.begin(), ch.end(), [](const Chunk& x, const Chunk& y) { return x.n < y.n; });
-          size_t pos = first;
-          for (const Chunk& c : ch) {
-            runs[c.n - 1] += 1;
-            for (size_t j = 0; j < c.n; ++j, ++pos) {
-              terms[pos] = tw[c.b + j] | (j + 1 == c.n ? (1u << 23) : 0u);
-              term_cg[pos] = tc[c.b + j];
-              term_trip[pos] = tq[c.b + j];
-            }
+          for (size_t k = 0; k < cnt; ++k) {
+            const bool end = k + 1 == cnt || (tw[k + 1] & kmask) != (tw[k] & kmask);
+            terms[first + k] = tw[k] | (end ? (1u << 23) : 0u);
+            term_cg[first + k] = tc[k];
+            term_trip[first + k] = tq[k];
           }
           terms.back() |= (1u << 22);
         }
-        term_runs.insert(term_runs.end(), runs.begin(), runs.end());
         term_out_first.push_back((int)first);
       }
   term_out_first.push_back((int)terms.size());
@@ -513,6 +492,240 @@ void HostTables::build(int J2, bool size_runs) {
     for (int q = 1; q < kRootDim; ++q) rootpq[p * kRootDim + q] = std::sqrt((double)p / (double)q);
 }
 
+void HostTables::build_classes(bool wide) {
+  yc_wide = wide;
+  const int J = twojmax, cw = wide ? 2 : 1;
+  // Output pairs of a task.  FP32: 4 where a block has hundreds of tasks (2J14,
+  // 2000 atoms: 387 us, with 2: 404), 2 where the largest would hold up the
+  // rest (2J8, 2000 atoms: 37 us, with 4: 43).
+  const int maxnp = wide ? 1 : J > 9 ? kYcOuts / 2 : 2;
+  // first slot of the vector of each stored m
+  std::vector<int> start((size_t)(2 * J + 1) * (J + 1), -1);
+  auto at = [&](int ma, int mb) -> int& { return start[(size_t)(ma + J) * (J + 1) - mb]; };  // mb <= 0
+  auto low = [](int ma, int mb) { return std::max(std::abs(ma), std::abs(mb)); };
+  yc_slot.assign(H, 0);
+  int n = 0;
+  for (int mb = -J; mb <= 0; ++mb)
+    for (int ma = -J; ma <= J; ++ma) {
+      if ((ma - mb) & 1) continue;
+      at(ma, mb) = n;
+      for (int t = low(ma, mb); t <= J; t += 2) yc_slot[half_base(t) + (mb + t) / 2 * (t + 1) + (ma + t) / 2] = n++;
+    }
+  std::vector<int> trip((size_t)(J + 1) * (J + 1) * (J + 1), -1);
+  for (int q = 0; q < (int)ztrip.size(); ++q)
+    trip[((size_t)ztrip[q].t1 * (J + 1) + ztrip[q].t2) * (J + 1) + ztrip[q].t] = q;
+  struct M {
+    int a, b;
+  };
+  // coefficient (without beta) of u_t1[m1] u_t2[m2] in Y_t of m1 + m2, and its triple
+  auto coef = [&](int t1, M m1, int t2, M m2, int t, int& q) {
+    const bool same = m1.a == m2.a && m1.b == m2.b;
+    q = -1;
+    if (t < std::abs(t1 - t2) || t > t1 + t2) return 0.0;
+    // a pair of equal m has each unordered (t1, t2) once; of different m, a
+    // triple with t1 = t2 has its two terms, equal ones, in one
+    if (same && t1 < t2) return 0.0;
+    double w = !same && t1 == t2 ? 2.0 : 1.0;
+    if (t1 < t2) {
+      std::swap(t1, t2);
+      std::swap(m1, m2);
+    }
+    q = trip[((size_t)t1 * (J + 1) + t2) * (J + 1) + t];
+    const ZTrip& z = ztrip[q];
+    auto c = [&](int x, int y) { return cg[z.cg_off + (x + t1) / 2 * (t2 + 1) + (y + t2) / 2]; };
+    w *= c(m1.a, m2.a) * c(m1.b, m2.b);
+    // mirrored vectors: (-1)^(ma + mb), ma + mb = (m_a + m_b) / 2 + t
+    if (m1.b > 0 && (((m1.a + m1.b) / 2 + t1) & 1)) w = -w;
+    if (m2.b > 0 && (((m2.a + m2.b) / 2 + t2) & 1)) w = -w;
+    return w;
+  };
+  auto place = [&](M m) {  // byte offset of its vector's [32] complex float, bit 31: conjugate
+    return m.b > 0 ? (unsigned)at(-m.a, -m.b) * 256u | 0x80000000u : (unsigned)at(m.a, m.b) * 256u;
+  };
+  yc_task.clear();
+  yc_trip.clear();
+  yc_head.clear();
+  yc_cg.clear();
+  yc_cost.clear();
+  struct Item {
+    M m1, m2;  // u[m2] the longer one
+    int l1, l2;
+  };
+  std::vector<Item> items;
+  for (int Mb = -J; Mb <= 0; ++Mb)
+    for (int Ma = -J; Ma <= (Mb < 0 ? J : 0); ++Ma) {
+      if ((Ma - Mb) & 1) continue;
+      items.clear();
+      for (int a1 = std::max(-J, Ma - J); a1 <= std::min(J, Ma + J); ++a1)
+        for (int b1 = std::max(-J, Mb - J); b1 <= std::min(J, Mb + J); ++b1) {
+          if ((a1 - b1) & 1) continue;
+          const M m1{a1, b1}, m2{Ma - a1, Mb - b1};
+          if (m2.a < m1.a || (m2.a == m1.a && m2.b < m1.b)) continue;
+          const int l1 = (J - low(m1.a, m1.b)) / 2 + 1, l2 = (J - low(m2.a, m2.b)) / 2 + 1;
+          items.push_back(l1 <= l2 ? Item{m1, m2, l1, l2} : Item{m2, m1, l2, l1});
+        }
+      std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) {
+        return x.l2 != y.l2 ? x.l2 > y.l2 : x.l1 > y.l1;
+      });
+      for (int tb = low(Ma, Mb); tb <= J; tb += 4 * maxnp) {
+        const int nout = std::min(2 * maxnp, (J - tb) / 2 + 1), np = (nout + 1) / 2;
+        // rows [r0, r1) of each item that have a coefficient, and its cost
+        struct Part {
+          int r0, r1;
+          long cost;
+        };
+        std::vector<Part> rows;
+        long total = 0;
+        for (const Item& it : items) {
+          const int lo1 = low(it.m1.a, it.m1.b), lo2 = low(it.m2.a, it.m2.b);
+          auto live = [&](int r) {
+            int q;
+            for (int k = 0; k < nout; ++k)
+              for (int c = 0; c < it.l2; ++c)
+                if (coef(lo1 + 2 * r, it.m1, lo2 + 2 * c, it.m2, tb + 2 * k, q) != 0.0) return true;
+            return false;
+          };
+          Part p{0, it.l1, 0};
+          while (p.r0 < p.r1 && !live(p.r0)) ++p.r0;
+          while (p.r1 > p.r0 && !live(p.r1 - 1)) --p.r1;
+          if (p.r1 > p.r0) p.cost = 30 + 4 * it.l2 + (long)(p.r1 - p.r0) * (8 + np * (4 * it.l2 + 8));
+          total += p.cost;
+          rows.push_back(p);
+        }
+        // two tasks of about equal cost, each with half of the pairs
+        size_t next = 0;
+        const int parts = total >= kYcWhole ? 2 : 1;
+        for (int part = 0; part < parts; ++part) {
+          const int task = (int)yc_cost.size();
+          std::vector<int> rec(kYcTask, -1);
+          rec[0] = (int)(yc_head.size() / kYcChunk);
+          rec[2] = nout;
+          rec[3] = parts == 1 ? 0 : 2 * (task - part) + 2 + part;
+          for (int k = 0; k < nout; ++k) {
+            const int t = tb + 2 * k, ma = (Ma + t) / 2, mb = (Mb + t) / 2, o = half_base(t) + mb * (t + 1) + ma;
+            rec[4 + k] = o;
+            if (Mb == 0 && Ma < 0) rec[4 + kYcOuts + k] = o + t - 2 * ma;
+          }
+          size_t pos = kYcChunk;  // words used of the open chunk
+          auto open = [&] {
+            yc_head.resize(yc_head.size() + kYcChunk, 0u);
+            yc_cg.resize(yc_head.size(), 0.0);
+            yc_trip.resize(yc_head.size(), -1);
+            unsigned* h = &yc_head[yc_head.size() - kYcChunk];
+            h[0] = (unsigned)task;
+            h[1] = (unsigned)np;
+            pos = 4;
+          };
+          open();
+          long cost = 200;
+          for (; next < items.size() && (part + 1 == parts || cost - 200 < total / 2); ++next) {
+            const Item& it = items[next];
+            const int lo1 = low(it.m1.a, it.m1.b), lo2 = low(it.m2.a, it.m2.b), l2p = (it.l2 + 1) & ~1;
+            const size_t row = (size_t)np * l2p * 2 * cw;
+            for (int r = rows[next].r0; r < rows[next].r1;) {
+              // four words are left at a chunk's end for the head that ends it
+              size_t fit = pos + 8 <= kYcChunk ? (kYcChunk - 8 - pos) / row : 0;
+              if (fit == 0) {
+                open();
+                fit = (kYcChunk - 8 - pos) / row;
+              }
+              const int n = (int)std::min<size_t>(fit, rows[next].r1 - r);
+              const size_t w0 = yc_head.size() - kYcChunk + pos;
+              yc_head[w0] = place(it.m1) + (unsigned)r * 256u;
+              yc_head[w0 + 1] = place(it.m2);
+              yc_head[w0 + 2] = (unsigned)n | (unsigned)it.l2 << 8;
+              for (size_t w = w0 + 4; w < w0 + 4 + n * row; w += row, ++r)
+                for (int o = 0; o < nout; ++o)
+                  for (int c = 0; c < it.l2; ++c) {
+                    const size_t x =
+                        wide ? w + ((size_t)o * l2p + c) * 2 : w + ((size_t)(o / 2) * l2p + c) * 2 + (o & 1);
+                    yc_cg[x] = coef(lo1 + 2 * r, it.m1, lo2 + 2 * c, it.m2, tb + 2 * o, yc_trip[x]);
+                  }
+              pos += 4 + n * row;
+            }
+            cost += rows[next].cost;
+          }
+          yc_head[yc_head.size() - kYcChunk] |= 0x80000000u;
+          rec[1] = (int)(yc_head.size() / kYcChunk) - rec[0];
+          yc_task.insert(yc_task.end(), rec.begin(), rec.end());
+          yc_cost.push_back(cost);
+        }
+      }
+    }
+}
+
+std::vector<unsigned> HostTables::yc_stream(const double* beta) const {
+  const std::vector<double> bw = beta_weights(beta);
+  std::vector<unsigned> w(yc_head);
+  for (size_t k = 0; k < w.size(); ++k) {
+    if (yc_trip[k] < 0) continue;
+    const float c = (float)(yc_cg[k] * bw[yc_trip[k]]);
+    std::memcpy(&w[k], &c, sizeof(c));
+  }
+  return w;
+}
+
+std::vector<unsigned> HostTables::yc_fixed(const double* beta) const {
+  const std::vector<double> bw = beta_weights(beta);
+  auto coef = [&](size_t x) { return yc_trip[x] < 0 ? 0.0 : yc_cg[x] * bw[yc_trip[x]]; };
+  std::vector<double> top(yc_cost.size() * kYcOuts, 0.0);  // largest sum over a record of each output
+  const unsigned* last[2] = {nullptr, nullptr};
+  double sum[2] = {0.0, 0.0};
+  yc_rows([&](int k, const unsigned* head, int, size_t w, int o, int len) {
+    if (last[o] != head) sum[o] = 0.0;
+    last[o] = head;
+    for (int c = 0; c < len; ++c) sum[o] += std::fabs(coef(w + 2 * c));
+    double& t = top[(size_t)k * kYcOuts + o];
+    if (!(sum[o] <= t)) t = sum[o];  // a NaN stays
+  });
+  std::vector<int> ex(top.size(), 0);  // top < 2^ex
+  for (size_t k = 0; k < top.size(); ++k) {
+    if (!std::isfinite(top[k])) ex[k] = kYcNan;
+    else if (top[k] > 0.0) std::frexp(top[k], &ex[k]);
+  }
+  std::vector<unsigned> w(yc_head);
+  for (size_t k = 0; k < yc_cost.size(); ++k)
+    for (int ch = yc_task[k * kYcTask]; ch < yc_task[k * kYcTask] + yc_task[k * kYcTask + 1]; ++ch)
+      for (int o = 0; o < 2; ++o) w[(size_t)ch * kYcChunk + 2 + o] = (unsigned)ex[k * kYcOuts + o];
+  yc_rows([&](int k, const unsigned*, int, size_t p, int o, int len) {
+    const int e = ex[(size_t)k * kYcOuts + o];
+    for (int c = 0; c < len; ++c) {
+      const long long v = e == kYcNan ? 0 : std::llrint(std::ldexp(coef(p + 2 * c), 60 - e));
+      const int hi = (int)((v + (1LL << 29)) >> 30);
+      w[p + 2 * c] = (unsigned)hi;
+      w[p + 2 * c + 1] = (unsigned)(int)(v - hi * (1LL << 30));
+    }
+  });
+  return w;
+}
+
+std::vector<int> HostTables::yc_bins(int nbins) const {
+  // units: a task, or the two halves of a sum (they meet in one CTA)
+  std::vector<std::array<int, 2>> unit;
+  auto cost = [&](const std::array<int, 2>& u) { return yc_cost[u[0]] + (u[1] < 0 ? 0 : yc_cost[u[1]]); };
+  for (int k = 0; k < (int)yc_cost.size(); ++k) {
+    const bool two = yc_task[(size_t)k * kYcTask + 3] != 0;
+    unit.push_back({k, two ? k + 1 : -1});
+    if (two) ++k;
+  }
+  std::stable_sort(unit.begin(), unit.end(), [&](const auto& x, const auto& y) { return cost(x) > cost(y); });
+  std::vector<std::vector<int>> bin(nbins);
+  std::vector<long> load(nbins, 0);
+  for (const auto& u : unit) {  // the next largest to the least loaded CTA
+    const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    bin[b].push_back(u[0]);
+    if (u[1] >= 0) bin[b].push_back(u[1]);
+    load[b] += cost(u);
+  }
+  std::vector<int> out(1, 0);
+  for (auto& b : bin) {
+    std::stable_sort(b.begin(), b.end(), [&](int x, int y) { return yc_cost[x] > yc_cost[y]; });
+    out.push_back(out.back() + (int)b.size());
+  }
+  for (const auto& b : bin) out.insert(out.end(), b.begin(), b.end());
+  return out;
+}
+
 std::vector<double> HostTables::beta_weights(const double* beta) const {
   std::vector<double> w(ztrip.size());
   for (size_t q = 0; q < ztrip.size(); ++q) w[q] = ztrip[q].fac * beta[1 + ztrip[q].bidx];
@@ -569,24 +782,6 @@ std::vector<int> HostTables::lane_outputs(int lanes, int* m) const {
   }
   *m = mm;
   return t;
-}
-
-std::vector<int> HostTables::slices(int nslices) const {
-  // nslices contiguous runs of output elements with about equal term counts;
-  // entry k is the first output of run k (entry nslices = H)
-  const long total = (long)terms.size();
-  std::vector<int> b(1, 0);
-  int k = 1;
-  for (int o = 0; o < H; ++o) {
-    const long done = term_out_first[o + 1];
-    if (k < nslices && done * nslices >= total * k) {
-      b.push_back(o + 1);
-      ++k;
-    }
-  }
-  while ((int)b.size() < nslices + 1) b.push_back(H);
-  b[nslices] = H;
-  return b;
 }
 
 std::vector<unsigned> HostTables::bwords(bool cp) const {

@@ -23,9 +23,6 @@ struct HostTables {
   std::vector<double> term_cg;
   std::vector<int> term_trip;
   std::vector<int> term_out_first;  // [H+1] first term of every output
-  // [H][kYGroupMax]: number of groups of 1, 2, ... kYGroupMax terms of each
-  // output (they follow one another in that order)
-  std::vector<unsigned short> term_runs;
   // bispectrum terms (records as above, coefficient without beta), the U
   // element of each output group, and the first term of each component
   std::vector<unsigned> bterms;
@@ -67,12 +64,70 @@ struct HostTables {
   std::vector<unsigned> pair_idx;
   std::vector<double> pair_norm, pair_weight, pair_ab;
 
-  // size_runs: order each output's term groups by length (the run layout of
-  // the FP32 compute_Y); otherwise by first factor
-  void build(int twojmax, bool size_runs = true);
+  // compute_Y of the mixed path (yc_kernel, snap_kernels.cu).  With m = (2 ma -
+  // t, 2 mb - t) the doubled projections of an element, the elements of every
+  // rank t with one m are its vector u[m]; the outputs with one M are a class,
+  // and its Y is a sum over the unordered pairs m1 + m2 = M of bilinear forms
+  //   Y_t[M] += sum_t1 u_t1[m1] sum_t2 c[t][t1][t2] u_t2[m2].
+  // yc_slot: [H] position of each half-layout element when the vectors are
+  //   stored one after the other, t rising (a vector with m_b > 0 is the mirror
+  //   of a stored one: conjugated, its sign folded into c);
+  // yc_task: [ntask][kYcTask] first chunk, chunks, outputs, half, the output
+  //   elements (up to kYcOuts), and the element each zeroes (the mirror below
+  //   the centre of the middle column) or -1; a task has outputs of one class,
+  //   at most kYcOuts (wide: 2) of them, and all pairs m1 + m2 = M (half = 0) or
+  //   half of them (two tasks k, k + 1 with half = 2 k + 2 and 2 k + 3);
+  // the stream, kYcChunk words a chunk: word 0 the task (bit 31: its last
+  //   chunk), word 1 the output pairs np of the task, words 2-3 zero, then
+  //   records: a head {byte offset of u[m1] (bit 31: conjugate), the same of
+  //   u[m2], rows | length of u[m2] << 8, 0} and per row (t1) np x (length
+  //   rounded up to even) coefficient pairs (outputs 2k, 2k + 1); a head with
+  //   no rows ends the chunk.  yc_head holds the words that are not
+  //   coefficients, yc_cg / yc_trip the coefficients without beta and their
+  //   triples (-1: not one);
+  // yc_cost: about the instructions of each task.
+  // wide (the FP64 path): a coefficient is two words (yc_cg / yc_trip at the
+  // first), a row 2 outputs x (length rounded up to even), np = 1, and words
+  // 2-3 of a chunk are the exponents of its task's outputs (yc_fixed).
+  std::vector<int> yc_slot, yc_task, yc_trip;
+  std::vector<unsigned> yc_head;
+  std::vector<double> yc_cg;
+  std::vector<long> yc_cost;
+  bool yc_wide = false;
+  void build_classes(bool wide);
+  // f(task, word, output, rows' elements) over every row of every output: the
+  // coefficient of element c is at word + c * stride
+  template <typename F>
+  void yc_rows(F&& f) const {
+    const int cw = yc_wide ? 2 : 1;
+    for (size_t k = 0; k < yc_cost.size(); ++k) {
+      const int* rec = &yc_task[k * kYcTask];
+      for (int ch = rec[0]; ch < rec[0] + rec[1]; ++ch) {
+        const size_t base = (size_t)ch * kYcChunk;
+        const int np = (int)yc_head[base + 1];
+        for (size_t p = base + 4; (yc_head[p + 2] & 255u) != 0;) {
+          const unsigned* head = &yc_head[p];
+          const int len = (int)(head[2] >> 8), lp = (len + 1) & ~1;
+          p += 4;
+          for (int r = 0; r < (int)(head[2] & 255u); ++r, p += (size_t)np * lp * 2 * cw)
+            for (int o = 0; o < 2 * np; ++o)
+              f((int)k, head, r, yc_wide ? p + (size_t)o * lp * 2 : p + (size_t)(o / 2) * lp * 2 + (o & 1), o, len);
+        }
+      }
+    }
+  }
+  // The stream's words with the coefficients of beta: FP32, or (wide) in 60-bit
+  // fixed point scaled by the power of two above each output's largest sum of
+  // their sizes over a record (kYcNan: not finite, the output is not a number).
+  std::vector<unsigned> yc_stream(const double* beta) const;
+  std::vector<unsigned> yc_fixed(const double* beta) const;
+  // The tasks dealt to nbins CTAs of about equal cost, decreasing in each:
+  // nbins + 1 offsets, then the tasks
+  std::vector<int> yc_bins(int nbins) const;
+
+  void build(int twojmax);
   std::vector<double> beta_weights(const double* beta) const;
   std::vector<double> term_coef(const double* beta) const;
-  std::vector<int> slices(int nslices) const;
   // outputs dealt to `lanes` lanes in decreasing term count, snake order:
   // [lanes][m] output indices, -1 past a lane's last; m returned in *m
   std::vector<int> lane_outputs(int lanes, int* m) const;
