@@ -77,11 +77,12 @@ struct snap_ctx {
   };
   std::map<int, BPart> bpart_cache;
   int nbparts = 0;
-  void* d_root = nullptr;
   void* d_hscale = nullptr;
   unsigned* d_pair_idx = nullptr;  // closed form of u (HostTables::pair_*)
   void* d_pair_scale = nullptr;
+  void* d_pair_norm = nullptr;
   void* d_pair_ab = nullptr;
+  int* d_u_units = nullptr;
   int* d_yc_bins = nullptr;
   int* d_ysched = nullptr;  // lane schedule of the warp-per-atom compute_Y
   int ysched_m = 0;
@@ -517,12 +518,41 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
     a.bmaxchunks = bp.maxchunks;
     a.bmaxterms = bp.maxterms;
   }
-  a.rootpq = c->d_root;
   a.hscale = c->d_hscale;
   a.pair_idx = c->d_pair_idx;
   a.pair_scale = c->d_pair_scale;
+  a.pair_norm = c->d_pair_norm;
   a.pair_ab = c->d_pair_ab;
+  a.npair_steps = (int)c->tab.pair_idx.size();
+  a.u_units = c->d_u_units;
+  a.u_nunits = c->tab.u_nunits;
+  a.u_nfine = (int)c->tab.u_units.size() / snap::kUUnit - c->tab.u_nunits;
+  a.u_cost = c->tab.u_cost;
   return a;
+}
+
+// FP32 up to 2J = 9 runs compute_U by the layer recursion, fused with the
+// neighbour build: one launch less, and the closed form gains little there.
+// Neighbour build and compute_U, layers / closed form: 2J8 2000 atoms 36 / 40 us,
+// 16000 atoms 183 / 192; 2J6 1024 atoms 20 / 30; above, 2J11 57 / 50, 2J14 86 / 57.
+bool u_by_layers(const snap_ctx* c) {
+  return c->precision == SNAP_MIXED && c->twojmax >= 1 && c->twojmax <= snap::kUColMax;
+}
+
+// The neighbour build with the slots' geometry, and compute_U; the launches
+// are added to *launches.
+int launch_neigh_and_u(snap_ctx* c, const snap::NeighArgs& na, const snap::WorkArgs& a, int ncta, cudaStream_t s,
+                       int* launches) {
+  if (u_by_layers(c)) {
+    SNAP_CUDA(c, snap::launch_neigh_u(na, a, ncta, s));
+    *launches += 1;
+    return SNAP_OK;
+  }
+  const bool mixed = c->precision == SNAP_MIXED;
+  SNAP_CUDA(c, mixed ? snap::launch_neigh_geom<float>(na, a, ncta, s) : snap::launch_neigh_geom<double>(na, a, ncta, s));
+  SNAP_CUDA(c, mixed ? snap::launch_u<float>(a, s) : snap::launch_u<double>(a, s));
+  *launches += 2;
+  return SNAP_OK;
 }
 
 // Enqueue the whole evaluation on stream s (no synchronisation).
@@ -569,20 +599,14 @@ int enqueue(snap_ctx* c, int n, const double* pos, const double* box, const int*
   a.virial = virial;
   a.B = B;
   const bool mixed = c->precision == SNAP_MIXED;
-  // register column-chain kernels: FP32 for 2J >= 1; FP64 up to 2J = 8 (above,
-  // the FP64 columns need all 255 registers and the occupancy loss costs more
-  // than the layout gains: fused dE 6.1 vs 4.6 ms at 2J = 14, 2000 atoms)
-  const bool colk = c->twojmax >= 1 && (mixed || c->twojmax <= 8);
-  auto launch_u = [&]() -> cudaError_t {
-    return colk ? (mixed ? snap::launch_ui_col<float>(a, s) : snap::launch_ui_col<double>(a, s))
-                : (mixed ? snap::launch_ui<float>(a, s) : snap::launch_ui<double>(a, s));
-  };
   if (user) {
-    SNAP_CUDA(c, snap::launch_neigh_ingest(n, K, pos, box[0], box[1], box[2], ucnt, uidx, uimg, ucap,
-                                           c->d_cnt, c->d_nbr, c->d_img, c->d_rij, c->d_key, c->d_flags, s));
+    SNAP_CUDA(c, (mixed ? snap::launch_neigh_ingest<float> : snap::launch_neigh_ingest<double>)(
+                     a, !u_by_layers(c), pos, box[0], box[1], box[2], ucnt, uidx, uimg, ucap, c->d_cnt, c->d_nbr,
+                     c->d_img, c->d_rij, c->d_key, c->d_flags, s));
     c->launches += 1;
     SNAP_CUDA(c, mark());
-    SNAP_CUDA(c, launch_u());
+    if (u_by_layers(c)) SNAP_CUDA(c, snap::launch_ui_col(a, s));
+    else SNAP_CUDA(c, mixed ? snap::launch_u<float>(a, s) : snap::launch_u<double>(a, s));
     c->launches += 1;
   } else {
     snap::NeighArgs na;
@@ -611,15 +635,8 @@ int enqueue(snap_ctx* c, int n, const double* pos, const double* box, const int*
     if (pos_stage) na.pos = pos_stage;
     c->launches += 1;
     SNAP_CUDA(c, mark());
-    if (colk) {
-      // the neighbour build fused with compute_U
-      SNAP_CUDA(c, mixed ? snap::launch_neigh_u<float>(na, a, 0, s) : snap::launch_neigh_u<double>(na, a, 0, s));
-      c->launches += 1;
-    } else {
-      SNAP_CUDA(c, snap::launch_neigh_build(na, s));
-      SNAP_CUDA(c, launch_u());
-      c->launches += 2;
-    }
+    rc = launch_neigh_and_u(c, na, a, 0, s, &c->launches);
+    if (rc) return rc;
   }
   SNAP_CUDA(c, mark());
   c->generation += 1;
@@ -745,18 +762,10 @@ int launch_batch(snap_ctx* c, const double* pos, double* energy, double* forces,
   a.virial = virial;
   a.vatom = c->d_vatom;
   const bool mixed = c->precision == SNAP_MIXED;
-  const bool colk = c->twojmax >= 1 && (mixed || c->twojmax <= 8);
   SNAP_CUDA(c, snap::launch_pos4(n, pos, c->d_pos4, s));
   int nl = 1;
-  if (colk) {
-    SNAP_CUDA(c, mixed ? snap::launch_neigh_u<float>(na, a, c->bat_ncta, s)
-                       : snap::launch_neigh_u<double>(na, a, c->bat_ncta, s));
-    nl += 1;
-  } else {
-    SNAP_CUDA(c, snap::launch_neigh_build_batch(na, c->bat_ncta, s));
-    SNAP_CUDA(c, mixed ? snap::launch_ui<float>(a, s) : snap::launch_ui<double>(a, s));
-    nl += 2;
-  }
+  const int rc = launch_neigh_and_u(c, na, a, c->bat_ncta, s, &nl);
+  if (rc) return rc;
   SNAP_CUDA(c, mixed ? snap::launch_yi<float>(a, s) : snap::launch_yi<double>(a, s));
   SNAP_CUDA(c, mixed ? snap::launch_de<float>(a, s) : snap::launch_de<double>(a, s));
   a.hflags = c->d_hflags;  // the force kernel ends the evaluation (the virial sums use no flag)
@@ -794,18 +803,10 @@ int launch_batch_deriv(snap_ctx* c, const double* pos, const double* g, double* 
   na.flags = c->d_flags;
   snap::WorkArgs a = make_args(c, n, c->K);
   const bool mixed = c->precision == SNAP_MIXED;
-  const bool colk = c->twojmax >= 1 && (mixed || c->twojmax <= 8);
   SNAP_CUDA(c, snap::launch_pos4(n, pos, c->d_pos4, s));
   int nl = 1;
-  if (colk) {
-    SNAP_CUDA(c, mixed ? snap::launch_neigh_u<float>(na, a, c->bat_ncta, s)
-                       : snap::launch_neigh_u<double>(na, a, c->bat_ncta, s));
-    nl += 1;
-  } else {
-    SNAP_CUDA(c, snap::launch_neigh_build_batch(na, c->bat_ncta, s));
-    SNAP_CUDA(c, mixed ? snap::launch_ui<float>(a, s) : snap::launch_ui<double>(a, s));
-    nl += 2;
-  }
+  const int rc = launch_neigh_and_u(c, na, a, c->bat_ncta, s, &nl);
+  if (rc) return rc;
   SNAP_CUDA(c, mixed ? snap::launch_tan_col<float>(a, g, c->d_dU, s) : snap::launch_tan_col<double>(a, g, c->d_dU, s));
   SNAP_CUDA(c, mixed ? snap::launch_dbi<float>(a, c->d_dU, dB, s) : snap::launch_dbi<double>(a, c->d_dU, dB, s));
   SNAP_CUDA(c, close_flags(c, s));
@@ -1148,7 +1149,6 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
   if (!rc) rc = upload(c, &c->d_yc_slot, c->tab.yc_slot);
   if (!rc) rc = upload(c, &c->d_yc_task, c->tab.yc_task);
   if (!rc) rc = upload(c, &c->d_ysched, c->tab.lane_outputs(32, &c->ysched_m));
-  if (!rc) rc = upload_r(c, &c->d_root, c->tab.rootpq);
   if (!rc) rc = upload_r(c, &c->d_hscale, c->tab.half_scale);
   if (!rc) rc = upload(c, &c->d_pair_idx, c->tab.pair_idx);
   if (!rc) {
@@ -1156,7 +1156,9 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
     for (size_t k = 0; k < w.size(); ++k) w[k] *= c->tab.pair_weight[k];
     rc = upload_r(c, &c->d_pair_scale, w);
   }
+  if (!rc) rc = upload_r(c, &c->d_pair_norm, c->tab.pair_norm);
   if (!rc) rc = upload_r(c, &c->d_pair_ab, c->tab.pair_ab);
+  if (!rc) rc = upload(c, &c->d_u_units, c->tab.u_units);
   if (!rc) rc = upload_yrec(c);
   if (!rc) rc = upload_brec(c);
   if (!rc) rc = upload(c, &c->d_bchunk_term, c->tab.bchunk_term);
@@ -1745,11 +1747,12 @@ int snap_destroy(snap_ctx* c) {
   dfree(c->d_bcomp_chunk);
   for (auto& kv : c->bpart_cache) cudaFree(kv.second.d);
   c->bpart_cache.clear();
-  dfree(c->d_root);
   dfree(c->d_hscale);
   dfree(c->d_pair_idx);
   dfree(c->d_pair_scale);
+  dfree(c->d_pair_norm);
   dfree(c->d_pair_ab);
+  dfree(c->d_u_units);
   for (auto& kv : c->yc_bins_cache) cudaFree(kv.second);
   c->yc_bins_cache.clear();
   c->d_yc_bins = nullptr;

@@ -62,26 +62,6 @@ struct Shape {
   static constexpr int P = 32 / NC;
 };
 
-// Replace column mc = t/2 (on the lane with mb == mc) by the mirror of the
-// column held one lane below, for layer t-1 (length t).
-template <typename R, int T, int N>
-__device__ __forceinline__ void seed_column(c2<R> (&v)[N], bool take) {
-  constexpr int mc = T / 2;
-  c2<R> src[T];
-#pragma unroll
-  for (int k = 0; k < T; ++k) {
-    src[k].re = shfl_up(v[k].re);
-    src[k].im = shfl_up(v[k].im);
-  }
-  if (take) {
-#pragma unroll
-    for (int m = 0; m < T; ++m) {
-      const R s = (((T - 1 - m) + (mc - 1)) & 1) ? R(-1) : R(1);
-      v[m] = mk<R>(s * src[T - 1 - m].re, -s * src[T - 1 - m].im);
-    }
-  }
-}
-
 // ------------------------------------------- scaled layer recursion
 // With u_t[ma][mb] = S_t(ma, mb) v_t[ma][mb], S_t(ma, mb) =
 // sqrt((t - ma)! ma! / (t - mb)!), the recursion of Eq. (hysphrecur) becomes
@@ -148,18 +128,6 @@ __device__ __forceinline__ void v_seed(c2<R> (&v)[N], bool take) {
       const R sq = (((T - 1 - m) + (mc - 1)) & 1) ? -q : q;
       v[m] = mk<R>(sq * src[T - 1 - m].re, -sq * src[T - 1 - m].im);
     }
-  }
-}
-
-// 1 / sqrt((t - mb)!) for t = 0..J2 (0 below mb), once per warp.
-template <typename R, int J2>
-__device__ __forceinline__ void v_gscale(R (&gs)[J2 + 1], int mb) {
-  R f = R(1);
-  const R mbr = R(mb);
-#pragma unroll
-  for (int t = 0; t <= J2; ++t) {
-    if (t > mb) f *= R(t) - mbr;
-    gs[t] = (t >= mb) ? R(1) / sqrt(f) : R(0);
   }
 }
 

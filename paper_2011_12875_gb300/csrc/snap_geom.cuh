@@ -1,6 +1,6 @@
 // snap_geom.cuh -- per-slot Cayley-Klein geometry (computed where the
-// slot's separation is at hand: the fused neighbour build, or the compute_U
-// kernels for caller-supplied lists) and the reverse-slot search.
+// slot's separation is at hand: the neighbour build, or the first kernel that
+// reads a caller-supplied list) and the reverse-slot search.
 //
 // Geometry of a slot (Sec. II-A: the neighbour vector mapped to the
 // 3-sphere, with constants from the paper's SNAP reference):
@@ -29,8 +29,8 @@ namespace geo {
 
 // Geometry of slot q into geom[q][0..kGeomStride): a (2), b (2), f_c,
 // grad f_c (3), da/dr_d (3 x 2), db/dr_d (3 x 2).
-// With `abf` given, a (2), b (2) and f_c are also written there (the
-// compute_U kernel keeps its atom's in shared memory).
+// With `abf` given, a (2), b (2) and f_c are also written there (the fused
+// neighbour build and compute_U keep their atoms' in shared memory).
 //
 // FP64 work is kept to what the Cayley-Klein parameters need: r, theta0,
 // sin/cos theta0, a and b.  In the mixed path (G = float) everything else --
@@ -190,13 +190,6 @@ __device__ __forceinline__ int find_rev_key(const WorkArgs& a, int i, long q, in
     if (found >= 0) break;
   }
   return found;
-}
-
-// Geometry of atom i's slots s = first, first + stride, ...
-template <typename G>
-__device__ void atom_geom(const WorkArgs& a, int i, int first, int stride) {
-  const int cnt = a.cnt[i];
-  for (int s = first; s < cnt; s += stride) slot_geom<G>(a, (long)i * a.K + s);
 }
 
 }  // namespace geo

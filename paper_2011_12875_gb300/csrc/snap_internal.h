@@ -24,12 +24,12 @@ constexpr int kYcChunk = 256;  // words of a compute_Y stream chunk (snap_tables
 constexpr int kYcOuts = 8;     // most outputs of a compute_Y task
 constexpr int kYcTask = 4 + 2 * kYcOuts;
 constexpr long kYcWhole = 1000;  // cost from which a task's sum is split in two
+constexpr int kUUnit = 8;  // words of a compute_U unit (HostTables::u_units)
 constexpr int kYcNan = 0x7FFF;  // exponent of an output whose coefficients are not finite
 constexpr int kBChunk = 96;    // bispectrum terms a warp takes at a time (whole groups)
 constexpr int kBMaxChunks = 1024;  // chunks are lengthened past this count
 constexpr int kBGroupMax = 8;      // longest bispectrum term piece (longer groups are cut)
 constexpr int kMaxNeighCap = 64;
-constexpr int kRootDim = 16;     // rootpq table is kRootDim x kRootDim
 constexpr int kGeomStride = 20;  // doubles per neighbour slot, see PairGeom
 
 // Half-matrix layout (Sec. V-A: u_j only needs floor(j)+1 of its columns):
@@ -203,28 +203,35 @@ struct WorkArgs {
   const int* bpart;         // [nbparts+1] first component of each CTA's run
   int nbparts, bmaxchunks, bmaxterms;  // runs, most chunks and most terms of one run
   double* B;              // [N][ncoeff]
-  const void* rootpq;
   const void* hscale;  // R [H]: S_t(ma, mb) of the scaled recursion (u = S v)
   // closed-form u of a pair (snap_pairs.cuh, HostTables::pair_*), per step
   const unsigned* pair_idx;
-  const void* pair_scale;  // R
+  const void* pair_scale;  // R: norm x weight
+  const void* pair_norm;   // R
   const void* pair_ab;     // R x 2
+  int npair_steps;
+  // compute_U's units, [u_nunits + u_nfine][kUUnit] (HostTables::u_units)
+  const int* u_units;
+  int u_nunits, u_nfine, u_cost;
 };
 
 // Launchers (snap_neigh.cu)
 cudaError_t launch_pos4(int n, const double* pos, float4* pos4, cudaStream_t s, float4* tiles = nullptr,
                         double* copy = nullptr);
 cudaError_t launch_neigh_build(const NeighArgs& a, cudaStream_t s);
-// batch: one launch over all configurations (ncta CTAs)
-cudaError_t launch_neigh_build_batch(const NeighArgs& a, int ncta, cudaStream_t s);
-cudaError_t launch_neigh_ingest(int n, int K, const double* pos, double Lx, double Ly,
-                                double Lz, const int* ucnt, const int* uidx,
-                                const signed char* uimg, int ucap, int* cnt, int* nbr,
+// Caller-supplied list to the internal tables, with (geom) the slots' geometry.
+template <typename R>
+cudaError_t launch_neigh_ingest(const WorkArgs& a, bool geom, const double* pos, double Lx, double Ly, double Lz,
+                                const int* ucnt, const int* uidx, const signed char* uimg, int ucap, int* cnt, int* nbr,
                                 signed char* img, double* rij, int* key, int* flags, cudaStream_t s);
-// reverse-slot map + geometry in the working precision G (one kernel)
+
+// Launchers (snap_u.cu): the neighbour build with the slots' geometry, one
+// configuration (ncta = 0) or a batch of ncta CTAs (na.confs); compute_U.
+template <typename R>
+cudaError_t launch_neigh_geom(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s);
+template <typename R> cudaError_t launch_u(const WorkArgs& a, cudaStream_t s);
 
 // Launchers (snap_kernels.cu), R = float (mixed) or double (FP64)
-template <typename R> cudaError_t launch_ui(const WorkArgs& a, cudaStream_t s);
 template <typename R> cudaError_t launch_yi(const WorkArgs& a, cudaStream_t s);
 
 // Launch shape of compute_Y for N atoms: nblk blocks of atoms x split CTAs of
@@ -267,12 +274,11 @@ BiPlan bi_plan(int rsize, int H, bool deriv, int maxchunks, int maxterms, int la
 // whether the conjugate-plane records can ever be used for this size and H
 bool bi_plane_fits(int rsize, int H);
 
-// Register column-chain kernels (snap_col_*.cu), for 1 <= twojmax <= 14;
-// cudaErrorInvalidValue when no instance exists for the precision/2J.
-template <typename R> cudaError_t launch_ui_col(const WorkArgs& a, cudaStream_t s);
-// Neighbour build fused with compute_U (FP32: 1 <= twojmax <= 14; FP64: up
-// to 8): one configuration (ncta = 0) or a batch of ncta CTAs (na.confs).
-template <typename R>
+// FP32 compute_U by the layer recursion (snap_col_f32.cu), 1 <= 2J <= kUColMax:
+// for caller lists, and fused with the neighbour build, one configuration
+// (ncta = 0) or a batch.
+constexpr int kUColMax = 9;
+cudaError_t launch_ui_col(const WorkArgs& a, cudaStream_t s);
 cudaError_t launch_neigh_u(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s);
 // Tangent of Ulisttot along the displacement field g ([N][3], device); 0..14.
 template <typename R>

@@ -67,118 +67,6 @@ __device__ __forceinline__ int half_weight(int t, int ma, int mb) {
   return ma < mb ? 2 : (ma == mb ? 1 : 0);
 }
 
-// Element (m, mb) of layer tp (= t - 1) stored in half layout at `lay`; the
-// column mb = (tp+1)/2 past the stored half comes from the inversion symmetry
-// u[m][mb] = (-1)^(m+mb) conj(u[tp-m][tp-mb]).
-template <typename R>
-__device__ __forceinline__ cx<R> prev_elem(const cx<R>* lay, int tp, int m, int mb) {
-  if (2 * mb <= tp) return lay[mb * (tp + 1) + m];
-  const cx<R> v = lay[(tp - mb) * (tp + 1) + (tp - m)];
-  const R s = ((m + mb) & 1) ? R(-1) : R(1);
-  return mk<R>(s * v.re, -s * v.im);
-}
-
-// The same in the scaled form v = u / S_t(ma, mb) (S_t = sqrt((t-ma)! ma! /
-// (t-mb)!)): the mirrored element of the new middle column mb = (tp+1)/2
-// also picks up S's ratio between the two columns, 1 / sqrt(mb) (qm).
-template <typename R>
-__device__ __forceinline__ cx<R> prev_elem_v(const cx<R>* lay, int tp, int m, int mb, R qm) {
-  if (2 * mb <= tp) return lay[mb * (tp + 1) + m];
-  const cx<R> v = lay[(tp - mb) * (tp + 1) + (tp - m)];
-  const R s = ((m + mb) & 1) ? -qm : qm;
-  return mk<R>(s * v.re, -s * v.im);
-}
-
-// ------------------------------------------------------------- compute_U
-// First the atom's slot geometry (snap_geom.cuh), then the recursion.  One
-// CTA per atom i, one warp per neighbour pair (lanes over the elements of
-// a layer), NW warps per CTA.  u_t of a pair follows the layer recursion
-// (Eq. hysphrecur): for mb <= t/2,
-//   u_t[ma][mb] = sqrt((t-ma)/(t-mb)) conj(a) u_{t-1}[ma][mb]
-//               - sqrt(ma/(t-mb))     conj(b) u_{t-1}[ma-1][mb],
-// with only the previous layer kept (double buffer, shared memory), run in the
-// scaled form u = S v, v_t[ma] = conj(a) v_{t-1}[ma] - conj(b) v_{t-1}[ma-1]
-// (S absorbs both root factors; a multiply and three fused multiply-adds a
-// component, with S_t(ma, mb) = sqrt((t-ma)! ma! / (t-mb)!)).  f_c v
-// is summed per warp in shared memory, the warps are summed in a fixed order,
-// multiplied by S once, and w_self is added on the diagonal (Eq. u).
-template <typename R, int NW>
-__global__ void __launch_bounds__(NW * 32) ui_kernel(WorkArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int H = a.H, L = a.lmax, J2 = a.twojmax;
-  R* root = reinterpret_cast<R*>(smem);
-  cx<R>* acc = reinterpret_cast<cx<R>*>(root + kRootDim * kRootDim);
-  cx<R>* buf = acc + NW * H;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x;
-  const R* rootg = reinterpret_cast<const R*>(a.rootpq);
-  for (int e = threadIdx.x; e < kRootDim * kRootDim; e += blockDim.x) root[e] = rootg[e];
-  for (int e = threadIdx.x; e < NW * H; e += blockDim.x) acc[e] = mk<R>(0, 0);
-  // the atom's slot geometry (snap_geom.cuh)
-  geo::atom_geom<R>(a, i, threadIdx.x, blockDim.x);
-  __syncthreads();
-  cx<R>* myacc = acc + warp * H;
-  cx<R>* b0 = buf + warp * 2 * L;
-  cx<R>* b1 = b0 + L;
-  const int cnt = a.cnt[i];
-  for (int s = warp; s < cnt; s += NW) {
-    const R* g = reinterpret_cast<const R*>(a.geom) + ((long)i * a.K + s) * kGeomStride;
-    const cx<R> ca = mk<R>(g[0], g[1]);
-    const cx<R> cb = mk<R>(g[2], g[3]);
-    const R fc = g[4];
-    cx<R>* cur = b0;
-    cx<R>* nxt = b1;
-    if (lane == 0) {
-      cur[0] = mk<R>(1, 0);
-      myacc[0].re += fc;
-    }
-    __syncwarp();
-    for (int t = 1; t <= J2; ++t) {
-      const int size = half_layer_size(t), hb = half_base(t);
-      const R qm = (t & 1) ? R(0) : root[kRootDim + t / 2];  // 1 / sqrt(t/2): the mirror's ratio
-      for (int e = lane; e < size; e += 32) {
-        const int mb = e / (t + 1), ma = e - mb * (t + 1);
-        cx<R> v = mk<R>(0, 0);
-        if (ma < t) {  // + conj(a) v_{t-1}[ma]
-          const cx<R> p = prev_elem_v(cur, t - 1, ma, mb, qm);
-          v.re = fmr(ca.im, p.im, ca.re * p.re);
-          v.im = fmr(-ca.im, p.re, ca.re * p.im);
-        }
-        if (ma > 0) {  // - conj(b) v_{t-1}[ma-1]
-          const cx<R> p = prev_elem_v(cur, t - 1, ma - 1, mb, qm);
-          v.re = fmr(-cb.im, p.im, fmr(-cb.re, p.re, v.re));
-          v.im = fmr(cb.im, p.re, fmr(-cb.re, p.im, v.im));
-        }
-        nxt[e] = v;
-        myacc[hb + e].re = fmr(fc, v.re, myacc[hb + e].re);
-        myacc[hb + e].im = fmr(fc, v.im, myacc[hb + e].im);
-      }
-      __syncwarp();
-      cx<R>* tmp = cur;
-      cur = nxt;
-      nxt = tmp;
-    }
-    __syncwarp();
-  }
-  __syncthreads();
-  cx<R>* Ug = reinterpret_cast<cx<R>*>(a.U);
-  const long blk = i >> 5;
-  const int li = i & 31;
-  for (int e = threadIdx.x; e < H; e += blockDim.x) {
-    cx<R> s = acc[e];
-    for (int w = 1; w < NW; ++w) {
-      s.re += acc[w * H + e].re;
-      s.im += acc[w * H + e].im;
-    }
-    const R sc = reinterpret_cast<const R*>(a.hscale)[e];  // u = S v
-    s.re *= sc;
-    s.im *= sc;
-    const int p = a.half_tmm[e];
-    if (tmm_ma(p) == tmm_mb(p)) s.re += (R)a.wself;
-    Ug[(blk * H + e) * 32 + li] = s;
-  }
-}
-
 // ------------------------------------------- staging (bulk copies, waits)
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
@@ -1415,13 +1303,6 @@ __global__ void __launch_bounds__(kFThreads) force_kernel(WorkArgs a) {
   if (tid < 6) a.virial[tid] = (wv[0][tid] + wv[1][tid]) + (wv[2][tid] + wv[3][tid]);
 }
 
-constexpr int kUiWarps = 4;
-
-template <typename R>
-size_t ui_smem(int H, int L) {
-  return sizeof(R) * kRootDim * kRootDim + sizeof(cx<R>) * (size_t)kUiWarps * (H + 2 * L);
-}
-
 template <typename K>
 cudaError_t allow_smem(K kernel, size_t bytes) {
   // the default 48 KB limit covers static and dynamic shared memory together
@@ -1434,15 +1315,6 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
 
 }  // namespace
 
-
-template <typename R>
-cudaError_t launch_ui(const WorkArgs& a, cudaStream_t s) {
-  if (a.n <= 0) return cudaSuccess;
-  const size_t sm = ui_smem<R>(a.H, a.lmax);
-  cudaError_t e = allow_smem(ui_kernel<R, kUiWarps>, sm);
-  if (e != cudaSuccess) return e;
-  return launch_k(ui_kernel<R, kUiWarps>, dim3(a.n), dim3(kUiWarps * 32), sm, s, a);
-}
 
 // Split of each block's outputs into ysplit CTAs.  CTAs of one launch take
 // about equal time, so the launch lasts ceil(CTAs / per) CTA lifetimes; the
@@ -1637,8 +1509,6 @@ cudaError_t launch_virial_conf(const double* vatom, const NeighConf* confs, int 
   return launch_k(virial_conf_kernel, dim3(nconf), dim3(256), 0, s, vatom, confs, virial);
 }
 
-template cudaError_t launch_ui<float>(const WorkArgs&, cudaStream_t);
-template cudaError_t launch_ui<double>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_yi<float>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_yi<double>(const WorkArgs&, cudaStream_t);
 template cudaError_t launch_force<float>(const WorkArgs&, cudaStream_t);

@@ -9,20 +9,15 @@
 #include <math.h>
 
 #include "snap_internal.h"
+#include "snap_geom.cuh"
 #include "snap_neigh.cuh"
 
 namespace snap {
 
 namespace {
 
-constexpr int kNbWarps = 8;        // warps per CTA of the batch build
-constexpr int kNbWarpsSingle = 2;  // warps (= atoms) per CTA of a single configuration: small
-                                   // CTAs spread the one-warp atoms evenly over the SMs
-// Warps per centre atom: a batch build scans every block of its
-// configuration, so four warps share the scan; a single-configuration build
-// skips far tiles and one warp per atom suffices.
-constexpr int kNbSplitBatch = 4;
-static_assert(kNbWarps / kNbSplitBatch == kNeighAtomsPerCta, "batch CTA map and kernel disagree");
+constexpr int kNbWarpsSingle = 2;  // warps (= atoms) per CTA: small CTAs spread the one-warp atoms
+                                   // evenly over the SMs
 constexpr unsigned kFull = 0xffffffffu;
 
 // FP32 positions, (when `tiles` is given) the bounding box of every tile of
@@ -72,12 +67,16 @@ __global__ void __launch_bounds__(NW * 32) neigh_build_kernel(NeighArgs a) {
   nb::neigh_build_cta<BATCH, SPLIT, NW>(a, [](int, long, int, long, double, double, double) {});
 }
 
-// Caller-supplied list -> internal [N][K] tables with exact separations.
-__global__ void neigh_ingest_kernel(int n, int K, const double* __restrict__ pos, double Lx,
-                                    double Ly, double Lz, const int* __restrict__ ucnt,
-                                    const int* __restrict__ uidx, const signed char* __restrict__ uimg,
-                                    int ucap, int* cnt, int* nbr, signed char* img, double* rij,
-                                    int* key, int* flags) {
+// Caller-supplied list -> internal [N][K] tables with exact separations, and
+// (GEOM) the slots' geometry.
+template <typename G, bool GEOM>
+__global__ void __launch_bounds__(128) neigh_ingest_kernel(WorkArgs a, const double* __restrict__ pos, double Lx,
+                                                           double Ly, double Lz, const int* __restrict__ ucnt,
+                                                           const int* __restrict__ uidx,
+                                                           const signed char* __restrict__ uimg, int ucap, int* cnt,
+                                                           int* nbr, signed char* img, double* rij, int* key,
+                                                           int* flags) {
+  const int n = a.n, K = a.K;
   const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= (long)n * K) return;
   const int i = (int)(q / K), s = (int)(q - (long)i * K);
@@ -96,6 +95,7 @@ __global__ void neigh_ingest_kernel(int n, int K, const double* __restrict__ pos
     img[3 * q] = img[3 * q + 1] = img[3 * q + 2] = 0;
     rij[3 * q] = rij[3 * q + 1] = rij[3 * q + 2] = 1e30;  // beyond rcut: ignored
     key[q] = -1;
+    if (GEOM) geo::pair_geom<G>(a, q, 1e30, 1e30, 1e30);
     return;
   }
   const int ix = uimg[3 * u], iy = uimg[3 * u + 1], iz = uimg[3 * u + 2];
@@ -103,10 +103,14 @@ __global__ void neigh_ingest_kernel(int n, int K, const double* __restrict__ pos
   img[3 * q] = (signed char)ix;
   img[3 * q + 1] = (signed char)iy;
   img[3 * q + 2] = (signed char)iz;
-  rij[3 * q] = nb::sep1(i, k, pos[3 * i], pos[3 * k], ix, Lx);
-  rij[3 * q + 1] = nb::sep1(i, k, pos[3 * i + 1], pos[3 * k + 1], iy, Ly);
-  rij[3 * q + 2] = nb::sep1(i, k, pos[3 * i + 2], pos[3 * k + 2], iz, Lz);
+  const double x = nb::sep1(i, k, pos[3 * i], pos[3 * k], ix, Lx);
+  const double y = nb::sep1(i, k, pos[3 * i + 1], pos[3 * k + 1], iy, Ly);
+  const double z = nb::sep1(i, k, pos[3 * i + 2], pos[3 * k + 2], iz, Lz);
+  rij[3 * q] = x;
+  rij[3 * q + 1] = y;
+  rij[3 * q + 2] = z;
   key[q] = pair_key(k, ix, iy, iz, n);
+  if (GEOM) geo::pair_geom<G>(a, q, x, y, z);
 }
 
 inline int blocks_for(long n, int t) { return (int)((n + t - 1) / t); }
@@ -125,19 +129,20 @@ cudaError_t launch_neigh_build(const NeighArgs& a, cudaStream_t s) {
                   dim3(kNbWarpsSingle * 32), 0, s, a);
 }
 
-cudaError_t launch_neigh_build_batch(const NeighArgs& a, int ncta, cudaStream_t s) {
-  if (ncta <= 0) return cudaSuccess;
-  return launch_k(neigh_build_kernel<true, kNbSplitBatch, kNbWarps>, dim3(ncta), dim3(kNbWarps * 32), 0, s, a);
-}
-
-cudaError_t launch_neigh_ingest(int n, int K, const double* pos, double Lx, double Ly,
-                                double Lz, const int* ucnt, const int* uidx,
-                                const signed char* uimg, int ucap, int* cnt, int* nbr,
+template <typename R>
+cudaError_t launch_neigh_ingest(const WorkArgs& a, bool geom, const double* pos, double Lx, double Ly, double Lz,
+                                const int* ucnt, const int* uidx, const signed char* uimg, int ucap, int* cnt, int* nbr,
                                 signed char* img, double* rij, int* key, int* flags, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  return launch_k(neigh_ingest_kernel, dim3(blocks_for((long)n * K, 256)), dim3(256), 0, s, n, K, pos, Lx, Ly,
-                  Lz, ucnt, uidx, uimg, ucap, cnt, nbr, img, rij, key, flags);
+  if (a.n <= 0) return cudaSuccess;
+  return launch_k(geom ? neigh_ingest_kernel<R, true> : neigh_ingest_kernel<R, false>,
+                  dim3(blocks_for((long)a.n * a.K, 128)), dim3(128), 0, s, a, pos, Lx, Ly, Lz, ucnt, uidx, uimg, ucap,
+                  cnt, nbr, img, rij, key, flags);
 }
-
+template cudaError_t launch_neigh_ingest<float>(const WorkArgs&, bool, const double*, double, double, double,
+                                                const int*, const int*, const signed char*, int, int*, int*,
+                                                signed char*, double*, int*, int*, cudaStream_t);
+template cudaError_t launch_neigh_ingest<double>(const WorkArgs&, bool, const double*, double, double, double,
+                                                 const int*, const int*, const signed char*, int, int*, int*,
+                                                 signed char*, double*, int*, int*, cudaStream_t);
 
 }  // namespace snap

@@ -487,9 +487,32 @@ void HostTables::build(int J2) {
       }
     }
 
-  rootpq.assign(kRootDim * kRootDim, 0.0);
-  for (int p = 0; p < kRootDim; ++p)
-    for (int q = 1; q < kRootDim; ++q) rootpq[p * kRootDim + q] = std::sqrt((double)p / (double)q);
+  // classes of one length in units of about 50 multiply-adds a pair (the last
+  // unit of a length repeats its last class), then the same classes one a unit
+  u_units.clear();
+  u_nunits = u_cost = 0;
+  for (int fine = 0; fine < 2; ++fine) {
+    if (fine) u_nunits = (int)u_units.size() / kUUnit;
+    for (int K = J2 / 2 + 1; K >= 1; --K) {
+      const int most = fine || K >= 5 ? 1 : K >= 3 ? 2 : K == 2 ? 3 : 5;
+      std::vector<int> cls;
+      int at = 0;
+      for (int p = 0; p <= J2; ++p)
+        for (int q = J2 - p; q >= 0; --q) {
+          const int steps = (J2 - p - q) / 2 + 1;
+          if (steps == K) cls.push_back(p | q << 4 | at << 8);
+          at += steps;
+        }
+      for (size_t c = 0; c < cls.size(); c += most) {
+        std::vector<int> u(kUUnit, 0);
+        u[0] = K;
+        u[1] = most;
+        for (int k = 0; k < most; ++k) u[2 + k] = cls[std::min(c + k, cls.size() - 1)];
+        u_units.insert(u_units.end(), u.begin(), u.end());
+        if (fine) u_cost += 6 + 6 * K;
+      }
+    }
+  }
 }
 
 void HostTables::build_classes(bool wide) {

@@ -46,7 +46,6 @@ struct HostTables {
   std::vector<double> bdev_coef;
   std::vector<int> bdev_o;
   std::vector<unsigned short> bchunk_runs;
-  std::vector<double> rootpq;
   // [H]: S_t(ma, mb) = sqrt((t - ma)! ma! / (t - mb)!) of every half-layout
   // element, the factor between the scaled recursion's v and u
   std::vector<double> half_scale;
@@ -63,6 +62,12 @@ struct HostTables {
   // pair_ab: alpha_{k-1}, beta_{k-1} of the recursion to P_k (0, 0 at k = 0).
   std::vector<unsigned> pair_idx;
   std::vector<double> pair_norm, pair_weight, pair_ab;
+  // compute_U's units (snap_u.cu): [nunits][kUUnit] the steps K of its classes,
+  // their number M, and per class p | q << 4 | first step << 8; longest first:
+  // u_nunits of about equal work, then each class by itself.  u_cost: about the
+  // multiply-adds of all classes for a pair.
+  std::vector<int> u_units;
+  int u_nunits = 0, u_cost = 0;
 
   // compute_Y of the mixed path (yc_kernel, snap_kernels.cu).  With m = (2 ma -
   // t, 2 mb - t) the doubled projections of an element, the elements of every
