@@ -1002,11 +1002,12 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
   std::vector<__int128> s(nt * 4, 0);
   ll acc[2][4];  // of each output's record: ph, pc, qh, qc
   tab.yc_rows([&](int k, const unsigned* h, int r, size_t p, int o, int len) {
-    const int s1 = (h[0] >> 31) ? -1 : 1, s2 = (h[1] >> 31) ? -s1 : s1;
+    const unsigned at = h[o];  // half o's u[m1] and u[m2]
+    const int s1 = (at >> 15 & 1u) ? -1 : 1, s2 = (at >> 31) ? -s1 : s1;
     ll rh = 0, rc = half, ih = 0, ic = half;
     for (int c2 = 0; c2 < len; ++c2) {
       const ll wh = (int)words[p + 2 * c2], wl = (int)words[p + 2 * c2 + 1];
-      const int e = 2 * elem[(h[1] & 0x7FFFFFFFu) / 256 + c2];
+      const int e = 2 * elem[(at >> 16 & 0x7FFFu) + c2];
       rh += wh * uh[e];
       rc += wh * ul[e] + wl * uh[e];
       ih += s2 * wh * uh[e + 1];
@@ -1015,7 +1016,7 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
     ll Ah, Al, Bh, Bl;
     split(rh + (rc >> 30), Ah, Al);
     split(ih + (ic >> 30), Bh, Bl);
-    const int e = 2 * elem[(h[0] & 0x7FFFFFFFu) / 256 + r];
+    const int e = 2 * elem[(at & 0x7FFFu) + r];
     const ll xh = uh[e], xl = ul[e], zh = uh[e + 1], zl = ul[e + 1];
     ll* a = acc[o];
     if (r == 0) {
@@ -1027,8 +1028,9 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
     a[2] += xh * Bh + zh * Ah;
     a[3] += xh * Bl + xl * Bh + zh * Al + zl * Ah;
     if (r + 1 == (int)(h[2] & 255u)) {
-      s[(size_t)k * 4 + 2 * o] += a[0] + (a[1] >> 30);
-      s[(size_t)k * 4 + 2 * o + 1] += s1 * (a[2] + (a[3] >> 30));
+      const int out = tab.yc_task[(size_t)k * snap::kYcTask + 2] == 1 ? 0 : o;
+      s[(size_t)k * 4 + 2 * out] += a[0] + (a[1] >> 30);
+      s[(size_t)k * 4 + 2 * out + 1] += s1 * (a[2] + (a[3] >> 30));
     }
   });
   for (size_t k = 0; k < nt; ++k)

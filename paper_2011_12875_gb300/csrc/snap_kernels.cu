@@ -200,8 +200,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // memory 42%, FMA pipe 36% of the launch).
 // Measured, list of terms -> now: FP32, 2000 atoms, 2J8 41 -> 35 us, 2J11 199 ->
 // 120, 2J14 845 -> 388; 16000 atoms, 2J8 218 -> 179, 2J14 6005 -> 2809; FP64 (in
-// fixed point, below), 2000 atoms, 2J8 404 -> 197, 2J11 2388 -> 944, 2J14 9335 ->
-// 3390; 128 atoms, 2J8 119 -> 29.
+// fixed point, below), 2000 atoms, 2J8 404 -> 170, 2J11 2388 -> 820, 2J14 9335 ->
+// 3039; 128 atoms, 2J8 119 -> 28.
 // Chunks of a warp's ring
 __host__ __device__ constexpr int yc_slots(int rsize) { return rsize == 8 ? 2 : 3; }
 // Warps of a CTA, by the longest vector LM: one CTA an SM above 2J = 9 (the
@@ -421,7 +421,8 @@ struct YcSingle {
 //
 // A block is 16 atoms (a row of 16 x 16 bytes is then 256, as in FP32, and the
 // whole of 2J14 stays in shared memory); a warp's halves take the two outputs
-// of a task.
+// of a task, or halves of the pairs of a single one (the classes' odd outputs:
+// with a half idle there, 2J8 took 197 us and 2J14 3390).
 __device__ __forceinline__ void wide_add(long long& s, int x, int y) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(x), "r"(y));
 }
@@ -434,10 +435,20 @@ struct Acc96 {
         : "+r"(lo), "+r"(mid), "+r"(hi)
         : "r"(l), "r"(h), "r"(s));
   }
+  __device__ __forceinline__ void add(const Acc96& v) {
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(lo), "+r"(mid), "+r"(hi)
+        : "r"(v.lo), "r"(v.mid), "r"(v.hi));
+  }
   __device__ __forceinline__ double value() const {
     return fma((double)(long long)(((unsigned long long)hi << 32) | mid), 4294967296.0, (double)lo);
   }
 };
+
+// the sum of the lane in the warp's other half
+__device__ __forceinline__ Acc96 shfl16(const Acc96& v) {
+  return Acc96{__shfl_xor_sync(kFull, v.lo, 16), __shfl_xor_sync(kFull, v.mid, 16), __shfl_xor_sync(kFull, v.hi, 16)};
+}
 
 // hi hi and cross sums to one number, rounded (the cross sum starts at half
 // of 2^30), plus 2^29
@@ -454,10 +465,11 @@ __device__ __forceinline__ void yf_run(const unsigned* __restrict__& p, YcHead& 
                                        Acc96& yr, Acc96& yi) {
   constexpr int LP = (L + 1) & ~1, ROW = LP * 4;
   do {
-    const char* u1 = ul + (h.h.x & 0x7FFFFFFFu);
-    const char* u2 = ul + (h.h.y & 0x7FFFFFFFu);
+    const unsigned at = half ? h.h.y : h.h.x;
+    const char* u1 = ul + ((at & 0x7FFFu) << 8);
+    const char* u2 = ul + ((at >> 8) & 0x7FFF00u);
     // conj(u1) v = conj(u1 conj(v)): u[m1] is taken as it is
-    const int c1 = (int)h.h.x >> 31, c2 = c1 ^ ((int)h.h.y >> 31);  // -1: conjugate
+    const int c1 = (int)(at << 16) >> 31, c2 = c1 ^ ((int)at >> 31);  // -1: conjugate
     const unsigned* q = p + 4 + half * LP * 2;
     p += 4 + h.rows() * ROW;
     const unsigned* end = p + half * LP * 2;
@@ -543,8 +555,13 @@ struct YcFixed {
   static constexpr int kBad = 1 << 20;
   __device__ __forceinline__ void store(const int* __restrict__ rec, uint4 h, char* Yb, const char* other, int lane,
                                         int ex) const {
-    const int o = lane >> 4;
-    if (o >= __ldg(rec + 2)) return;
+    const int o = lane >> 4, nout = __ldg(rec + 2);
+    Acc96 r = yr, i = yi;
+    if (nout == 1) {  // the halves are parts of one sum
+      r.add(shfl16(yr));
+      i.add(shfl16(yi));
+    }
+    if (o >= nout) return;
     const int ec = (int)(o ? h.w : h.z), n = 2 * ex + ec - 58;
     // 2^n in two factors (a coefficient may be as small or large as a double)
     const int n1 = n >> 1, n2 = n - n1;
@@ -552,7 +569,7 @@ struct YcFixed {
     const double f2 = __hiloint2double((n2 + 1023) << 20, 0);
     if (ex == kBad || ec == kYcNan) f1 = __longlong_as_double(0x7FF8000000000000LL);
     const int at = __ldg(rec + 4 + o) * 32 + (lane & 15);
-    cx<double> v = mk<double>(yr.value() * f1 * f2, yi.value() * f1 * f2);
+    cx<double> v = mk<double>(r.value() * f1 * f2, i.value() * f1 * f2);
     if (other) {
       const cx<double> w = reinterpret_cast<const cx<double>*>(other)[at];
       v = mk<double>(v.re + w.re, v.im + w.im);

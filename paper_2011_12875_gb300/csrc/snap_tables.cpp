@@ -515,6 +515,9 @@ void HostTables::build(int J2) {
   }
 }
 
+// a vector's byte offset and conjugation (bit 31) in 16 bits
+static unsigned yc_pack(unsigned w) { return (w & 0x7FFFFFFFu) >> 8 | (w >> 31) << 15; }
+
 void HostTables::build_classes(bool wide) {
   yc_wide = wide;
   const int J = twojmax, cw = wide ? 2 : 1;
@@ -615,6 +618,26 @@ void HostTables::build_classes(bool wide) {
           total += p.cost;
           rows.push_back(p);
         }
+        // What a record holds: one pair (m1, m2), or (wide, a single output) two of
+        // one shape, the second for the warp's other half
+        struct Unit {
+          int a, b;
+        };
+        std::vector<Unit> units;
+        const bool split = wide && nout == 1;
+        for (int k = 0; k < (int)items.size(); ++k) {
+          if (rows[k].r1 <= rows[k].r0) continue;
+          auto shape = [&](int x) { return items[x].l2 * 16 + rows[x].r1 - rows[x].r0; };
+          if (split) {
+            auto it = std::find_if(units.begin(), units.end(), [&](const Unit& u) { return u.b < 0 && shape(u.a) == shape(k); });
+            if (it != units.end()) {
+              it->b = k;
+              total -= rows[k].cost;
+              continue;
+            }
+          }
+          units.push_back({k, split ? -1 : k});
+        }
         // two tasks of about equal cost, each with half of the pairs
         size_t next = 0;
         const int parts = total >= kYcWhole ? 2 : 1;
@@ -641,32 +664,42 @@ void HostTables::build_classes(bool wide) {
           };
           open();
           long cost = 200;
-          for (; next < items.size() && (part + 1 == parts || cost - 200 < total / 2); ++next) {
-            const Item& it = items[next];
-            const int lo1 = low(it.m1.a, it.m1.b), lo2 = low(it.m2.a, it.m2.b), l2p = (it.l2 + 1) & ~1;
+          for (; next < units.size() && (part + 1 == parts || cost - 200 < total / 2); ++next) {
+            const Unit u = units[next];
+            const Item& it = items[u.a];
+            const int l2p = (it.l2 + 1) & ~1, r0 = rows[u.a].r0, nrows = rows[u.a].r1 - r0;
             const size_t row = (size_t)np * l2p * 2 * cw;
-            for (int r = rows[next].r0; r < rows[next].r1;) {
+            for (int r = 0; r < nrows;) {
               // four words are left at a chunk's end for the head that ends it
               size_t fit = pos + 8 <= kYcChunk ? (kYcChunk - 8 - pos) / row : 0;
               if (fit == 0) {
                 open();
                 fit = (kYcChunk - 8 - pos) / row;
               }
-              const int n = (int)std::min<size_t>(fit, rows[next].r1 - r);
+              const int n = (int)std::min<size_t>(fit, nrows - r);
               const size_t w0 = yc_head.size() - kYcChunk + pos;
-              yc_head[w0] = place(it.m1) + (unsigned)r * 256u;
-              yc_head[w0 + 1] = place(it.m2);
+              for (int h = 0; h < 2; ++h) {
+                const int k = h == 0 || u.b < 0 ? u.a : u.b;
+                const unsigned o1 = place(items[k].m1) + (unsigned)(rows[k].r0 + r) * 256u, o2 = place(items[k].m2);
+                if (wide) yc_head[w0 + h] = yc_pack(o1) | yc_pack(o2) << 16;
+                else yc_head[w0 + h] = h == 0 ? o1 : o2;
+              }
               yc_head[w0 + 2] = (unsigned)n | (unsigned)it.l2 << 8;
               for (size_t w = w0 + 4; w < w0 + 4 + n * row; w += row, ++r)
-                for (int o = 0; o < nout; ++o)
-                  for (int c = 0; c < it.l2; ++c) {
+                for (int o = 0; o < (wide ? 2 : nout); ++o) {
+                  const int k = split && o == 1 ? u.b : u.a, out = split ? 0 : o;
+                  if (k < 0 || out >= nout) continue;
+                  const Item& p = items[k];
+                  const int t1 = low(p.m1.a, p.m1.b) + 2 * (rows[k].r0 + r), lo2 = low(p.m2.a, p.m2.b);
+                  for (int c = 0; c < p.l2; ++c) {
                     const size_t x =
                         wide ? w + ((size_t)o * l2p + c) * 2 : w + ((size_t)(o / 2) * l2p + c) * 2 + (o & 1);
-                    yc_cg[x] = coef(lo1 + 2 * r, it.m1, lo2 + 2 * c, it.m2, tb + 2 * o, yc_trip[x]);
+                    yc_cg[x] = coef(t1, p.m1, lo2 + 2 * c, p.m2, tb + 2 * out, yc_trip[x]);
                   }
+                }
               pos += 4 + n * row;
             }
-            cost += rows[next].cost;
+            cost += rows[u.a].cost;
           }
           yc_head[yc_head.size() - kYcChunk] |= 0x80000000u;
           rec[1] = (int)(yc_head.size() / kYcChunk) - rec[0];
@@ -691,6 +724,8 @@ std::vector<unsigned> HostTables::yc_stream(const double* beta) const {
 std::vector<unsigned> HostTables::yc_fixed(const double* beta) const {
   const std::vector<double> bw = beta_weights(beta);
   auto coef = [&](size_t x) { return yc_trip[x] < 0 ? 0.0 : yc_cg[x] * bw[yc_trip[x]]; };
+  // the output of a half: the same one in tasks of a single output
+  auto out_of = [&](size_t k, int h) { return yc_task[k * kYcTask + 2] == 1 ? 0 : h; };
   std::vector<double> top(yc_cost.size() * kYcOuts, 0.0);  // largest sum over a record of each output
   const unsigned* last[2] = {nullptr, nullptr};
   double sum[2] = {0.0, 0.0};
@@ -698,7 +733,7 @@ std::vector<unsigned> HostTables::yc_fixed(const double* beta) const {
     if (last[o] != head) sum[o] = 0.0;
     last[o] = head;
     for (int c = 0; c < len; ++c) sum[o] += std::fabs(coef(w + 2 * c));
-    double& t = top[(size_t)k * kYcOuts + o];
+    double& t = top[(size_t)k * kYcOuts + out_of(k, o)];
     if (!(sum[o] <= t)) t = sum[o];  // a NaN stays
   });
   std::vector<int> ex(top.size(), 0);  // top < 2^ex
@@ -709,9 +744,9 @@ std::vector<unsigned> HostTables::yc_fixed(const double* beta) const {
   std::vector<unsigned> w(yc_head);
   for (size_t k = 0; k < yc_cost.size(); ++k)
     for (int ch = yc_task[k * kYcTask]; ch < yc_task[k * kYcTask] + yc_task[k * kYcTask + 1]; ++ch)
-      for (int o = 0; o < 2; ++o) w[(size_t)ch * kYcChunk + 2 + o] = (unsigned)ex[k * kYcOuts + o];
+      for (int o = 0; o < 2; ++o) w[(size_t)ch * kYcChunk + 2 + o] = (unsigned)ex[k * kYcOuts + out_of(k, o)];
   yc_rows([&](int k, const unsigned*, int, size_t p, int o, int len) {
-    const int e = ex[(size_t)k * kYcOuts + o];
+    const int e = ex[(size_t)k * kYcOuts + out_of(k, o)];
     for (int c = 0; c < len; ++c) {
       const long long v = e == kYcNan ? 0 : std::llrint(std::ldexp(coef(p + 2 * c), 60 - e));
       const int hi = (int)((v + (1LL << 29)) >> 30);

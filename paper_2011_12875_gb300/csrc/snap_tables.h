@@ -92,8 +92,11 @@ struct HostTables {
   //   triples (-1: not one);
   // yc_cost: about the instructions of each task.
   // wide (the FP64 path): a coefficient is two words (yc_cg / yc_trip at the
-  // first), a row 2 outputs x (length rounded up to even), np = 1, and words
-  // 2-3 of a chunk are the exponents of its task's outputs (yc_fixed).
+  // first), a row 2 halves x (length rounded up to even), np = 1, words 2-3 of a
+  // chunk are the exponents of its task's outputs (yc_fixed), and words 0-1 of a
+  // head are for a warp's two halves, u[m1] in the lower and u[m2] in the upper 16
+  // bits (slot, bit 15: conjugate).  The halves take the two outputs of a task,
+  // from one pair (m1, m2), or, in a task of one output, two pairs of one shape.
   std::vector<int> yc_slot, yc_task, yc_trip;
   std::vector<unsigned> yc_head;
   std::vector<double> yc_cg;
