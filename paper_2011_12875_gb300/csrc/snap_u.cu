@@ -15,15 +15,15 @@
 // are summed (two buffers).
 //
 // A step (two elements) takes 2 multiply-adds for P_k and 4 for the sums, a
-// class 8 for its monomials, 8 J for the powers: about 840 a pair at 2J8, 2,700
-// at 2J14, where the layer recursion (the form before) took 1,550 and 6,500,
+// class 8 for its monomials, up to 8 J for the powers: about 840 a pair at 2J8,
+// 2,700 at 2J14, where the layer recursion (the form before) took 1,550 and 6,500,
 // with a lane a column (31% of the lanes idle).  FP64 is bound by the FP64 pipe
 // (a warp's multiply-add takes 15 cycles of an SM) and by SMs that hold one CTA
 // more than others; FP32 by latency and instruction fetch, which is why the CTAs'
 // warps run the same code and FP32 takes this form only above 2J = 9.  Neighbour
-// build and compute_U together, before -> now, 2000 atoms: FP64 2J8 278 -> 163 us,
-// 2J11 690 -> 295, 2J14 1113 -> 420; FP32 2J11 57 -> 50, 2J14 86 -> 57, 16000 atoms
-// 556 -> 345.  (128 atoms FP64 2J8: 58 -> 61.)
+// build and compute_U together, before -> now, 2000 atoms: FP64 2J8 278 -> 164 us,
+// 2J11 690 -> 274, 2J14 1113 -> 384; FP32 2J11 57 -> 50, 2J14 86 -> 57, 16000 atoms
+// 556 -> 347; 128 atoms FP64 2J8 58 -> 53.
 #include <algorithm>
 
 #include "snap_geom.cuh"
@@ -72,10 +72,11 @@ struct Slot {
 };
 
 // The chains of powers of a chunk's slots [s0, s0 + S) from the staged geometry
-// ([slot][a, b, f_c][32]): warp w takes chains w, w + nw, ...
+// ([slot][a, b, f_c][32]), up to the CTA's highest: warp w takes chains w, w +
+// nw, ...
 template <typename R>
-__device__ __noinline__ void u_tables(const R* __restrict__ geo, R* t, int J, int s0, int nslots, int warp, int nw,
-                                         int lane) {
+__device__ __noinline__ void u_tables(const R* __restrict__ geo, R* t, int J, int pmax, int qmax, int s0, int nslots,
+                                       int warp, int nw, int lane) {
   constexpr int S = u_slots(sizeof(R));
   for (int j = warp; j < 2 * S; j += nw) {
     const int s = s0 + (j >> 1);
@@ -90,14 +91,14 @@ __device__ __noinline__ void u_tables(const R* __restrict__ geo, R* t, int J, in
       T.x[lane] = na < nb ? fm(R(2), na, R(-1)) : fm(R(-2), nb, R(1));
       r2<R> v = {g[128], R(0)};
       T.A[lane] = v;
-      for (int p = 1; p <= J; ++p) {
+      for (int p = 1; p <= pmax; ++p) {
         v = cmul(v, ca);
         T.A[p * 32 + lane] = v;
       }
     } else {
       r2<R> v = {R(1), R(0)};
       T.B[lane] = v;
-      for (int q = 1; q <= J; ++q) {
+      for (int q = 1; q <= qmax; ++q) {
         v = q == 1 ? b : cmul(v, b);
         T.B[q * 32 + lane] = v;
       }
@@ -109,6 +110,7 @@ struct UArgs {
   const int* un;  // the warp's unit
   int part, sums;  // half of the slots, place of the unit's sums in shared memory
   int warp, nw, lane, nslots;
+  int pmax, qmax;  // highest powers of the CTA's classes
   long blk;
 };
 
@@ -132,10 +134,11 @@ __device__ __forceinline__ void u_unit(const WorkArgs& a, const UArgs& u, const 
 #pragma unroll
     for (int k = 0; k < K; ++k) sp[m][k] = sm[m][k] = r2<R>{R(0), R(0)};
   }
-  u_tables<R>(geo, tab, J, 0, u.nslots, u.warp, u.nw, lane);
+  u_tables<R>(geo, tab, J, u.pmax, u.qmax, 0, u.nslots, u.warp, u.nw, lane);
   __syncthreads();
   for (int s0 = 0, buf = 0; s0 < u.nslots; s0 += S, buf ^= 1) {
-    u_tables<R>(geo, tab + (size_t)(buf ^ 1) * S * len, J, s0 + S, u.nslots, u.warp, u.nw, lane);
+    u_tables<R>(geo, tab + (size_t)(buf ^ 1) * S * len, J, u.pmax, u.qmax, s0 + S, u.nslots, u.warp, u.nw,
+                lane);
     if (M > 0) {
 #pragma unroll 1
       for (int j = u.part; j < S; j += 2) {
@@ -236,6 +239,18 @@ __global__ void __launch_bounds__(kUMaxWarps * 32, 1) u_kernel(WorkArgs a, int u
   R* geo = reinterpret_cast<R*>(ab + a.npair_steps);
   R* tab = geo + (size_t)a.K * 160;
   for (int k = threadIdx.x; k < a.npair_steps; k += blockDim.x) ab[k] = reinterpret_cast<const r2<R>*>(a.pair_ab)[k];
+  {  // a lane a class of the CTA's units
+    const int n = min(per, nu - per * (int)blockIdx.y) * (kUUnit - 2);
+    int p = 0, q = 0;
+    for (int k = u.lane; k < n; k += 32) {
+      const int* un = a.u_units + (size_t)(u0 + per * (int)blockIdx.y + k / (kUUnit - 2)) * kUUnit;
+      const int w = __ldg(un + 2 + k % (kUUnit - 2));  // 0 past the unit's classes
+      p = max(p, w & 15);
+      q = max(q, (w >> 4) & 15);
+    }
+    u.pmax = __reduce_max_sync(kFull, p);
+    u.qmax = __reduce_max_sync(kFull, q);
+  }
   const long i = u.blk * 32 + u.lane;
   const int cnt = i < a.n ? min(a.cnt[i], a.K) : 0;
   u.nslots = __reduce_max_sync(kFull, cnt);  // the same on every warp
@@ -309,8 +324,8 @@ cudaError_t launch_neigh_geom(const NeighArgs& na, const WorkArgs& a, int ncta, 
 // The units (several classes each, or one: HostTables::u_units) and the
 // groups.  The CTAs an SM holds share its pipes, a quarter of them each warp:
 // in multiply-adds a slot a launch lasts about
-//   max(ceil(blocks G / SMs) (cost / G + 8 J) / 4, half the longest unit),
-// cost = a block's units, 8 J = the powers that each CTA tabulates; at most
+//   max(ceil(blocks G / SMs) (cost / G + 4 J) / 4, half the longest unit),
+// cost = a block's units, 4 J = about the powers that each CTA tabulates; at most
 // kUMaxWarps / 2 units a CTA.  Fewer than four warps would build the tables one
 // chain after the other.
 template <typename R>
@@ -322,7 +337,7 @@ cudaError_t launch_u(const WorkArgs& a, cudaStream_t s) {
   for (int f = 0; f < 2; ++f) {
     const int nu = f ? a.u_nfine : a.u_nunits;
     for (int g = (nu + kUMaxWarps / 2 - 1) / (kUMaxWarps / 2); g <= nu; ++g) {
-      const double t = std::max((double)((nblk * g + nsm - 1) / nsm) * ((double)a.u_cost / g + 8.0 * a.twojmax) / 4.0,
+      const double t = std::max((double)((nblk * g + nsm - 1) / nsm) * ((double)a.u_cost / g + 4.0 * a.twojmax) / 4.0,
                                 f ? 27.0 : 30.0);
       if (t < best - 1e-9) {
         best = t;
