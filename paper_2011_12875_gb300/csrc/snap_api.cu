@@ -989,7 +989,11 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
   typedef long long ll;
   const std::vector<unsigned> words = tab.yc_fixed(beta);
   double mx = 0.0;
-  for (int e = 0; e < 2 * tab.H; ++e) mx = std::max(mx, std::fabs(u[e]));
+  for (int e = 0; e < 2 * tab.H; ++e) mx = std::isfinite(u[e]) ? std::max(mx, std::fabs(u[e])) : INFINITY;
+  if (!std::isfinite(mx)) {
+    for (int e = 0; e < 2 * tab.H; ++e) y[e] = NAN;
+    return SNAP_OK;
+  }
   int ex = 0;
   std::frexp(mx, &ex);
   const ll half = 1LL << 29, one30 = 1LL << 30;
@@ -1037,7 +1041,7 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
     for (int o = 0; o < tab.yc_task[k * snap::kYcTask + 2]; ++o) {
       const int e = (int)words[(size_t)tab.yc_task[k * snap::kYcTask] * snap::kYcChunk + 2 + o];
       const __int128* d = &s[k * 4 + 2 * o];
-      if (e == snap::kYcNan || !std::isfinite(mx)) store(k, o, NAN, NAN);
+      if (e == snap::kYcNan) store(k, o, NAN, NAN);
       else store(k, o, std::ldexp((double)d[0], 2 * ex + e - 58), std::ldexp((double)d[1], 2 * ex + e - 58));
     }
   return SNAP_OK;
@@ -1159,7 +1163,17 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
     rc = upload_r(c, &c->d_pair_scale, w);
   }
   if (!rc) rc = upload_r(c, &c->d_pair_norm, c->tab.pair_norm);
-  if (!rc) rc = upload_r(c, &c->d_pair_ab, c->tab.pair_ab);
+  if (!rc) {
+    std::vector<double> ab(c->tab.pair_ab);
+    if (precision == SNAP_MIXED) {  // alpha, beta, and what their rounding to FP32 leaves off
+      ab.clear();
+      for (size_t k = 0; k < c->tab.pair_ab.size(); k += 2) {
+        const double al = c->tab.pair_ab[k], be = c->tab.pair_ab[k + 1];
+        ab.insert(ab.end(), {al, be, al - (double)(float)al, be - (double)(float)be});
+      }
+    }
+    rc = upload_r(c, &c->d_pair_ab, ab);
+  }
   if (!rc) rc = upload(c, &c->d_u_units, c->tab.u_units);
   if (!rc) rc = upload_yrec(c);
   if (!rc) rc = upload_brec(c);

@@ -1,5 +1,5 @@
-// snap_col_f32.cu -- register column-chain compute_U and fused dE kernels,
-// FP32 working precision (mixed mode), one instance per 2J.
+// snap_col_f32.cu -- instances in FP32 working precision (mixed mode), one per
+// 2J: compute_U by the layer recursion, the fused dE, the tangent of Ulisttot.
 #include "snap_colkernels.cuh"
 #include "snap_pairs.cuh"
 

@@ -1,6 +1,5 @@
-// snap_col_f64.cu -- register column-chain kernels in FP64 working
-// precision, one instance per 2J: compute_U, the reverse-mode fused dE and
-// the tangent of Ulisttot along a displacement field.
+// snap_col_f64.cu -- instances in FP64 working precision, one per 2J: the fused
+// dE and the tangent of Ulisttot along a displacement field.
 #include "snap_colkernels.cuh"
 #include "snap_pairs.cuh"
 

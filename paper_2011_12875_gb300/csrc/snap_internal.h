@@ -208,7 +208,7 @@ struct WorkArgs {
   const unsigned* pair_idx;
   const void* pair_scale;  // R: norm x weight
   const void* pair_norm;   // R
-  const void* pair_ab;     // R x 2
+  const void* pair_ab;     // rec_ab<R>
   int npair_steps;
   // compute_U's units, [u_nunits + u_nfine][kUUnit] (HostTables::u_units)
   const int* u_units;

@@ -1,4 +1,4 @@
-// snap_kernels.cu -- compute_U, compute_Y, fused dU/dE and the force gather.
+// snap_kernels.cu -- compute_Y, the bispectrum and the force gather.
 //
 // Notation follows arXiv:2011.12875: t = 2j, U_t = Ulisttot, Y_t = adjoint
 // (Eq. y), dE_i/dr_ik = Re sum_t Y_t : conj(dU_t/dr_ik) (Eq. snapforce2).

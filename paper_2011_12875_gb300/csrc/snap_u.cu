@@ -40,8 +40,24 @@ struct __align__(2 * sizeof(R)) r2 {
   R x, y;
 };
 
+// alpha_k, beta_k of a step, in FP32 with what their rounding leaves off (as in
+// snap_pairs.cuh)
+template <typename R>
+struct rec_ab;
+template <>
+struct __align__(16) rec_ab<float> {
+  float x, y, z, w;
+};
+template <>
+struct __align__(16) rec_ab<double> {
+  double x, y;
+};
+
 __device__ __forceinline__ float fm(float x, float y, float z) { return __fmaf_rn(x, y, z); }
 __device__ __forceinline__ double fm(double x, double y, double z) { return __fma_rn(x, y, z); }
+
+__device__ __forceinline__ float rec_t(const rec_ab<float>& c, float x) { return fm(c.x, x, c.y) + fm(c.z, x, c.w); }
+__device__ __forceinline__ double rec_t(const rec_ab<double>& c, double x) { return fm(c.x, x, c.y); }
 
 template <typename R>
 __device__ __forceinline__ r2<R> cmul(r2<R> v, r2<R> b) {
@@ -119,7 +135,7 @@ struct UArgs {
 // at the end, always in this way.  un: {K, M, (p, q, first step) x M}.
 template <typename R, int K, int M>
 __device__ __forceinline__ void u_unit(const WorkArgs& a, const UArgs& u, const R* __restrict__ geo, R* tab,
-                                       const r2<R>* __restrict__ ab) {
+                                       const rec_ab<R>* __restrict__ ab) {
   constexpr int S = u_slots(sizeof(R)), MM = M > 0 ? M : 1;
   static_assert(K * M * 4 * 32 <= kUSums, "the unit's sums fit");
   const int J = a.twojmax, len = u_slot_len(J), lane = u.lane;
@@ -155,8 +171,7 @@ __device__ __forceinline__ void u_unit(const WorkArgs& a, const UArgs& u, const 
           P[0] = R(1);
 #pragma unroll
           for (int k = 1; k < K; ++k) {
-            const r2<R> c = ab[st[m] + k];
-            const R t = fm(c.x, x, c.y);
+            const R t = rec_t(ab[st[m] + k], x);
             P[k] = k == 1 ? t : fm(t, P[k - 1], k == 2 ? R(-1) : -P[k - 2]);
           }
           sp[m][0].x += mp.x;
@@ -235,10 +250,10 @@ __global__ void __launch_bounds__(kUMaxWarps * 32, 1) u_kernel(WorkArgs a, int u
   u.lane = threadIdx.x & 31;
   u.nw = blockDim.x >> 5;
   u.blk = blockIdx.x;
-  r2<R>* ab = reinterpret_cast<r2<R>*>(smem);  // [steps]
+  rec_ab<R>* ab = reinterpret_cast<rec_ab<R>*>(smem);  // [steps]
   R* geo = reinterpret_cast<R*>(ab + a.npair_steps);
   R* tab = geo + (size_t)a.K * 160;
-  for (int k = threadIdx.x; k < a.npair_steps; k += blockDim.x) ab[k] = reinterpret_cast<const r2<R>*>(a.pair_ab)[k];
+  for (int k = threadIdx.x; k < a.npair_steps; k += blockDim.x) ab[k] = reinterpret_cast<const rec_ab<R>*>(a.pair_ab)[k];
   {  // a lane a class of the CTA's units
     const int n = min(per, nu - per * (int)blockIdx.y) * (kUUnit - 2);
     int p = 0, q = 0;
@@ -348,7 +363,7 @@ cudaError_t launch_u(const WorkArgs& a, cudaStream_t s) {
   }
   const int nu = fine ? a.u_nfine : a.u_nunits, per = (nu + G - 1) / G, nw = std::max(4, 2 * per);
   const size_t tables = std::max((size_t)2 * u_slots(sizeof(R)) * u_slot_len(a.twojmax), (size_t)per * kUSums);
-  const size_t smem = sizeof(r2<R>) * (size_t)a.npair_steps + sizeof(R) * ((size_t)a.K * 160 + tables);
+  const size_t smem = sizeof(rec_ab<R>) * (size_t)a.npair_steps + sizeof(R) * ((size_t)a.K * 160 + tables);
   cudaError_t e = allow_smem(u_kernel<R>, smem);
   if (e != cudaSuccess) return e;
   return launch_k(u_kernel<R>, dim3((unsigned)nblk, (unsigned)G), dim3(nw * 32), smem, s, a, fine ? a.u_nunits : 0, nu,
