@@ -220,8 +220,8 @@ int snap_bispectrum_deriv_batch(snap_ctx* ctx, int nconf, const int* natoms, con
  *    warps per CTA) from the system size and the largest neighbour count
  *    seen; a 32-pair batch is shared by four warps when an SM would hold fewer
  *    than 2 col_warps batches;
- *  yi_waves (1..8): fineness of the compute_Y split; the slices per 32-atom
- *    block minimise ceil(CTAs / resident CTAs) * (1/slices + 0.02/yi_waves);
+ *  yi_waves (1..8): fineness of the compute_Y split; the CTAs a block of
+ *    atoms minimise ceil(CTAs / SMs) * (1/CTAs a block + 0.02/yi_waves);
  *  yi_layout: 0 = compute_Y with a warp of 32 atoms (lanes = atoms, the
  *    block's Ulisttot staged by TMA; the paper's AoSoA layout, Sec. V-B),
  *    1 = a warp per atom (its Ulisttot staged in shared memory, lanes over
@@ -324,12 +324,13 @@ int snap_half_size(int twojmax);
  * context stays usable.  Returns SNAP_ERR_ARG for on outside {0, 1}. */
 int snap_test_stage_timeout(snap_ctx* ctx, int on);
 
-/* compute_Y's term list for one atom, evaluated on the host in FP64 from the
- * same tables the device walks (Sec. III, Eq. y: Y = sum over the Y triples
- * of beta~ C C U_t1 U_t2, with the list's exact reductions: the two terms of
- * a t1 == t2 triple with swapped factors kept as one, the factors of each
- * output grouped, and the outputs below the centre of the middle column,
- * 2 mb = t with ma > mb, left at zero).  No GPU work: a check of the tables.
+/* compute_Y's stream of coefficients for one atom, walked on the host from the
+ * same tables the device walks (Sec. III, Eq. y: Y = sum over the Y triples of
+ * beta~ C C U_t1 U_t2, ordered as dense forms of two vectors of equal
+ * projections; the outputs below the centre of the middle column, 2 mb = t
+ * with ma > mb, are left at zero): SNAP_MIXED with FP64 arithmetic in place of
+ * FP32, SNAP_FP64 in the kernel's fixed point.  No GPU work: a check of the
+ * tables.
  *   precision: SNAP_FP64 or SNAP_MIXED (the table variant of that path)
  *   beta:      double [snap_num_coeff(twojmax) + 1], beta_0 first
  *   u:         double [H][2] (re, im), Ulisttot of the atom in half layout
