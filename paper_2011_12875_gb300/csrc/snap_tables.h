@@ -69,7 +69,7 @@ struct HostTables {
   std::vector<int> u_units;
   int u_nunits = 0, u_cost = 0;
 
-  // compute_Y of the mixed path (yc_kernel, snap_kernels.cu).  With m = (2 ma -
+  // compute_Y (yc_kernel, snap_kernels.cu).  With m = (2 ma -
   // t, 2 mb - t) the doubled projections of an element, the elements of every
   // rank t with one m are its vector u[m]; the outputs with one M are a class,
   // and its Y is a sum over the unordered pairs m1 + m2 = M of bilinear forms
