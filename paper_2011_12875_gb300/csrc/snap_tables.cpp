@@ -734,7 +734,7 @@ std::vector<unsigned> HostTables::yc_fixed(const double* beta) const {
     last[o] = head;
     for (int c = 0; c < len; ++c) sum[o] += std::fabs(coef(w + 2 * c));
     double& t = top[(size_t)k * kYcOuts + out_of(k, o)];
-    if (!(sum[o] <= t)) t = sum[o];  // a NaN stays
+    if (!std::isnan(t) && !(sum[o] <= t)) t = sum[o];  // a NaN enters, and stays
   });
   std::vector<int> ex(top.size(), 0);  // top < 2^ex
   for (size_t k = 0; k < top.size(); ++k) {
