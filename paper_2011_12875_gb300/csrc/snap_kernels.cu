@@ -87,6 +87,10 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
+// Orders this thread's ordinary accesses to shared memory before bulk copies
+// into it (the async proxy) that are issued after the next barrier: a barrier by
+// itself does not order the two.
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned phase) {
   unsigned ok;
   asm volatile(
@@ -703,7 +707,9 @@ __host__ __device__ constexpr size_t yc_smem(int rsize, int H, int ntasks, int w
 // by TMA bulk copies, one an element (256 bytes), which put it in class-major
 // order.  QUEUE: a persistent launch, (block, split) items from a device
 // counter (flags[5], zeroed with the flags by every evaluation); the staging
-// barrier is reused item after item (its phase flips per completed copy).
+// barrier is reused item after item (its phase flips per completed copy), and a
+// proxy fence stands between an item's accesses to the block and the copies of
+// the next.
 template <class P, int LM, bool QUEUE>
 __global__ void __launch_bounds__(P::kWarps * 32, LM <= 5 ? 2 : 1) yc_kernel(WorkArgs a, int ysplit) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -761,7 +767,8 @@ __global__ void __launch_bounds__(P::kWarps * 32, LM <= 5 ? 2 : 1) yc_kernel(Wor
     yc_tasks<P>(a, reinterpret_cast<const char*>(smem) + (FIXED ? (lane & 15) * 16 : lane * 8), ring, tl, nt, &next_s,
                 met, at, lane, ex);
     if (!QUEUE) break;
-    __syncthreads();  // item_s and the staged block are rewritten next
+    fence_proxy_async();  // this thread's accesses to the staged block (yf_prepare stores to it) come first
+    __syncthreads();      // item_s and the staged block are rewritten next
   }
 }
 
