@@ -339,6 +339,18 @@ int snap_test_stage_timeout(snap_ctx* ctx, int on);
  * precision or a NULL pointer. */
 int snap_yi_host(int twojmax, int precision, const double* beta, const double* u, double* y);
 
+/* The fused dE's sums of npairs pairs of one atom, on the host in the
+ * kernel's arithmetic and from its tables.  No GPU work: a check of the closed
+ * form and of its tables' rounding.
+ *   precision: SNAP_FP64 or SNAP_MIXED (FP32 arithmetic)
+ *   ab:        double [npairs][4], the Cayley-Klein parameters a, b (re, im)
+ *   y:         double [H][2] (re, im), Y of the atom in half layout
+ *   sums:      double [npairs][6]: S = Re Y : conj(u), its derivatives in a
+ *              (re, im) and b (re, im) at fixed x = |a|^2 - |b|^2, and the one
+ *              in x (on the sphere dx = 4 Re(conj(a) da))
+ * Returns SNAP_ERR_ARG for a bad argument. */
+int snap_pair_host(int twojmax, int precision, int npairs, const double* ab, const double* y, double* sums);
+
 /* The bispectrum kernels' term records for one atom, walked on the host in
  * FP64 exactly as the device walks them (Sec. II-A, Eq. z: B_l = Re of the
  * triple product Z^t_{t1t2} : conj(U_t), each output element's terms summed

@@ -82,6 +82,9 @@ struct snap_ctx {
   void* d_pair_scale = nullptr;
   void* d_pair_norm = nullptr;
   void* d_pair_ab = nullptr;
+  double* d_pair_fix = nullptr;  // FP64 alone
+  int* d_pair_cls = nullptr;
+  int npair_cls = 0;
   int* d_u_units = nullptr;
   int* d_yc_bins = nullptr;
   int* d_ysched = nullptr;  // lane schedule of the warp-per-atom compute_Y
@@ -523,6 +526,9 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
   a.pair_scale = c->d_pair_scale;
   a.pair_norm = c->d_pair_norm;
   a.pair_ab = c->d_pair_ab;
+  a.pair_fix = c->d_pair_fix;
+  a.pair_cls = c->d_pair_cls;
+  a.npair_cls = c->npair_cls;
   a.npair_steps = (int)c->tab.pair_idx.size();
   a.u_units = c->d_u_units;
   a.u_nunits = c->tab.u_nunits;
@@ -1097,6 +1103,16 @@ int snap_bi_host(int twojmax, int layout, const double* u, double* b) {
   return SNAP_OK;
 }
 
+int snap_pair_host(int twojmax, int precision, int npairs, const double* ab, const double* y, double* sums) {
+  if (twojmax < 0 || twojmax > snap::kMaxTwoJ || (precision != SNAP_FP64 && precision != SNAP_MIXED) || npairs < 0 ||
+      !ab || !y || !sums)
+    return SNAP_ERR_ARG;
+  snap::HostTables tab;
+  tab.build(twojmax);
+  return precision == SNAP_FP64 ? snap::pair_host<double>(tab, npairs, ab, y, sums)
+                                : snap::pair_host<float>(tab, npairs, ab, y, sums);
+}
+
 int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switchflag,
                 const double* beta, int precision, snap_ctx** out) {
   if (!out) {
@@ -1157,22 +1173,15 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
   if (!rc) rc = upload(c, &c->d_ysched, c->tab.lane_outputs(32, &c->ysched_m));
   if (!rc) rc = upload_r(c, &c->d_hscale, c->tab.half_scale);
   if (!rc) rc = upload(c, &c->d_pair_idx, c->tab.pair_idx);
-  if (!rc) {
-    std::vector<double> w(c->tab.pair_norm);  // the weighted Y of the fused dE
-    for (size_t k = 0; k < w.size(); ++k) w[k] *= c->tab.pair_weight[k];
-    rc = upload_r(c, &c->d_pair_scale, w);
-  }
-  if (!rc) rc = upload_r(c, &c->d_pair_norm, c->tab.pair_norm);
-  if (!rc) {
-    std::vector<double> ab(c->tab.pair_ab);
-    if (precision == SNAP_MIXED) {  // alpha, beta, and what their rounding to FP32 leaves off
-      ab.clear();
-      for (size_t k = 0; k < c->tab.pair_ab.size(); k += 2) {
-        const double al = c->tab.pair_ab[k], be = c->tab.pair_ab[k + 1];
-        ab.insert(ab.end(), {al, be, al - (double)(float)al, be - (double)(float)be});
-      }
-    }
-    rc = upload_r(c, &c->d_pair_ab, ab);
+  const bool fp64 = precision == SNAP_FP64;
+  if (!rc) rc = upload_r(c, &c->d_pair_scale, c->tab.pair_scales(fp64));  // the weighted Y of the fused dE
+  if (!rc) rc = upload_r(c, &c->d_pair_norm, fp64 ? c->tab.pair_norm_fix : c->tab.pair_norm);
+  if (!rc) rc = upload_r(c, &c->d_pair_ab, c->tab.pair_recursion(fp64));
+  if (!rc && fp64) {
+    const std::vector<int> cls = c->tab.pair_classes();
+    c->npair_cls = (int)cls.size();
+    rc = upload(c, &c->d_pair_cls, cls);
+    if (!rc) rc = upload(c, &c->d_pair_fix, c->tab.pair_fix);
   }
   if (!rc) rc = upload(c, &c->d_u_units, c->tab.u_units);
   if (!rc) rc = upload_yrec(c);
@@ -1768,6 +1777,8 @@ int snap_destroy(snap_ctx* c) {
   dfree(c->d_pair_scale);
   dfree(c->d_pair_norm);
   dfree(c->d_pair_ab);
+  dfree(c->d_pair_fix);
+  dfree(c->d_pair_cls);
   dfree(c->d_u_units);
   for (auto& kv : c->yc_bins_cache) cudaFree(kv.second);
   c->yc_bins_cache.clear();

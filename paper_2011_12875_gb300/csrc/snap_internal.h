@@ -24,6 +24,7 @@ constexpr int kYcChunk = 256;  // words of a compute_Y stream chunk (snap_tables
 constexpr int kYcOuts = 8;     // most outputs of a compute_Y task
 constexpr int kYcTask = 4 + 2 * kYcOuts;
 constexpr long kYcWhole = 1000;  // cost from which a task's sum is split in two
+constexpr int kPairFix = 8;  // most steps of a class (HostTables::pair_fix)
 constexpr int kUUnit = 8;  // words of a compute_U unit (HostTables::u_units)
 constexpr int kYcNan = 0x7FFF;  // exponent of an output whose coefficients are not finite
 constexpr int kBChunk = 96;    // bispectrum terms a warp takes at a time (whole groups)
@@ -209,7 +210,9 @@ struct WorkArgs {
   const void* pair_scale;  // R: norm x weight
   const void* pair_norm;   // R
   const void* pair_ab;     // rec_ab<R>
-  int npair_steps;
+  const double* pair_fix;  // FP64: [step][kPairFix], the polynomials' rounding (HostTables::pair_fix)
+  const int* pair_cls;     // FP64: the classes of several steps, first step | steps << 16
+  int npair_steps, npair_cls;
   // compute_U's units, [u_nunits + u_nfine][kUUnit] (HostTables::u_units)
   const int* u_units;
   int u_nunits, u_nfine, u_cost;

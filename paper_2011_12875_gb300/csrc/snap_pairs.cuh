@@ -35,7 +35,8 @@
 // 178); 128 atoms at 2J8 FP64 74 -> 26.
 #pragma once
 #include <algorithm>
-#include <mutex>
+#include <cmath>
+#include <vector>
 
 #include "snap_internal.h"
 
@@ -43,6 +44,9 @@ namespace snap {
 namespace pr {
 
 constexpr unsigned kFull = 0xffffffffu;
+
+// the arithmetic of a pair is the host walk's too (snap_pair_host)
+#define SNAP_HD __host__ __device__ __forceinline__
 
 template <typename R>
 struct __align__(2 * sizeof(R)) r2 {
@@ -55,12 +59,18 @@ struct __align__(16) y4 {
   R pr, pi, mr, mi;
 };
 
-// alpha_k, beta_k of a step.  FP32: with the part that their rounding leaves
-// off, z and w; that rounding is the same for every pair, so its effect adds up
-// over them (2J14: 1.3e-7 of the virial's sum of sizes, the rest of a pair's
-// rounding averages out).  Eight 2000-atom cells, mean error of the virial with
-// the rounded ones / now / the layer recursion: 2J10 7.7e-7 / 5.3e-7 / 5.3e-7, 2J14
-// 3.4e-7 / 2.8e-7 / 3.1e-7, for three operations a step (dE 26.6 -> 28.1 us).
+// alpha_k, beta_k of a step.  Their rounding is the same for every pair, so its
+// effect adds up over them, where the rest of a pair's rounding averages out.
+// FP64 takes them rounded to FP32 and turns the weighted Y, once an atom, into
+// the coefficients in the polynomials that those give (fix_class).  The error
+// that all pairs share, of the size of S, 2J8 / 2J11 / 2J14, in units of 2^-53:
+// 0.7 each, which is the scales' and Y's own rounding; rounded to FP64 and left
+// so 0.8 / 1.1 / 1.4 (tests/test_pair_closed_form.py).  It takes 1% of a step.
+// FP32: with the part that their rounding leaves off, z and w (rounded and left
+// so, 2J14: 1.3e-7 of the virial's sum of sizes).  Eight 2000-atom cells, mean
+// error of the virial with the rounded ones / now / the layer recursion: 2J10
+// 7.7e-7 / 5.3e-7 / 5.3e-7, 2J14 3.4e-7 / 2.8e-7 / 3.1e-7, for three operations a
+// step (dE 26.6 -> 28.1 us).
 template <typename R>
 struct rec_ab;
 template <>
@@ -73,15 +83,20 @@ struct __align__(16) rec_ab<double> {
 };
 
 // x * y + z in one rounding, also where the compiler would split it
+#ifdef __CUDA_ARCH__
 __device__ __forceinline__ float fm(float x, float y, float z) { return __fmaf_rn(x, y, z); }
 __device__ __forceinline__ double fm(double x, double y, double z) { return __fma_rn(x, y, z); }
+#else
+__host__ __device__ inline float fm(float x, float y, float z) { return std::fma(x, y, z); }
+__host__ __device__ inline double fm(double x, double y, double z) { return std::fma(x, y, z); }
+#endif
 
 // alpha x + beta
-__device__ __forceinline__ float rec_t(const rec_ab<float>& c, float x) { return fm(c.x, x, c.y) + fm(c.z, x, c.w); }
-__device__ __forceinline__ double rec_t(const rec_ab<double>& c, double x) { return fm(c.x, x, c.y); }
+SNAP_HD float rec_t(const rec_ab<float>& c, float x) { return fm(c.x, x, c.y) + fm(c.z, x, c.w); }
+SNAP_HD double rec_t(const rec_ab<double>& c, double x) { return fm(c.x, x, c.y); }
 // alpha p + d
-__device__ __forceinline__ float rec_d(const rec_ab<float>& c, float p, float d) { return fm(c.x, p, fm(c.z, p, d)); }
-__device__ __forceinline__ double rec_d(const rec_ab<double>& c, double p, double d) { return fm(c.x, p, d); }
+SNAP_HD float rec_d(const rec_ab<float>& c, float p, float d) { return fm(c.x, p, fm(c.z, p, d)); }
+SNAP_HD double rec_d(const rec_ab<double>& c, double p, double d) { return fm(c.x, p, d); }
 
 // steps (p, q, k) of the classes with p' < p: a class of remainder
 // r = 2J - p - q has r / 2 + 1 steps, stored p rising, then r rising
@@ -121,10 +136,56 @@ struct Sums {
   R s, gar, gai, gbr, gbi, x;
 };
 
+// The weighted, scaled Y of a step (w: HostTables::pair_idx) from the Y of its
+// two elements, at(element) each.
+template <typename R, typename F>
+SNAP_HD y4<R> weighted_y(unsigned w, R sc, F&& at) {
+  const r2<R> u = at(w & 1023u);
+  y4<R> v;
+  const R sp = (w >> 11) & 1u ? -sc : sc;
+  v.pr = sp * u.x;
+  v.pi = ((w >> 10) & 1u) ? -sp * u.y : sp * u.y;
+  v.mr = v.mi = R(0);
+  if ((w >> 22) & 1u) {
+    const r2<R> m = at((w >> 12) & 1023u);
+    v.mr = sc * m.x;
+    v.mi = sc * m.y;
+  }
+  return v;
+}
+
+// One component (y: its values of the steps, 4 apart) of a class of K steps,
+// in place: sum_k Y_k P_k = sum_j (Y_j + sum_{k > j} f_kj Y_k) PP_j, 1 + d_kk being
+// in the scale (fix: HostTables::pair_fix from the class's first step on).
+template <int K>
+SNAP_HD void fix_steps(double* __restrict__ y, const double* __restrict__ fix) {
+  double v[K];
+#pragma unroll
+  for (int j = 0; j < K; ++j) v[j] = y[4 * j];
+#pragma unroll
+  for (int j = 0; j + 1 < K; ++j) {
+#pragma unroll
+    for (int i = 1; j + i < K; ++i) v[j] = fm(fix[j * kPairFix + i], v[j + i], v[j]);
+    y[4 * j] = v[j];
+  }
+}
+SNAP_HD void fix_class(double* y, const double* fix, int K) {
+  switch (K) {
+    case 2: return fix_steps<2>(y, fix);
+    case 3: return fix_steps<3>(y, fix);
+    case 4: return fix_steps<4>(y, fix);
+    case 5: return fix_steps<5>(y, fix);
+    case 6: return fix_steps<6>(y, fix);
+    case 7: return fix_steps<7>(y, fix);
+    case 8: return fix_steps<8>(y, fix);
+    default: return;
+  }
+}
+
 // Q = sum_k Y P_k and X = sum_k Y P_k' of a class of K steps, one or both
 // elements.
 template <typename R, int K, bool BOTH>
-__device__ __forceinline__ void class_sums(const y4<R>* __restrict__ y, const rec_ab<R>* __restrict__ ab, R x, r2<R>& qp,
+SNAP_HD void class_sums(const y4<R>* __restrict__ y, const rec_ab<R>* __restrict__ ab, R x, r2<R>& qp,
                                            r2<R>& qm, r2<R>& xp, r2<R>& xm) {
   qp.x = y[0].pr;
   qp.y = y[0].pi;
@@ -168,14 +229,14 @@ __device__ __forceinline__ void class_sums(const y4<R>* __restrict__ y, const re
 
 // v * b + c (complex)
 template <typename R>
-__device__ __forceinline__ r2<R> cfma(r2<R> v, r2<R> b, r2<R> c) {
+SNAP_HD r2<R> cfma(r2<R> v, r2<R> b, r2<R> c) {
   r2<R> o;
   o.x = fm(-v.y, b.y, fm(v.x, b.x, c.x));
   o.y = fm(v.y, b.x, fm(v.x, b.y, c.y));
   return o;
 }
 template <typename R>
-__device__ __forceinline__ r2<R> cmul(r2<R> v, r2<R> b) {
+SNAP_HD r2<R> cmul(r2<R> v, r2<R> b) {
   r2<R> o;
   o.x = fm(-v.y, b.y, v.x * b.x);
   o.y = fm(v.y, b.x, v.x * b.y);
@@ -192,7 +253,7 @@ struct Horner {
 // The classes r = r0, r0 + 1, ... of one p (q = J2 - p - r falling); `last` =
 // J2 - p.  BOTH: p > 0 (both elements for q > 0).
 template <typename R, int J2, int RR, bool BOTH>
-__device__ __forceinline__ void q_steps(const y4<R>* __restrict__ y, const rec_ab<R>* __restrict__ ab, R x, r2<R> cb,
+SNAP_HD void q_steps(const y4<R>* __restrict__ y, const rec_ab<R>* __restrict__ ab, R x, r2<R> cb,
                                         r2<R> mb, int last, Horner<R>& h) {
   if constexpr (RR <= J2) {
     constexpr int K = RR / 2 + 1;
@@ -228,7 +289,7 @@ __device__ __forceinline__ void q_steps(const y4<R>* __restrict__ y, const rec_a
 
 // The parts [part0, part1) of one pair's sums.
 template <typename R, int J2>
-__device__ __forceinline__ Sums<R> pair_sums(const y4<R>* __restrict__ yat, const rec_ab<R>* __restrict__ abt, r2<R> a,
+SNAP_HD Sums<R> pair_sums(const y4<R>* __restrict__ yat, const rec_ab<R>* __restrict__ abt, r2<R> a,
                                              r2<R> b, int part) {
   // x: the smaller of |a|^2 and |b|^2 from 1 (both carry the rounding of a, b)
   const R na = fm(a.x, a.x, a.y * a.y), nb = fm(b.x, b.x, b.y * b.y);
@@ -282,7 +343,7 @@ __device__ __forceinline__ Sums<R> pair_sums(const y4<R>* __restrict__ yat, cons
 }
 
 template <typename R>
-__device__ __forceinline__ void add_sums(Sums<R>& t, const Sums<R>& o) {
+SNAP_HD void add_sums(Sums<R>& t, const Sums<R>& o) {
   t.s += o.s;
   t.gar += o.gar;
   t.gai += o.gai;
@@ -359,20 +420,7 @@ __global__ void __launch_bounds__(de_max_warps<R>() * 32, 1) de_pair_kernel(Work
       const int st = k / na, al = k - st * na;
       const long i = i0 + al;
       const r2<R>* Yg = reinterpret_cast<const r2<R>*>(a.Y) + (i >> 5) * (long)H * 32 + (i & 31);
-      const unsigned w = __ldg(a.pair_idx + st);
-      const R sc = scg[st];
-      const r2<R> u = Yg[(w & 1023u) * 32];
-      y4<R> v;
-      const R sp = (w >> 11) & 1u ? -sc : sc;
-      v.pr = sp * u.x;
-      v.pi = ((w >> 10) & 1u) ? -sp * u.y : sp * u.y;
-      v.mr = v.mi = R(0);
-      if ((w >> 22) & 1u) {
-        const r2<R> m = Yg[((w >> 12) & 1023u) * 32];
-        v.mr = sc * m.x;
-        v.mi = sc * m.y;
-      }
-      Yw[(size_t)al * NS + st] = v;
+      Yw[(size_t)al * NS + st] = weighted_y<R>(__ldg(a.pair_idx + st), scg[st], [&](unsigned e) { return Yg[e * 32]; });
     }
     if (warp == 0) {  // exclusive offsets of the atoms' pairs (inclusive scan, 32 at a time)
       int carry = 0;
@@ -389,6 +437,13 @@ __global__ void __launch_bounds__(de_max_warps<R>() * 32, 1) de_pair_kernel(Work
       }
     }
     __syncthreads();
+    if constexpr (sizeof(R) == 8) {  // a thread a component of a class (2% of the pairs' work at 2J14)
+      for (int k = threadIdx.x; k < a.npair_cls * na * 4; k += blockDim.x) {
+        const int c = __ldg(a.pair_cls + k / (4 * na)), st = c & 0xFFFF, al = (k >> 2) % na;
+        fix_class(reinterpret_cast<double*>(Yw + (size_t)al * NS + st) + (k & 3), a.pair_fix + st * kPairFix, c >> 16);
+      }
+      __syncthreads();
+    }
     const int total = coff[na];
     const int per = nw / SPLIT;  // batches in flight
     const int nbatch = (total + 31) / 32;
@@ -522,6 +577,32 @@ cudaError_t launch_de_t(const WorkArgs& a, cudaStream_t s) {
   DePlan p = de_plan<R, J2>(a.n, maxcnt, nsm, a.col_warps, a.de_atoms);
   if (p.A == 0) p = de_plan<R, J2>(a.n, maxcnt, nsm, a.col_warps, 0);  // a forced A that does not fit
   return p.split > 1 ? launch_de_split<R, J2, kParts>(a, p, s) : launch_de_split<R, J2, 1>(a, p, s);
+}
+
+// The pairs' sums on the host, in the kernel's arithmetic: ab [npairs][4] the
+// Cayley-Klein parameters, y [H][2], out [npairs][6] the Sums.
+template <typename R, int J2>
+void pair_host_t(const std::vector<unsigned>& idx, const std::vector<double>& scale, const std::vector<double>& ab,
+                 const std::vector<double>& fix, const std::vector<int>& cls, int npairs, const double* par,
+                 const double* y, double* out) {
+  constexpr int NS = steps_total(J2);
+  std::vector<y4<R>> Y(NS);
+  std::vector<rec_ab<R>> t(NS);
+  constexpr int W = sizeof(rec_ab<R>) / sizeof(R);
+  for (int st = 0; st < NS; ++st) {
+    Y[st] = weighted_y<R>(idx[st], (R)scale[st], [&](unsigned e) { return r2<R>{(R)y[2 * e], (R)y[2 * e + 1]}; });
+    for (int k = 0; k < W; ++k) (&t[st].x)[k] = (R)ab[W * st + k];
+  }
+  if constexpr (sizeof(R) == 8)
+    for (int c : cls)
+      for (int k = 0; k < 4; ++k) fix_class(&Y[c & 0xFFFF].pr + k, &fix[(c & 0xFFFF) * kPairFix], c >> 16);
+  for (int n = 0; n < npairs; ++n) {
+    const double* g = par + 4 * n;
+    Sums<R> q{R(0), R(0), R(0), R(0), R(0), R(0)};
+    for (int part = 0; part < kParts; ++part)
+      add_sums(q, pair_sums<R, J2>(Y.data(), t.data(), r2<R>{(R)g[0], (R)g[1]}, r2<R>{(R)g[2], (R)g[3]}, part));
+    for (int k = 0; k < 6; ++k) out[6 * n + k] = (double)(&q.s)[k];
+  }
 }
 
 }  // namespace pr

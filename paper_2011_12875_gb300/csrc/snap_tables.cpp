@@ -448,15 +448,26 @@ void HostTables::build(int J2) {
   // closed form of u: see snap_pairs.cuh.  P_k^(q,p) monic has the recursion
   // pi_{k+1} = (x - b_k) pi_k - g_k pi_{k-1} (Jacobi polynomials, alpha = q,
   // beta = p); with pi_k = s_k P_k, s_{k+1} = g_k s_{k-1}, the last factor is 1.
+  // The kernels hold alpha and beta rounded to FP32, so their polynomials are
+  // others, PP_k, of the same degrees: P_k = PP_k + sum_{j <= k} d_kj PP_j.  From
+  // the two recursions, with x PP_j = (PP_{j+1} + PP_{j-1} - bb_j PP_j) / aa_j,
+  //   d_{k+1,j} = al_k (d_{k,j-1} / aa_{j-1} + d_{k,j+1} / aa_{j+1} - d_kj bb_j / aa_j) + be_k d_kj - d_{k-1,j}
+  // and, for the PP_k in P_k itself, (al_k - aa_k) / aa_k at j = k + 1 and k - 1
+  // and be_k - al_k bb_k / aa_k at j = k.  1 + d_kk goes into the norm.
   pair_idx.clear();
   pair_norm.clear();
+  pair_norm_fix.clear();
   pair_weight.clear();
   pair_ab.clear();
+  pair_fix.clear();
   std::array<long double, kMaxTwoJ + 2> fact;
   for (int k = 0; k < (int)fact.size(); ++k) fact[k] = lfact(k);
   for (int p = 0; p <= J2; ++p)
     for (int q = J2 - p; q >= 0; --q) {
       long double s0 = 1.0L, s1 = 1.0L, al = 0.0L, be = 0.0L;  // s_{k-1}, s_k and the coefficients to P_k
+      long double aa[kPairFix] = {}, bb[kPairFix] = {}, d[kPairFix][kPairFix] = {};
+      const size_t first = pair_idx.size();
+      pair_fix.resize((first + (J2 - p - q) / 2 + 1) * kPairFix, 0.0);
       for (int k = 0; p + q + 2 * k <= J2; ++k) {
         const int t = p + q + 2 * k, c = 2 * k + p + q;
         if (k > 0) {  // s0 = s_{k-1}, s1 = s_k
@@ -464,14 +475,29 @@ void HostTables::build(int J2) {
                                        : (long double)(p * p - q * q) / ((long double)(c - 2) * c);
           al = s0 / s1;
           be = -al * b;
+          const int m = k - 1;
+          aa[m] = (float)al;
+          bb[m] = (float)be;
+          for (int j = 0; j <= k; ++j) {
+            long double v = j > 0 ? al * d[m][j - 1] / aa[j - 1] : 0.0L;
+            if (j <= m) v += (be - al * bb[j] / aa[j]) * d[m][j];
+            if (j < m) v += al * d[m][j + 1] / aa[j + 1] - d[m - 1][j];
+            if (j == k || j == m - 1) v += (al - aa[m]) / aa[m];
+            if (j == m) v += be - al * bb[m] / aa[m];
+            d[k][j] = v;
+          }
+          for (int j = 0; j < k; ++j)
+            pair_fix[(first + j) * kPairFix + k - j] = (double)(d[k][j] / (1.0L + d[k][k]));
         }
         unsigned w;
         if (2 * (k + q) <= t) w = (unsigned)(half_base(t) + (k + q) * (t + 1) + k);
         else w = (unsigned)(half_base(t) + (t - k - q) * (t + 1) + (t - k)) | (1u << 10) | ((unsigned)(q & 1) << 11);
         if (p > 0 && q > 0) w |= ((unsigned)(half_base(t) + k * (t + 1) + k + q) << 12) | (1u << 22);
         pair_idx.push_back(w);
-        pair_norm.push_back((double)(fact[t] / std::pow(2.0L, k) /
-                                     std::sqrt(fact[t - k] * fact[k] * fact[t - k - q] * fact[k + q]) * s1));
+        const long double n = fact[t] / std::pow(2.0L, k) /
+                              std::sqrt(fact[t - k] * fact[k] * fact[t - k - q] * fact[k + q]) * s1;
+        pair_norm.push_back((double)n);
+        pair_norm_fix.push_back((double)(n + n * d[k][k]));
         pair_weight.push_back(p == 0 && q == 0 ? 1.0 : 2.0);
         pair_ab.push_back((double)al);
         pair_ab.push_back((double)be);
@@ -513,6 +539,34 @@ void HostTables::build(int J2) {
       }
     }
   }
+}
+
+std::vector<double> HostTables::pair_scales(bool fp64) const {
+  std::vector<double> w(fp64 ? pair_norm_fix : pair_norm);
+  for (size_t k = 0; k < w.size(); ++k) w[k] *= pair_weight[k];
+  return w;
+}
+
+std::vector<double> HostTables::pair_recursion(bool fp64) const {
+  std::vector<double> ab;
+  for (size_t k = 0; k < pair_ab.size(); k += 2) {
+    const double al = (float)pair_ab[k], be = (float)pair_ab[k + 1];
+    ab.insert(ab.end(), {al, be});
+    if (!fp64) ab.insert(ab.end(), {pair_ab[k] - al, pair_ab[k + 1] - be});
+  }
+  return ab;
+}
+
+std::vector<int> HostTables::pair_classes() const {
+  std::vector<int> cls;
+  int st = 0;
+  for (int p = 0; p <= twojmax; ++p)
+    for (int q = twojmax - p; q >= 0; --q) {
+      const int steps = (twojmax - p - q) / 2 + 1;
+      if (steps > 1) cls.push_back(st | steps << 16);
+      st += steps;
+    }
+  return cls;
 }
 
 // a vector's byte offset and conjugation (bit 31) in 16 bits

@@ -59,9 +59,19 @@ struct HostTables {
   // pair_norm: n s_k, u = n s_k monomial P_k(x);
   // pair_weight: the step's weight in a full-matrix contraction (2; 1 for p =
   //   q = 0);
-  // pair_ab: alpha_{k-1}, beta_{k-1} of the recursion to P_k (0, 0 at k = 0).
+  // pair_ab: alpha_{k-1}, beta_{k-1} of the recursion to P_k (0, 0 at k = 0);
+  // with alpha and beta rounded to FP32 the recursion gives other polynomials PP:
+  // P_k = (1 + d_kk) (PP_k + sum_{j < k} f_kj PP_j).  pair_fix: [kPairFix] a step
+  //   j, f_kj at k - j (0 at 0 and past the class); pair_norm_fix: pair_norm (1 +
+  //   d_kk).
   std::vector<unsigned> pair_idx;
-  std::vector<double> pair_norm, pair_weight, pair_ab;
+  std::vector<double> pair_norm, pair_norm_fix, pair_weight, pair_ab, pair_fix;
+  // What the kernels take of these.  pair_scales: norm x weight; pair_recursion:
+  // a step's rec_ab (snap_pairs.cuh), in FP32 with what the rounding leaves off;
+  // pair_classes: the classes of several steps, first step | steps << 16.
+  std::vector<double> pair_scales(bool fp64) const;
+  std::vector<double> pair_recursion(bool fp64) const;
+  std::vector<int> pair_classes() const;
   // compute_U's units (snap_u.cu): [nunits][kUUnit] the steps K of its classes,
   // their number M, and per class p | q << 4 | first step << 8; longest first:
   // u_nunits of about equal work, then each class by itself.  u_cost: about the
@@ -160,5 +170,9 @@ struct HostTables {
 
 double clebsch_gordan(int tj1, int tm1, int tj2, int tm2, int tj, int tm);
 int count_coeff(int twojmax);
+
+// One atom's pairs in the fused dE's arithmetic, on the host (snap_col_*.cu).
+template <typename R>
+int pair_host(const HostTables& tab, int npairs, const double* par, const double* y, double* out);
 
 }  // namespace snap

@@ -40,8 +40,8 @@ struct __align__(2 * sizeof(R)) r2 {
   R x, y;
 };
 
-// alpha_k, beta_k of a step, in FP32 with what their rounding leaves off (as in
-// snap_pairs.cuh)
+// alpha_k, beta_k of a step, as in snap_pairs.cuh: in FP32 with what their
+// rounding leaves off, in FP64 rounded to FP32 (the sums are then put right)
 template <typename R>
 struct rec_ab;
 template <>
@@ -214,21 +214,44 @@ __device__ __forceinline__ void u_unit(const WorkArgs& a, const UArgs& u, const 
   if (M == 0 || u.part == 1 || u.blk * 32 + lane >= a.n) return;
   r2<R>* U = reinterpret_cast<r2<R>*>(a.U) + u.blk * a.H * 32 + lane;
 #pragma unroll
-  for (int m = 0; m < M; ++m)
+  for (int m = 0; m < M; ++m) {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const R* d = sums + (m * K + k) * 128;
+      sp[m][k].x += d[0];
+      sp[m][k].y += d[32];
+      sm[m][k].x += d[64];
+      sm[m][k].y += d[96];
+    }
+    if constexpr (sizeof(R) == 8) {
+      // P_k from the rounded recursion's PP_k (HostTables::pair_fix)
+#pragma unroll
+      for (int k = K - 1; k > 0; --k)
+#pragma unroll
+        for (int j = 0; j < k; ++j) {
+          const double f = __ldg(a.pair_fix + (st[m] + j) * kPairFix + k - j);
+          sp[m][k].x = fm(f, sp[m][j].x, sp[m][k].x);
+          sp[m][k].y = fm(f, sp[m][j].y, sp[m][k].y);
+          sm[m][k].x = fm(f, sm[m][j].x, sm[m][k].x);
+          sm[m][k].y = fm(f, sm[m][j].y, sm[m][k].y);
+        }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < M; ++m)
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
       const unsigned w = __ldg(a.pair_idx + st[m] + k);
       const R n = reinterpret_cast<const R*>(a.pair_norm)[st[m] + k];
       const R odd = (q[m] & 1) ? R(-1) : R(1);
       // (k, k + q): stored, or its mirror (-1)^q conj is
-      r2<R> v = {n * (sp[m][k].x + d[0]), n * (sp[m][k].y + d[32])};
+      r2<R> v = {n * sp[m][k].x, n * sp[m][k].y};
       if (q[m] == 0) v.x += (R)a.wself;
       const r2<R> mir = {odd * v.x, -odd * v.y};
       U[(w & 1023u) * 32] = ((w >> 10) & 1u) ? mir : v;
       if (p[m] > 0 && q[m] > 0) {
         const R on = odd * n;
-        U[((w >> 12) & 1023u) * 32] = r2<R>{on * (sm[m][k].x + d[64]), on * (sm[m][k].y + d[96])};
+        U[((w >> 12) & 1023u) * 32] = r2<R>{on * sm[m][k].x, on * sm[m][k].y};
         // on the middle column (2 (k + q) = t, p = q) the mirror is stored too
         if (p[m] == q[m]) {
           const int t = p[m] + q[m] + 2 * k, mb = k + q[m];

@@ -51,7 +51,7 @@ EXPORTS = ("snap_num_coeff", "snap_create", "snap_set_beta", "snap_set_neigh_cap
            "snap_compute_bispectrum_async",
            "snap_bispectrum_deriv", "snap_force_weighted", "snap_generation",
            "snap_compute_batch", "snap_set_tuning", "snap_get_tuning", "snap_autotune",
-           "snap_neighbors_noalloc", "snap_yi_host", "snap_bi_host", "snap_test_stage_timeout",
+           "snap_neighbors_noalloc", "snap_yi_host", "snap_bi_host", "snap_pair_host", "snap_test_stage_timeout",
            "snap_probe_fma", "snap_bispectrum_deriv_batch", "snap_set_knob", "snap_get_knob")
 NSTAGES = 5
 
@@ -134,6 +134,8 @@ def load(path: str | None = None):
     L.snap_half_size.restype = i
     L.snap_yi_host.argtypes = [i, i, p, p, p]
     L.snap_yi_host.restype = i
+    L.snap_pair_host.argtypes = [i, i, i, p, p, p]
+    L.snap_pair_host.restype = i
     L.snap_bi_host.argtypes = [i, i, p, p]
     L.snap_bi_host.restype = i
     L.snap_probe_fma.argtypes = [i, i, p, p]
@@ -181,6 +183,18 @@ def yi_host(twojmax: int, beta, u_half, precision: int = MIXED) -> np.ndarray:
     if rc != 0:
         raise SnapError(rc, "snap_yi_host: invalid argument")
     return y
+
+
+def pair_host(twojmax: int, ab, y_half, precision: int = FP64) -> np.ndarray:
+    """The fused dE's sums of one atom's pairs on the host (snap_pair_host):
+    ab [n][4], y_half [H][2] -> [n][6].  No GPU work."""
+    ab = np.ascontiguousarray(ab, dtype=np.float64).reshape(-1, 4)
+    y = np.ascontiguousarray(y_half, dtype=np.float64).reshape(half_size(twojmax), 2)
+    out = np.zeros((len(ab), 6))
+    rc = load().snap_pair_host(twojmax, precision, len(ab), _np_ptr(ab), _np_ptr(y), _np_ptr(out))
+    if rc != 0:
+        raise SnapError(rc, "snap_pair_host: invalid argument")
+    return out
 
 
 def bi_host(twojmax: int, u_half, layout: int = 0) -> np.ndarray:
