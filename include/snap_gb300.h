@@ -38,9 +38,13 @@ extern "C" {
 typedef struct snap_ctx snap_ctx;
 
 /* Working precision of the U, Y and dU recursions.  SNAP_FP64: everything
- * in FP64.  SNAP_MIXED: the three recursions run in FP32; the Cayley-Klein
- * parameters and the per-atom energy, force and virial accumulations stay
- * in FP64. */
+ * in FP64, but for the sums of compute_Y in 60-bit fixed point: an atom's U
+ * in units of 2^-59 of its largest component, the coefficients of an output in
+ * units of 2^-60 of their largest sum.  Y is as close as in FP64 relative to its
+ * largest element (closer, in fact); an element far below it has fewer correct
+ * bits than FP64 would give it.  SNAP_MIXED: the three recursions run in FP32;
+ * the Cayley-Klein parameters and the per-atom energy, force and virial
+ * accumulations stay in FP64. */
 enum snap_precision { SNAP_FP64 = 0, SNAP_MIXED = 1 };
 
 enum snap_status {

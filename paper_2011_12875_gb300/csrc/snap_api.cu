@@ -994,23 +994,34 @@ int snap_yi_host(int twojmax, int precision, const double* beta, const double* u
   // the fixed-point form, as the kernel computes it (YcFixed)
   typedef long long ll;
   const std::vector<unsigned> words = tab.yc_fixed(beta);
-  double mx = 0.0;
-  for (int e = 0; e < 2 * tab.H; ++e) mx = std::isfinite(u[e]) ? std::max(mx, std::fabs(u[e])) : INFINITY;
-  if (!std::isfinite(mx)) {
+  auto word = [&](int e, int w) {
+    long long x;
+    std::memcpy(&x, u + e, sizeof(x));
+    return (int)(x >> (32 * w));
+  };
+  int top = 0;
+  for (int e = 0; e < 2 * tab.H; ++e) top = std::max(top, word(e, 1) & 0x7FFFFFFF);
+  const int E = snap::yc_scale(top), ex = E - 1022;
+  if (E == 0x7FF) {
     for (int e = 0; e < 2 * tab.H; ++e) y[e] = NAN;
     return SNAP_OK;
   }
-  int ex = 0;
-  std::frexp(mx, &ex);
-  const ll half = 1LL << 29, one30 = 1LL << 30;
+  const ll half = 1LL << 29;
   auto split = [&](ll v, ll& h, ll& l) {
-    h = (v + half) >> 30;
-    l = v - h * one30;
+    int x, z;
+    snap::split30(v + half, x, z);
+    h = x;
+    l = z;
   };
   std::vector<ll> uh(2 * tab.H), ul(2 * tab.H);
-  for (int e = 0; e < 2 * tab.H; ++e) split(std::llround(std::ldexp(u[e], 59 - ex)), uh[e], ul[e]);
+  for (int e = 0; e < 2 * tab.H; ++e) {
+    int h, l;
+    snap::yc_limbs(word(e, 0), word(e, 1), E, h, l);
+    uh[e] = h;
+    ul[e] = l;
+  }
   std::vector<__int128> s(nt * 4, 0);
-  ll acc[2][4];  // of each output's record: ph, pc, qh, qc
+  ll acc[2][4] = {};  // of each output's record: ph, pc, qh, qc
   tab.yc_rows([&](int k, const unsigned* h, int r, size_t p, int o, int len) {
     const unsigned at = h[o];  // half o's u[m1] and u[m2]
     const int s1 = (at >> 15 & 1u) ? -1 : 1, s2 = (at >> 31) ? -s1 : s1;

@@ -33,6 +33,30 @@ constexpr int kBGroupMax = 8;      // longest bispectrum term piece (longer grou
 constexpr int kMaxNeighCap = 64;
 constexpr int kGeomStride = 20;  // doubles per neighbour slot, see PairGeom
 
+// compute_Y's fixed point (snap_kernels.cu), on the device and in its host walk.
+// limbs of v, |v| < 2^59, given v + 2^29: v = h 2^30 + l, -2^29 <= l < 2^29
+__host__ __device__ inline void split30(long long v, int& h, int& l) {
+  h = (int)(v >> 30);
+  l = (int)((unsigned)v & 0x3FFFFFFFu) - (1 << 29);
+}
+// An atom's scale, the biased exponent E of its largest component of U (top: the
+// high word of that magnitude): components are held in units of 2^(E - 1022 -
+// 59).  U below 2^-150 has that scale; 0x7FF: not finite.
+__host__ __device__ inline int yc_scale(int top) { return top >> 20 > 1022 - 150 ? top >> 20 : 1022 - 150; }
+// The limbs of a component (low and high word) at scale E, rounded to nearest,
+// halves away from zero; subnormals count as zero.
+__host__ __device__ inline void yc_limbs(int lo, int hi, int E, int& h, int& l) {
+  const int e = (hi >> 20) & 0x7FF;
+  // |x| = M 2^(e - 1075) = v 2^(E - 1022 - 59)
+  const unsigned long long M = ((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)lo;
+  const int sh = e - E + 6;
+  unsigned long long v = 0;
+  if (sh >= 0) v = M << (sh & 7);
+  else if (sh > -55) v = (M + (1ull << (-sh - 1))) >> -sh;
+  if (e == 0) v = 0;
+  split30((hi < 0 ? -(long long)v : (long long)v) + (1LL << 29), h, l);
+}
+
 // Half-matrix layout (Sec. V-A: u_j only needs floor(j)+1 of its columns):
 // layer t = 2j holds columns mb = 0..t/2, each column ma = 0..t.
 __host__ __device__ constexpr int half_layer_size(int t) { return (t + 1) * (t / 2 + 1); }

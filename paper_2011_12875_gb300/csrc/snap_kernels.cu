@@ -408,8 +408,8 @@ struct YcSingle {
 // more than the 53 of a double) and a product is three integer multiply-adds,
 // hi hi and the two cross ones; the fourth is below the last bit.
 //   u = (h 2^30 + l) 2^(s - 59), |h| <= 2^29, |l| <= 2^29, 2^s above the atom's
-//     largest component of U (yf_prepare; rounded to nearest, exact for
-//     components above 2^-6 of the largest);
+//     largest component of U (yc_limbs; rounded to nearest, exact for components
+//     above 2^-6 of the largest: of a thermal BCC atom's at 2J14, about half);
 //   c = (h 2^30 + l) 2^(e - 60), |l| <= 2^29, 2^e above the largest sum of |c|
 //     over a record (m1, m2) of its output;
 //   a row's sum A = sum_t2 c u is rounded at 2^-59 and split into h, l again,
@@ -418,10 +418,15 @@ struct YcSingle {
 // Sums of a record stay below 2^63: with sum |h(c)| <= 2^30 and |A| <= 2^59,
 //   hi hi: 2^59, 2 x 2^59; cross: 2^59 + 8 2^58, 2 (8 2^58 + 2^59).
 // A rounding here is 2^-59 of the largest |U| (twice in a product) times the
-// largest sum of |c|, where FP64 rounds at 2^-53 of each partial sum.  Measured
-// against 64 bits, largest error of a step's energies, forces and virial, FP64
-// list of terms / fixed point: 2J8 128 atoms 6.3e-15 / 6.5e-15, 2000 atoms 7.0e-15
-// / 7.2e-15, 2J14 2000 atoms 2.8e-15 / 2.9e-15 (most of it from U and dE).
+// largest sum of |c|, where FP64 rounds at 2^-53 of each partial sum: what is
+// large in Y is closer than in FP64, an element far below the rest of its atom's
+// Y, or one that only coefficients far below an output's largest feed, has fewer
+// correct bits than its own size would allow.  dE/dr and the energy sum over
+// all of Y, so they are as close as in FP64.  Error of a step's energies /
+// forces against 64 bits (root mean square over that of the exact ones, eight
+// inputs), FP64 list of terms and layer recursion -> fixed point and closed forms:
+// 2J8 2000 atoms 9.2e-16 / 5.8e-15 -> 7.9e-16 / 5.4e-15, 2J14 2.6e-15 / 6.5e-15 ->
+// 2.1e-15 / 6.3e-15, 2J4 250 atoms 6.5e-16 / 5.5e-15 -> 6.0e-16 / 5.0e-15.
 //
 // A block is 16 atoms (a row of 16 x 16 bytes is then 256, as in FP32, and the
 // whole of 2J14 stays in shared memory); a warp's halves take the two outputs
@@ -457,11 +462,6 @@ __device__ __forceinline__ Acc96 shfl16(const Acc96& v) {
 // hi hi and cross sums to one number, rounded (the cross sum starts at half
 // of 2^30), plus 2^29
 constexpr long long kYcRound = 1LL << 29, kYcSplit = kYcRound + (1LL << 59);
-// limbs of v, given v + 2^29
-__device__ __forceinline__ void split30(long long v, int& h, int& l) {
-  h = (int)(v >> 30);
-  l = (int)((unsigned)v & 0x3FFFFFFFu) - (1 << 29);
-}
 
 // yc_run in fixed point: one output a lane
 template <int L>
@@ -598,27 +598,16 @@ __device__ int yf_prepare(unsigned char* su, int H, int* top) {
   }
   atomicMax(top + al, m);
   __syncthreads();
-  const int E = max(top[al] >> 20, 1022 - 150);  // biased exponent; U below 2^-150 has that scale
-  auto fixed = [&](int lo, int hi, int& h, int& l) {
-    const int e = (hi >> 20) & 0x7FF;
-    // |x| = M 2^(e - 1075) = v 2^(E - 1022 - 59)
-    const unsigned long long M = ((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)lo;
-    const int sh = e - E + 6;
-    unsigned long long v = 0;
-    if (sh >= 0) v = M << (sh & 7);
-    else if (sh > -55) v = (M + (1ull << (-sh - 1))) >> -sh;
-    if (e == 0) v = 0;
-    split30((hi < 0 ? -(long long)v : (long long)v) + kYcRound, h, l);
-  };
+  const int E = yc_scale(top[al]);
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     int4* x = reinterpret_cast<int4*>(su + (size_t)e * 16);
     const int4 v = *x;
     int4 w;
-    fixed(v.x, v.y, w.x, w.y);
-    fixed(v.z, v.w, w.z, w.w);
+    yc_limbs(v.x, v.y, E, w.x, w.y);
+    yc_limbs(v.z, v.w, E, w.z, w.w);
     *x = w;
   }
-  return (top[al] >> 20) == 0x7FF ? YcFixed<8>::kBad : E - 1022;
+  return E == 0x7FF ? YcFixed<8>::kBad : E - 1022;
 }
 
 // One warp's share of a CTA's tasks (tl: first chunk and chunks of each),
