@@ -223,9 +223,9 @@ int upload_yrec(snap_ctx* c) {
   if (rc) return rc;
   // the records of the warp-per-atom layout
   auto word = [&](unsigned w) -> unsigned {
-    const unsigned e1 = w & 1023u, e2 = (w >> 10) & 1023u, c1 = (w >> 20) & 1u, c2 = (w >> 21) & 1u;
-    const unsigned ge = (w >> 23) & 1u, oe = (w >> 22) & 1u;
-    return (e2 << 8) | (e1 << 18) | (ge << 28) | (oe << 29) | (c1 << 30) | (c2 << 31);
+    const unsigned H = (unsigned)c->tab.H;
+    const unsigned e1 = (w & 1023u) + ((w >> 20) & 1u) * H, e2 = ((w >> 10) & 1023u) + ((w >> 21) & 1u) * H;
+    return e1 | e2 << 11 | ((w >> 23) & 1u ? snap::kYaGroup : 0u);
   };
   if (c->precision == SNAP_MIXED) {
     std::vector<snap::YRec<float>> r(n);

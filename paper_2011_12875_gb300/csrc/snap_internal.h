@@ -267,9 +267,9 @@ struct YiGeometry {
   int nblk, split, threads;
   size_t smem;
 };
-// Term record word of the warp-per-atom layout: bits 8-17 the second factor's
-// element, 18-27 the first's, bit 28 ends a group, 29 an output, 30 / 31
-// conjugate the first / second factor.
+// The warp-per-atom layout's term record word ends a group (the rest of the
+// word: yi_atom_kernel).
+constexpr unsigned kYaGroup = 1u << 28;
 YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves, int ntasks);
 
 // End of an evaluation: flags[0..3] into the host-mapped status words

@@ -768,9 +768,11 @@ __global__ void __launch_bounds__(P::kWarps * 32, LM <= 5 ? 2 : 1) yc_kernel(Wor
 // decreasing term count, snake order, so their loads balance); each lane walks
 // its outputs' term records, grouped by their first factor:
 //   Y += U_e1 * sum_k coef_k U_e2,k
-// (a word: two element offsets, conjugation flags, end-of-group and
-// end-of-output bits; and the coefficient).
+// (a word: the two elements' places in the [2][H] block, the first factor's in
+// bits 0-10 and the second's in 11-21, and kYaGroup where a group ends; and the
+// coefficient).
 constexpr int kYaWarps = 8;
+constexpr int kYaSum = 16;
 
 template <typename R>
 __global__ void __launch_bounds__(kYaWarps * 32) yi_atom_kernel(WorkArgs a) {
@@ -796,41 +798,59 @@ __global__ void __launch_bounds__(kYaWarps * 32) yi_atom_kernel(WorkArgs a) {
     if (o < 0) break;
     YAcc<R> y;
     y.re = y.im = y.ar = y.ai = R(0);
-    // every 16 groups are summed by themselves and added up by Kahan's sum (a
-    // long FP32 sum is further off)
+    // FP32: what every 4 kYaSum records have added is put into a compensated sum
+    // (a long FP32 sum is further off), on all lanes at the same record, and the
+    // records are taken four at a time, their loads together.  Bound by the loads'
+    // latency; compute_Y, 54 atoms, 2J8 / 2J14: 98 / 2430 us in FP32 (one long sum,
+    // record by record: 90 / 2530; compensated at each lane's own groups' ends: 186 /
+    // 4880), 455 / 12100 in FP64.
     R sr = R(0), si = R(0), er = R(0), ei = R(0);
     auto add = [](R& s, R& e, R x) {
       const R v = x - e, t = s + v;
       e = (t - s) - v;
       s = t;
     };
-    int groups = 0;
-    const int q1 = a.yfirst[o + 1];
-    for (int q = a.yfirst[o]; q < q1; ++q) {
-      const unsigned w = rec[q].w;
-      const R c = rec[q].c;
-      // elements of the factors in the [2][H] block: the staged-conjugate
-      // record format indexes it directly, the other one sets the sign bits
-      const int e2 = (int)((w >> 8) & 1023u) + (int)(w >> 31) * H;
-      const cx<R> u2 = ua[e2];
+    auto term = [&](unsigned w, R c, cx<R> u2) {
       y.ar += c * u2.re;
       y.ai += c * u2.im;
-      if (w & (1u << 28)) {
-        const int e1 = (int)((w >> 18) & 1023u) + (int)((w >> 30) & 1u) * H;
-        const cx<R> u1 = ua[e1];
+      if (w & kYaGroup) {
+        const cx<R> u1 = ua[w & 2047u];
         y.re = fmr(-u1.im, y.ai, fmr(u1.re, y.ar, y.re));
         y.im = fmr(u1.im, y.ar, fmr(u1.re, y.ai, y.im));
         y.ar = R(0);
         y.ai = R(0);
-        if ((++groups & 15) == 0) {
-          add(sr, er, y.re);
-          add(si, ei, y.im);
-          y.re = y.im = R(0);
-        }
+      }
+    };
+    int q = a.yfirst[o], n = 0;
+    const int q1 = a.yfirst[o + 1];
+    for (; q + 4 <= q1; q += 4) {
+      unsigned w[4];
+      R c[4];
+      cx<R> u2[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        w[j] = rec[q + j].w;
+        c[j] = rec[q + j].c;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) u2[j] = ua[(w[j] >> 11) & 2047u];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) term(w[j], c[j], u2[j]);
+      if (sizeof(R) == 4 && ++n == kYaSum) {
+        n = 0;
+        add(sr, er, y.re);
+        add(si, ei, y.im);
+        y.re = y.im = R(0);
       }
     }
-    add(sr, er, y.re);
-    add(si, ei, y.im);
+    for (; q < q1; ++q) term(rec[q].w, rec[q].c, ua[(rec[q].w >> 11) & 2047u]);
+    if (sizeof(R) == 4) {
+      add(sr, er, y.re);
+      add(si, ei, y.im);
+    } else {
+      sr = y.re;
+      si = y.im;
+    }
     Yg[(long)o * 32] = mk<R>(sr, si);
   }
 }
