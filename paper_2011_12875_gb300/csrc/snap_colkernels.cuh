@@ -16,7 +16,6 @@
 // unit per working precision.
 #pragma once
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "snap_geom.cuh"
@@ -506,23 +505,13 @@ __global__ void __launch_bounds__(64, ui_min_ctas<R, J2>()) tan_col_kernel(WorkA
   }
 }
 
-template <typename K>
-inline cudaError_t col_allow_smem(K kernel, size_t bytes) {
-  // the default 48 KB limit covers static and dynamic shared memory together
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  if (bytes + fa.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename R, int J2>
 cudaError_t launch_ui_col_t(const WorkArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
   using UP = UiPlan<R, J2>;
   if (a.H != UP::HH) return cudaErrorInvalidValue;
   const size_t smem = (size_t)UP::A * (UP::Q * UP::warp_bytes + sizeof(R) * 5 * (size_t)a.K);
-  cudaError_t e = col_allow_smem(ui_col_kernel<R, J2>, smem);
+  cudaError_t e = allow_smem(ui_col_kernel<R, J2>, smem);
   if (e != cudaSuccess) return e;
   return launch_k(ui_col_kernel<R, J2>, dim3((unsigned)((a.n + UP::A - 1) / UP::A)), dim3(UP::A * UP::Q * 32),
                   smem, s, a);
@@ -537,12 +526,12 @@ cudaError_t launch_neigh_u_t(const NeighArgs& na, const WorkArgs& a, int ncta, c
   if (a.H != UP::HH) return cudaErrorInvalidValue;
   const size_t smem = (size_t)2 * (UP::Q * UP::warp_bytes + sizeof(R) * 5 * (size_t)a.K);
   if (ncta > 0) {
-    cudaError_t e = col_allow_smem(neigh_u_kernel<R, J2, true>, smem);
+    cudaError_t e = allow_smem(neigh_u_kernel<R, J2, true>, smem);
     if (e != cudaSuccess) return e;
     return launch_k(neigh_u_kernel<R, J2, true>, dim3((unsigned)ncta), dim3(NuShape<true>::NW * 32), smem, s, na,
                     a);
   }
-  cudaError_t e = col_allow_smem(neigh_u_kernel<R, J2, false>, smem);
+  cudaError_t e = allow_smem(neigh_u_kernel<R, J2, false>, smem);
   if (e != cudaSuccess) return e;
   return launch_k(neigh_u_kernel<R, J2, false>, dim3((unsigned)((a.n + 1) / 2)), dim3(NuShape<false>::NW * 32),
                   smem, s, na, a);
@@ -554,7 +543,7 @@ cudaError_t launch_tan_col_t(const WorkArgs& a, const double* g, void* dU, cudaS
   using UP = UiPlan<R, J2>;
   if (a.H != UP::HH) return cudaErrorInvalidValue;
   const size_t smem = (size_t)UP::A * (UP::Q * UP::warp_bytes + sizeof(R) * 10 * (size_t)a.K);
-  cudaError_t e = col_allow_smem(tan_col_kernel<R, J2>, smem);
+  cudaError_t e = allow_smem(tan_col_kernel<R, J2>, smem);
   if (e != cudaSuccess) return e;
   return launch_k(tan_col_kernel<R, J2>, dim3((unsigned)((a.n + UP::A - 1) / UP::A)), dim3(UP::A * UP::Q * 32),
                   smem, s, a, g, dU);

@@ -5,6 +5,8 @@
 #include <stdint.h>
 
 #include <cmath>
+#include <mutex>
+#include <unordered_map>
 
 namespace snap {
 
@@ -18,6 +20,39 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
   return cudaGetLastError();
 }
 #endif
+
+// Shared memory of a CTA: the most there is, and what a launch may use without
+// being allowed to.
+constexpr size_t kSmemMax = 227 * 1024, kSmemFree = 48 * 1024;
+
+// Allows a launch of `kernel` with `bytes` of dynamic shared memory.  The limit
+// is an attribute of the function, which every context and host thread shares,
+// so it is always set to the same value, the most the kernel can have: set to a
+// launch's own bytes, one thread could lower it between another's setting it
+// and launching.
+inline cudaError_t allow_smem_of(const void* kernel, size_t bytes) {
+  size_t fixed;  // static shared memory, looked up once
+  {
+    static std::mutex mu;
+    static std::unordered_map<const void*, size_t> seen;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = seen.find(kernel);
+    if (it == seen.end()) {
+      cudaFuncAttributes fa;
+      const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+      if (e != cudaSuccess) return e;
+      it = seen.emplace(kernel, fa.sharedSizeBytes).first;
+    }
+    fixed = it->second;
+  }
+  if (bytes + fixed <= kSmemFree) return cudaSuccess;
+  if (bytes + fixed > kSmemMax) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemMax - fixed));
+}
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t bytes) {
+  return allow_smem_of(reinterpret_cast<const void*>(kernel), bytes);
+}
 
 constexpr int kMaxTwoJ = 14;
 constexpr int kYcChunk = 256;  // words of a compute_Y stream chunk (snap_tables.h)

@@ -8,8 +8,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <utility>
 
 #include "snap_geom.cuh"
@@ -1334,16 +1332,6 @@ __global__ void __launch_bounds__(kFThreads) force_kernel(WorkArgs a) {
   if (lane % 4 == 0) wv[w][lane / 4] = xs;
   __syncthreads();
   if (tid < 6) a.virial[tid] = (wv[0][tid] + wv[1][tid]) + (wv[2][tid] + wv[3][tid]);
-}
-
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes) {
-  // the default 48 KB limit covers static and dynamic shared memory together
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  if (bytes + fa.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 }  // namespace

@@ -539,16 +539,6 @@ inline DePlan de_plan(int n, int maxcnt, int nsm, int col_warps, int force_A) {
   return best;
 }
 
-template <typename K>
-inline cudaError_t allow_smem(K kernel, size_t bytes) {
-  // the default 48 KB limit covers static and dynamic shared memory together
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  if (bytes + fa.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename R, int J2, int SPLIT>
 cudaError_t launch_de_split(const WorkArgs& a, const DePlan& p, cudaStream_t s) {
   const long nitems = (a.n + p.A - 1) / p.A;

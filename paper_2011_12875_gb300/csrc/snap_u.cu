@@ -340,16 +340,6 @@ __global__ void __launch_bounds__(BATCH ? 256 : 128) neigh_geom_kernel(NeighArgs
   });
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes) {
-  // the default 48 KB limit covers static and dynamic shared memory together
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  if (bytes + fa.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 template <typename R>
