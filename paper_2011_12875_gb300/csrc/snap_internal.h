@@ -197,6 +197,7 @@ __host__ __device__ constexpr int pair_key(int k, int ix, int iy, int iz, long n
              : -1;
 }
 
+// What a kernel reads stands together: every CTA fetches its lines of it.
 struct WorkArgs {
   int n, K, twojmax, H, lmax;
   double rcut, rfac0, rmin0, wself, beta0;
@@ -218,7 +219,6 @@ struct WorkArgs {
   // Ulisttot and Y: complex (re, im interleaved), AoSoA [ceil(N/32)][H][32]
   void* U;
   void* Y;
-  void* Y2;  // compute_Y: the second halves of split sums (as Y)
   double* dedr;
   double* vatom;   // per-atom virial [N][6] (batch mode) or nullptr
   double* energy;
@@ -230,20 +230,7 @@ struct WorkArgs {
   // last CTA writes flags[0..3] to this host-mapped copy and zeroes the flags
   int* hflags;
   const int* half_tmm;
-  // compute_Y's tables (HostTables::yc_*); yc_bins for yc_split CTAs a block
-  const int* yc_bins;
-  int yc_split;
-  const int* yc_slot;
-  const int* yc_task;
-  const unsigned* yc_stream;
-  int yc_ntask;
-  int yi_layout;          // 0: warp of 32 atoms (AoSoA), 1: warp per atom
-  // warp-per-atom layout: term records (snap_tables.cpp), [H+1] first term of
-  // each output element, [32][ysched_m] outputs of each lane
-  const void* yrec;
-  const int* yfirst;
-  const int* ysched;
-  int ysched_m;
+  const void* hscale;  // R [H]: S_t(ma, mb) of the scaled recursion (u = S v)
   int nsm;
   int col_warps;  // fused dE: an SM with fewer than 2 col_warps batches shares them (tunable)
   int de_maxcnt;  // neighbour count the fused dE launch is planned for (last seen maximum, else K)
@@ -263,7 +250,20 @@ struct WorkArgs {
   const int* bpart;         // [nbparts+1] first component of each CTA's run
   int nbparts, bmaxchunks, bmaxterms;  // runs, most chunks and most terms of one run
   double* B;              // [N][ncoeff]
-  const void* hscale;  // R [H]: S_t(ma, mb) of the scaled recursion (u = S v)
+  // compute_Y's tables (HostTables::yc_*); yc_bins for yc_split CTAs a block
+  void* Y2;  // the second halves of split sums (as Y)
+  const int* yc_bins;
+  const int* yc_slot;
+  const int* yc_task;
+  const unsigned* yc_stream;
+  int yc_split, yc_ntask;
+  int yi_layout;          // 0: warp of 32 atoms (AoSoA), 1: warp per atom
+  // warp-per-atom layout: term records (snap_tables.cpp), [H+1] first term of
+  // each output element, [32][ysched_m] outputs of each lane
+  int ysched_m;
+  const void* yrec;
+  const int* yfirst;
+  const int* ysched;
   // closed-form u of a pair (snap_pairs.cuh, HostTables::pair_*), per step
   const unsigned* pair_idx;
   const void* pair_scale;  // R: norm x weight
