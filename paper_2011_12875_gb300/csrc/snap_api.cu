@@ -107,8 +107,7 @@ struct snap_ctx {
   double* d_dedr = nullptr;
   void* d_U = nullptr;  // complex AoSoA [ceil(N/32)][H][32]
   void* d_Y = nullptr;
-  void* d_Y2 = nullptr;
-  void* d_dU = nullptr;  // tangent of U (bispectrum derivative)
+  void* d_dU = nullptr;  // tangent of U (bispectrum derivative); compute_Y's second halves (WorkArgs::Y2)
   long long generation = 0;  // number of evaluations enqueued
   snap::WorkArgs last_args;   // arguments of the last evaluation (weighted gather)
   bool have_last = false;
@@ -286,7 +285,6 @@ void free_workspace(snap_ctx* c) {
   dfree(c->d_dedr);
   dfree(c->d_U);
   dfree(c->d_Y);
-  dfree(c->d_Y2);
   dfree(c->d_dU);
   dfree(c->d_vpart);
   c->cap_nk = 0;
@@ -314,7 +312,6 @@ int ensure_workspace(snap_ctx* c, int n, int K) {
   SNAP_CUDA(c, cudaMalloc(&c->d_dedr, sizeof(double) * 3 * nkcap));
   SNAP_CUDA(c, cudaMalloc(&c->d_U, uy));
   SNAP_CUDA(c, cudaMalloc(&c->d_Y, uy));
-  SNAP_CUDA(c, cudaMalloc(&c->d_Y2, uy));
   SNAP_CUDA(c, cudaMalloc(&c->d_dU, uy));
   // lanes past the last atom read zeros in compute_Y
   SNAP_CUDA(c, cudaMemset(c->d_U, 0, uy));
@@ -483,7 +480,7 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
   a.geom = c->d_geom;
   a.U = c->d_U;
   a.Y = c->d_Y;
-  a.Y2 = c->d_Y2;
+  a.Y2 = c->d_dU;  // no evaluation has both
   a.dedr = c->d_dedr;
   a.vpart = c->d_vpart;
   a.flags = c->d_flags;

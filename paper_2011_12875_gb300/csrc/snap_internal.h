@@ -251,7 +251,7 @@ struct WorkArgs {
   int nbparts, bmaxchunks, bmaxterms;  // runs, most chunks and most terms of one run
   double* B;              // [N][ncoeff]
   // compute_Y's tables (HostTables::yc_*); yc_bins for yc_split CTAs a block
-  void* Y2;  // the second halves of split sums (as Y)
+  void* Y2;  // the second halves of split sums (as Y; the tangent's buffer)
   const int* yc_bins;
   const int* yc_slot;
   const int* yc_task;
