@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(P::kWarps * 32, LM <= 5 ? 2 : 1) yc_kernel(Wor
 // bits 0-10 and the second's in 11-21, and kYaGroup where a group ends; and the
 // coefficient).
 constexpr int kYaWarps = 8;
-constexpr int kYaSum = 16;
+constexpr int kYaSum = 4;
 
 template <typename R>
 __global__ void __launch_bounds__(kYaWarps * 32) yi_atom_kernel(WorkArgs a) {
@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(kYaWarps * 32) yi_atom_kernel(WorkArgs a) {
     if (o < 0) break;
     YAcc<R> y;
     y.re = y.im = y.ar = y.ai = R(0);
-    // FP32: what every 4 kYaSum records have added is put into a compensated sum
+    // FP32: what every 4 kYaSum = 16 records have added is put into a compensated sum
     // (a long FP32 sum is further off), on all lanes at the same record, and the
     // records are taken four at a time, their loads together.  Bound by the loads'
     // latency; compute_Y, 54 atoms, 2J8 / 2J14: 98 / 2430 us in FP32 (one long sum,
