@@ -212,15 +212,11 @@ int upload_inplace(snap_ctx* c, T** dst, const std::vector<T>& v) {
   return SNAP_OK;
 }
 
-// compute_Y term records (index word + coefficient in the working precision)
-int upload_yrec(snap_ctx* c) {
+// Term records of the warp-per-atom compute_Y (index word + coefficient in the
+// working precision).
+int upload_terms(snap_ctx* c) {
   const std::vector<double> coef = c->tab.term_coef(c->beta.data());
   const size_t n = c->tab.terms.size();
-  // the class stream
-  int rc = upload_inplace(c, &c->d_yc_stream, c->precision == SNAP_MIXED ? c->tab.yc_stream(c->beta.data())
-                                                                         : c->tab.yc_fixed(c->beta.data()));
-  if (rc) return rc;
-  // the records of the warp-per-atom layout
   auto word = [&](unsigned w) -> unsigned {
     const unsigned H = (unsigned)c->tab.H;
     const unsigned e1 = (w & 1023u) + ((w >> 20) & 1u) * H, e2 = ((w >> 10) & 1023u) + ((w >> 21) & 1u) * H;
@@ -241,6 +237,24 @@ int upload_yrec(snap_ctx* c) {
     r[k].c = coef[k];
   }
   return upload_inplace(c, reinterpret_cast<snap::YRec<double>**>(&c->d_yrec), r);
+}
+
+// What the warp-per-atom layout needs, when it is first chosen.
+int ensure_terms(snap_ctx* c) {
+  if (!c->tab.terms.empty()) return SNAP_OK;
+  c->tab.build_terms();
+  int rc = upload(c, &c->d_yfirst, c->tab.term_out_first);
+  if (!rc) rc = upload(c, &c->d_ysched, c->tab.lane_outputs(32, &c->ysched_m));
+  if (!rc) rc = upload_terms(c);
+  if (rc) c->tab.terms.clear();
+  return rc;
+}
+
+// The tables that depend on beta.
+int upload_beta(snap_ctx* c) {
+  const int rc = upload_inplace(c, &c->d_yc_stream, c->precision == SNAP_MIXED ? c->tab.yc_stream(c->beta.data())
+                                                                               : c->tab.yc_fixed(c->beta.data()));
+  return rc || c->tab.terms.empty() ? rc : upload_terms(c);
 }
 
 // bispectrum term records (coefficients do not depend on beta), in both
@@ -1175,10 +1189,8 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
     return SNAP_ERR_CUDA;
   }
   int rc = upload(c, &c->d_half_tmm, c->tab.half_tmm);
-  if (!rc) rc = upload(c, &c->d_yfirst, c->tab.term_out_first);
   if (!rc) rc = upload(c, &c->d_yc_slot, c->tab.yc_slot);
   if (!rc) rc = upload(c, &c->d_yc_task, c->tab.yc_task);
-  if (!rc) rc = upload(c, &c->d_ysched, c->tab.lane_outputs(32, &c->ysched_m));
   if (!rc) rc = upload_r(c, &c->d_hscale, c->tab.half_scale);
   if (!rc) rc = upload(c, &c->d_pair_idx, c->tab.pair_idx);
   const bool fp64 = precision == SNAP_FP64;
@@ -1192,7 +1204,7 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
     if (!rc) rc = upload(c, &c->d_pair_fix, c->tab.pair_fix);
   }
   if (!rc) rc = upload(c, &c->d_u_units, c->tab.u_units);
-  if (!rc) rc = upload_yrec(c);
+  if (!rc) rc = upload_beta(c);
   if (!rc) rc = upload_brec(c);
   if (!rc) rc = upload(c, &c->d_bchunk_term, c->tab.bchunk_term);
   if (!rc) rc = upload(c, &c->d_bchunk_runs, c->tab.bchunk_runs);
@@ -1217,7 +1229,7 @@ int snap_set_beta(snap_ctx* c, const double* beta) {
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
   }
-  return upload_yrec(c);
+  return upload_beta(c);
 }
 
 int snap_set_neigh_cap(snap_ctx* c, int cap) {
@@ -1441,6 +1453,10 @@ int snap_set_tuning(snap_ctx* c, int col_warps, int yi_waves, int yi_layout) {
     return fail(c, SNAP_ERR_ARG, "col_warps must be 2, 4 or 8");
   if (yi_waves < 1 || yi_waves > 8) return fail(c, SNAP_ERR_ARG, "yi_waves must be in 1..8");
   if (yi_layout != 0 && yi_layout != 1) return fail(c, SNAP_ERR_ARG, "yi_layout must be 0 or 1");
+  if (yi_layout == 1) {
+    const int rc = ensure_terms(c);
+    if (rc) return rc;
+  }
   if (c->col_warps != col_warps || c->yi_waves != yi_waves || c->yi_layout != yi_layout) {
     c->col_warps = col_warps;
     c->yi_waves = yi_waves;

@@ -138,6 +138,20 @@ void orient_by_cover(std::vector<unsigned>& terms, size_t first) {
   }
 }
 
+// Half-layout place of element (xa, xb) of layer tt: past the stored columns its
+// mirror, conjugated, with the sign.
+void half_elem(int tt, int xa, int xb, int& idx, int& conj, double& sgn) {
+  if (2 * xb <= tt) {
+    idx = half_base(tt) + xb * (tt + 1) + xa;
+    conj = 0;
+    sgn = 1.0;
+  } else {
+    idx = half_base(tt) + (tt - xb) * (tt + 1) + (tt - xa);
+    conj = 1;
+    sgn = ((xa + xb) & 1) ? -1.0 : 1.0;
+  }
+}
+
 }  // namespace
 
 void HostTables::build(int J2) {
@@ -191,135 +205,6 @@ void HostTables::build(int J2) {
         }
         ztrip.push_back(z);
       }
-
-  // compute_Y term list.  For every half-layout output element (t, ma, mb)
-  // of Y, in output order, every nonzero term of every triple (t1 >= t2)
-  // with output rank t:
-  //   Y_t[ma][mb] += betaw * C(ma1, ma2) C(mb1, mb2) U_t1[ma1][mb1] U_t2[ma2][mb2],
-  // ma2 = ma + d - ma1, mb2 = mb + d - mb1, d = (t1+t2-t)/2.  An element of U
-  // past the stored half columns is (-1)^(ma+mb) conj of its mirror, so each
-  // term stores the two half-layout indices, two conjugation flags, and a
-  // coefficient with the signs, the CG product and betaw folded in.
-  terms.clear();
-  term_cg.clear();
-  term_trip.clear();
-  term_out_first.clear();
-  auto half_elem = [&](int tt, int xa, int xb, int& idx, int& conj, double& sgn) {
-    if (2 * xb <= tt) {
-      idx = half_base(tt) + xb * (tt + 1) + xa;
-      conj = 0;
-      sgn = 1.0;
-    } else {
-      idx = half_base(tt) + (tt - xb) * (tt + 1) + (tt - xa);
-      conj = 1;
-      sgn = ((xa + xb) & 1) ? -1.0 : 1.0;
-    }
-  };
-  // triples grouped by output rank
-  std::vector<std::vector<int>> by_t(J2 + 1);
-  std::unordered_map<unsigned long long, size_t> same_layer;  // (triple, word) -> term
-  for (int q = 0; q < (int)ztrip.size(); ++q) by_t[ztrip[q].t].push_back(q);
-  for (int t = 0; t <= J2; ++t)
-    for (int mb = 0; 2 * mb <= t; ++mb)
-      for (int ma = 0; ma <= t; ++ma) {
-        const size_t first = terms.size();
-        same_layer.clear();
-        // Below the centre of the middle column (2 mb = t, ma > mb) Y is the
-        // mirror of the element above it, and the contractions that read Y
-        // (energy, dE/dr) give it weight 0: one zero term there (Y = 0), and
-        // the host export fills in the mirror.
-        const bool mirrored = 2 * mb == t && ma > mb;
-        for (int q : by_t[t]) {
-          if (mirrored) break;
-          const ZTrip& z = ztrip[q];
-          const int dl = (z.t1 + z.t2 - t) / 2;
-          for (int mb1 = std::max(0, mb + dl - z.t2); mb1 <= std::min(z.t1, mb + dl); ++mb1) {
-            const int mb2 = mb + dl - mb1;
-            const double cb = cg[z.cg_off + mb1 * (z.t2 + 1) + mb2];
-            if (cb == 0.0) continue;
-            for (int ma1 = std::max(0, ma + dl - z.t2); ma1 <= std::min(z.t1, ma + dl); ++ma1) {
-              const int ma2 = ma + dl - ma1;
-              const double ca = cg[z.cg_off + ma1 * (z.t2 + 1) + ma2];
-              if (ca == 0.0) continue;
-              int i1, c1, i2, c2;
-              double s1, s2;
-              half_elem(z.t1, ma1, mb1, i1, c1, s1);
-              half_elem(z.t2, ma2, mb2, i2, c2, s2);
-              // t1 == t2: the term with the factors swapped, (ma2, mb2) as
-              // the first, has the same coefficient and the same product, so
-              // the two are kept as one term, the stored element with the
-              // lower (index, conjugation) first, with the summed coefficient
-              if (z.t1 == z.t2 && (i2 < i1 || (i2 == i1 && c2 < c1))) {
-                std::swap(i1, i2);
-                std::swap(c1, c2);
-              }
-              const unsigned w = (unsigned)i1 | ((unsigned)i2 << 10) | ((unsigned)c1 << 20) |
-                                 ((unsigned)c2 << 21);
-              const double cgp = ca * cb * s1 * s2;
-              if (z.t1 == z.t2) {
-                const auto ins = same_layer.emplace(((unsigned long long)q << 32) | w, terms.size());
-                if (!ins.second) {
-                  term_cg[ins.first->second] += cgp;
-                  continue;
-                }
-              }
-              terms.push_back(w);
-              term_cg.push_back(cgp);
-              term_trip.push_back(q);
-            }
-          }
-        }
-        {  // drop merged terms whose coefficients cancelled exactly
-          size_t o = first;
-          for (size_t k = first; k < terms.size(); ++k)
-            if (term_cg[k] != 0.0) {
-              terms[o] = terms[k];
-              term_cg[o] = term_cg[k];
-              term_trip[o] = term_trip[k];
-              ++o;
-            }
-          terms.resize(o);
-          term_cg.resize(o);
-          term_trip.resize(o);
-        }
-        if (mirrored) {
-          terms.push_back(0u);
-          term_cg.push_back(0.0);
-          term_trip.push_back(by_t[t].front());
-        }
-        orient_by_cover(terms, first);
-        // Group the output's terms by their first factor (index and
-        // conjugation flag, stable): compute_Y then forms
-        //   Y += U_t1[..] * sum_k coef_k U_t2,k[..]
-        // once per group.  Bit 23 ends a group, bit 22 the output; every output has at
-        // least one term: the term of the (t, 0, t) triple, whose
-        // Clebsch-Gordan product is 1, or the zero term of a mirrored output.
-        const size_t cnt = terms.size() - first;
-        if (cnt > 0) {
-          std::vector<size_t> ord(cnt);
-          for (size_t k = 0; k < cnt; ++k) ord[k] = k;
-          auto key = [&](size_t k) { return terms[first + k] & ((1023u) | (1u << 20)); };
-          std::stable_sort(ord.begin(), ord.end(), [&](size_t x, size_t y) { return key(x) < key(y); });
-          std::vector<unsigned> tw(cnt);
-          std::vector<double> tc(cnt);
-          std::vector<int> tq(cnt);
-          for (size_t k = 0; k < cnt; ++k) {
-            tw[k] = terms[first + ord[k]];
-            tc[k] = term_cg[first + ord[k]];
-            tq[k] = term_trip[first + ord[k]];
-          }
-          const unsigned kmask = 1023u | (1u << 20);
-          for (size_t k = 0; k < cnt; ++k) {
-            const bool end = k + 1 == cnt || (tw[k + 1] & kmask) != (tw[k] & kmask);
-            terms[first + k] = tw[k] | (end ? (1u << 23) : 0u);
-            term_cg[first + k] = tc[k];
-            term_trip[first + k] = tq[k];
-          }
-          terms.back() |= (1u << 22);
-        }
-        term_out_first.push_back((int)first);
-      }
-  term_out_first.push_back((int)terms.size());
 
   // Bispectrum term list (descriptor output, Eq. z): for every canonical
   // component l = (t1 >= t2, t >= t1), for every half-layout element (t, ma,
@@ -567,6 +452,126 @@ std::vector<int> HostTables::pair_classes() const {
       st += steps;
     }
   return cls;
+}
+
+void HostTables::build_terms() {
+  // For every half-layout output element (t, ma, mb)
+  // of Y, in output order, every nonzero term of every triple (t1 >= t2)
+  // with output rank t:
+  //   Y_t[ma][mb] += betaw * C(ma1, ma2) C(mb1, mb2) U_t1[ma1][mb1] U_t2[ma2][mb2],
+  // ma2 = ma + d - ma1, mb2 = mb + d - mb1, d = (t1+t2-t)/2.  An element of U
+  // past the stored half columns is (-1)^(ma+mb) conj of its mirror, so each
+  // term stores the two half-layout indices, two conjugation flags, and a
+  // coefficient with the signs, the CG product and betaw folded in.
+  terms.clear();
+  term_cg.clear();
+  term_trip.clear();
+  term_out_first.clear();
+  // triples grouped by output rank
+  std::vector<std::vector<int>> by_t(twojmax + 1);
+  std::unordered_map<unsigned long long, size_t> same_layer;  // (triple, word) -> term
+  for (int q = 0; q < (int)ztrip.size(); ++q) by_t[ztrip[q].t].push_back(q);
+  for (int t = 0; t <= twojmax; ++t)
+    for (int mb = 0; 2 * mb <= t; ++mb)
+      for (int ma = 0; ma <= t; ++ma) {
+        const size_t first = terms.size();
+        same_layer.clear();
+        // Below the centre of the middle column (2 mb = t, ma > mb) Y is the
+        // mirror of the element above it, and the contractions that read Y
+        // (energy, dE/dr) give it weight 0: one zero term there (Y = 0), and
+        // the host export fills in the mirror.
+        const bool mirrored = 2 * mb == t && ma > mb;
+        for (int q : by_t[t]) {
+          if (mirrored) break;
+          const ZTrip& z = ztrip[q];
+          const int dl = (z.t1 + z.t2 - t) / 2;
+          for (int mb1 = std::max(0, mb + dl - z.t2); mb1 <= std::min(z.t1, mb + dl); ++mb1) {
+            const int mb2 = mb + dl - mb1;
+            const double cb = cg[z.cg_off + mb1 * (z.t2 + 1) + mb2];
+            if (cb == 0.0) continue;
+            for (int ma1 = std::max(0, ma + dl - z.t2); ma1 <= std::min(z.t1, ma + dl); ++ma1) {
+              const int ma2 = ma + dl - ma1;
+              const double ca = cg[z.cg_off + ma1 * (z.t2 + 1) + ma2];
+              if (ca == 0.0) continue;
+              int i1, c1, i2, c2;
+              double s1, s2;
+              half_elem(z.t1, ma1, mb1, i1, c1, s1);
+              half_elem(z.t2, ma2, mb2, i2, c2, s2);
+              // t1 == t2: the term with the factors swapped, (ma2, mb2) as
+              // the first, has the same coefficient and the same product, so
+              // the two are kept as one term, the stored element with the
+              // lower (index, conjugation) first, with the summed coefficient
+              if (z.t1 == z.t2 && (i2 < i1 || (i2 == i1 && c2 < c1))) {
+                std::swap(i1, i2);
+                std::swap(c1, c2);
+              }
+              const unsigned w = (unsigned)i1 | ((unsigned)i2 << 10) | ((unsigned)c1 << 20) |
+                                 ((unsigned)c2 << 21);
+              const double cgp = ca * cb * s1 * s2;
+              if (z.t1 == z.t2) {
+                const auto ins = same_layer.emplace(((unsigned long long)q << 32) | w, terms.size());
+                if (!ins.second) {
+                  term_cg[ins.first->second] += cgp;
+                  continue;
+                }
+              }
+              terms.push_back(w);
+              term_cg.push_back(cgp);
+              term_trip.push_back(q);
+            }
+          }
+        }
+        {  // drop merged terms whose coefficients cancelled exactly
+          size_t o = first;
+          for (size_t k = first; k < terms.size(); ++k)
+            if (term_cg[k] != 0.0) {
+              terms[o] = terms[k];
+              term_cg[o] = term_cg[k];
+              term_trip[o] = term_trip[k];
+              ++o;
+            }
+          terms.resize(o);
+          term_cg.resize(o);
+          term_trip.resize(o);
+        }
+        if (mirrored) {
+          terms.push_back(0u);
+          term_cg.push_back(0.0);
+          term_trip.push_back(by_t[t].front());
+        }
+        orient_by_cover(terms, first);
+        // Group the output's terms by their first factor (index and
+        // conjugation flag, stable): compute_Y then forms
+        //   Y += U_t1[..] * sum_k coef_k U_t2,k[..]
+        // once per group.  Bit 23 ends a group, bit 22 the output; every output has at
+        // least one term: the term of the (t, 0, t) triple, whose
+        // Clebsch-Gordan product is 1, or the zero term of a mirrored output.
+        const size_t cnt = terms.size() - first;
+        if (cnt > 0) {
+          std::vector<size_t> ord(cnt);
+          for (size_t k = 0; k < cnt; ++k) ord[k] = k;
+          auto key = [&](size_t k) { return terms[first + k] & ((1023u) | (1u << 20)); };
+          std::stable_sort(ord.begin(), ord.end(), [&](size_t x, size_t y) { return key(x) < key(y); });
+          std::vector<unsigned> tw(cnt);
+          std::vector<double> tc(cnt);
+          std::vector<int> tq(cnt);
+          for (size_t k = 0; k < cnt; ++k) {
+            tw[k] = terms[first + ord[k]];
+            tc[k] = term_cg[first + ord[k]];
+            tq[k] = term_trip[first + ord[k]];
+          }
+          const unsigned kmask = 1023u | (1u << 20);
+          for (size_t k = 0; k < cnt; ++k) {
+            const bool end = k + 1 == cnt || (tw[k + 1] & kmask) != (tw[k] & kmask);
+            terms[first + k] = tw[k] | (end ? (1u << 23) : 0u);
+            term_cg[first + k] = tc[k];
+            term_trip[first + k] = tq[k];
+          }
+          terms.back() |= (1u << 22);
+        }
+        term_out_first.push_back((int)first);
+      }
+  term_out_first.push_back((int)terms.size());
 }
 
 // a vector's byte offset and conjugation (bit 31) in 16 bits

@@ -144,6 +144,8 @@ struct HostTables {
   std::vector<int> yc_bins(int nbins) const;
 
   void build(int twojmax);
+  // the list of terms (terms, term_*), which only the warp-per-atom compute_Y walks
+  void build_terms();
   std::vector<double> beta_weights(const double* beta) const;
   std::vector<double> term_coef(const double* beta) const;
   // outputs dealt to `lanes` lanes in decreasing term count, snake order:
