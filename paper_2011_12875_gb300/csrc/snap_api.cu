@@ -61,6 +61,11 @@ struct snap_ctx {
   int* d_yc_slot = nullptr;  // compute_Y (HostTables::yc_*)
   int* d_yc_task = nullptr;
   unsigned* d_yc_stream = nullptr;
+  snap::YcCoef* d_yc_coef = nullptr;  // for set_beta
+  snap::YcGroup* d_yc_group = nullptr;
+  unsigned long long* d_yc_top = nullptr;
+  double* d_bw = nullptr;
+  int nyc_coef = 0, nyc_group = 0, nyc_chunk = 0;
   void* d_brec = nullptr;
   void* d_brec_cp = nullptr;
   void* d_bscratch = nullptr;  // chunk partials of the bispectrum kernels (when shared memory is short)
@@ -250,11 +255,34 @@ int ensure_terms(snap_ctx* c) {
   return rc;
 }
 
+// compute_Y's stream without its coefficients, and those without beta.
+int upload_stream(snap_ctx* c) {
+  std::vector<snap::YcCoef> coef;
+  std::vector<snap::YcGroup> group;
+  c->tab.yc_list(coef, group);
+  c->nyc_coef = (int)coef.size();
+  c->nyc_group = (int)group.size() - 1;
+  int rc = upload(c, &c->d_yc_stream, c->tab.yc_head);
+  if (!rc) rc = upload(c, &c->d_yc_coef, coef);
+  if (!rc && c->precision == SNAP_FP64) {
+    rc = upload(c, &c->d_yc_group, group);
+    if (!rc) rc = upload(c, &c->d_yc_top, std::vector<unsigned long long>(c->tab.yc_cost.size() * snap::kYcOuts));
+  }
+  c->nyc_chunk = (int)(c->tab.yc_head.size() / snap::kYcChunk);
+  c->tab.drop_stream();
+  return rc;
+}
+
 // The tables that depend on beta.
 int upload_beta(snap_ctx* c) {
-  const int rc = upload_inplace(c, &c->d_yc_stream, c->precision == SNAP_MIXED ? c->tab.yc_stream(c->beta.data())
-                                                                               : c->tab.yc_fixed(c->beta.data()));
-  return rc || c->tab.terms.empty() ? rc : upload_terms(c);
+  int rc = upload_inplace(c, &c->d_bw, c->tab.beta_weights(c->beta.data()));
+  if (rc) return rc;
+  SNAP_CUDA(c, snap::launch_yc_coefs(c->precision == SNAP_FP64, c->d_yc_coef, c->nyc_coef, c->d_yc_group, c->nyc_group,
+                                     c->d_bw, c->d_yc_task, (int)c->tab.yc_cost.size(), c->nyc_chunk, c->d_yc_top,
+                                     c->d_yc_stream, 0));
+  if (!c->tab.terms.empty()) rc = upload_terms(c);
+  SNAP_CUDA(c, cudaStreamSynchronize(0));
+  return rc;
 }
 
 // bispectrum term records (coefficients do not depend on beta), in both
@@ -1204,6 +1232,7 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
     if (!rc) rc = upload(c, &c->d_pair_fix, c->tab.pair_fix);
   }
   if (!rc) rc = upload(c, &c->d_u_units, c->tab.u_units);
+  if (!rc) rc = upload_stream(c);
   if (!rc) rc = upload_beta(c);
   if (!rc) rc = upload_brec(c);
   if (!rc) rc = upload(c, &c->d_bchunk_term, c->tab.bchunk_term);
@@ -1787,6 +1816,10 @@ int snap_destroy(snap_ctx* c) {
   dfree(c->d_yc_slot);
   dfree(c->d_yc_task);
   dfree(c->d_yc_stream);
+  dfree(c->d_yc_coef);
+  dfree(c->d_yc_group);
+  dfree(c->d_yc_top);
+  dfree(c->d_bw);
   dfree(c->d_ysched);
   dfree(c->d_brec);
   dfree(c->d_brec_cp);

@@ -68,6 +68,17 @@ constexpr int kBGroupMax = 8;      // longest bispectrum term piece (longer grou
 constexpr int kMaxNeighCap = 64;
 constexpr int kGeomStride = 20;  // doubles per neighbour slot, see PairGeom
 
+// A coefficient of compute_Y's stream: without beta, its word and its triple
+// (HostTables::yc_list).
+struct __align__(16) YcCoef {
+  double cg;
+  int at, trip;
+};
+// The coefficients of a record for one output, coef[first ..) to the next one's.
+struct YcGroup {
+  int first, out;  // out: task x kYcOuts + output
+};
+
 // compute_Y's fixed point (snap_kernels.cu), on the device and in its host walk.
 // limbs of v, |v| < 2^59, given v + 2^29: v = h 2^30 + l, -2^29 <= l < 2^29
 __host__ __device__ inline void split30(long long v, int& h, int& l) {
@@ -295,6 +306,12 @@ template <typename R> cudaError_t launch_u(const WorkArgs& a, cudaStream_t s);
 
 // Launchers (snap_kernels.cu), R = float (mixed) or double (FP64)
 template <typename R> cudaError_t launch_yi(const WorkArgs& a, cudaStream_t s);
+
+// The stream's words that depend on beta (bw: HostTables::beta_weights, device).
+// fixed: the FP64 path's fixed point, top [tasks x kYcOuts] scratch.
+cudaError_t launch_yc_coefs(bool fixed, const YcCoef* coef, int ncoef, const YcGroup* group, int ngroup, const double* bw,
+                            const int* task, int ntask, int nchunk, unsigned long long* top, unsigned* stream,
+                            cudaStream_t s);
 
 // Launch shape of compute_Y for N atoms: nblk blocks of atoms x split CTAs of
 // `threads`, with `smem` bytes of shared memory.

@@ -759,6 +759,58 @@ __global__ void __launch_bounds__(P::kWarps * 32, LM <= 5 ? 2 : 1) yc_kernel(Wor
   }
 }
 
+// ------------------------------------------- compute_Y's coefficients
+// The stream of a new beta, on the device: on the host it took, with the upload
+// of 6 and 11 MB, 2.1 ms at 2J14 in FP32 and 7.5 in fixed point (the list of terms
+// before it 1.9); all of snap_set_beta takes 27 and 77 us now, at 2J8 22 and 38 (83).
+__global__ void __launch_bounds__(256) yc_coef_kernel(const YcCoef* __restrict__ coef, int n, const double* __restrict__ bw,
+                                                      float* __restrict__ stream) {
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  if (k < n) stream[coef[k].at] = (float)(coef[k].cg * bw[coef[k].trip]);
+}
+
+// Fixed point, first pass: the largest sum of sizes of every output (a thread a
+// group; of two numbers that are not negative the larger has the larger bits, and
+// a NaN the largest).
+__global__ void __launch_bounds__(128) yc_top_kernel(const YcCoef* __restrict__ coef, const YcGroup* __restrict__ group, int n,
+                                                     const double* __restrict__ bw, unsigned long long* __restrict__ top) {
+  const int g = blockIdx.x * 128 + threadIdx.x;
+  if (g >= n) return;
+  double s = 0.0;
+  for (int k = group[g].first; k < group[g + 1].first; ++k) s += fabs(coef[k].cg * bw[coef[k].trip]);
+  atomicMax(top + group[g].out, (unsigned long long)__double_as_longlong(s));
+}
+
+// the exponent above it, or kYcNan
+__device__ __forceinline__ int yc_exponent(unsigned long long top) {
+  const double t = __longlong_as_double((long long)top);
+  int e = 0;
+  if (t > 0.0) frexp(t, &e);
+  return isfinite(t) ? e : kYcNan;
+}
+
+// Second pass: a thread a group's coefficients, or (past the groups) the
+// exponents in a chunk's head.
+__global__ void __launch_bounds__(128) yc_fixed_kernel(const YcCoef* __restrict__ coef, const YcGroup* __restrict__ group, int n,
+                                                       const double* __restrict__ bw, const int* __restrict__ task, int nchunk,
+                                                       const unsigned long long* __restrict__ top, unsigned* __restrict__ stream) {
+  const int g = blockIdx.x * 128 + threadIdx.x;
+  if (g < n) {
+    const int e = yc_exponent(top[group[g].out]);
+    for (int k = group[g].first; k < group[g + 1].first; ++k) {
+      const YcCoef c = coef[k];
+      const long long v = e == kYcNan ? 0 : __double2ll_rn(ldexp(c.cg * bw[c.trip], 60 - e));
+      const int hi = (int)((v + (1LL << 29)) >> 30);
+      stream[c.at] = (unsigned)hi;
+      stream[c.at + 1] = (unsigned)(int)(v - hi * (1LL << 30));
+    }
+  } else if (g < n + nchunk) {
+    unsigned* ch = stream + (size_t)(g - n) * kYcChunk;
+    const int k = (int)(ch[0] & 0x7FFFFFFFu), nout = task[k * kYcTask + 2];
+    for (int o = 0; o < 2; ++o) ch[2 + o] = (unsigned)yc_exponent(top[k * kYcOuts + (nout == 1 ? 0 : o)]);
+  }
+}
+
 // ------------------------------------------- compute_Y, one atom per warp
 // The alternative layout to the warp of atoms (the paper compares the two,
 // Sec. V-B): warp = one atom, its Ulisttot and conj(Ulisttot) staged in shared
@@ -1367,6 +1419,19 @@ YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves, int ntasks) 
   g.smem = yc_smem(rsize, H, ntasks, warps);
   g.split = yi_split(g.nblk, nsm, 0.02 / std::max(1, waves));
   return g;
+}
+
+cudaError_t launch_yc_coefs(bool fixed, const YcCoef* coef, int ncoef, const YcGroup* group, int ngroup, const double* bw,
+                            const int* task, int ntask, int nchunk, unsigned long long* top, unsigned* stream,
+                            cudaStream_t s) {
+  if (!fixed)
+    return launch_k(yc_coef_kernel, dim3((ncoef + 255) / 256), dim3(256), 0, s, coef, ncoef, bw,
+                    reinterpret_cast<float*>(stream));
+  cudaError_t e = cudaMemsetAsync(top, 0, sizeof(*top) * ntask * kYcOuts, s);
+  if (e == cudaSuccess) e = launch_k(yc_top_kernel, dim3((ngroup + 127) / 128), dim3(128), 0, s, coef, group, ngroup, bw, top);
+  if (e != cudaSuccess) return e;
+  return launch_k(yc_fixed_kernel, dim3((ngroup + nchunk + 127) / 128), dim3(128), 0, s, coef, group, ngroup, bw, task, nchunk,
+                  top, stream);
 }
 
 template <typename K>

@@ -769,15 +769,31 @@ void HostTables::build_classes(bool wide) {
     }
 }
 
-std::vector<unsigned> HostTables::yc_stream(const double* beta) const {
-  const std::vector<double> bw = beta_weights(beta);
-  std::vector<unsigned> w(yc_head);
-  for (size_t k = 0; k < w.size(); ++k) {
-    if (yc_trip[k] < 0) continue;
-    const float c = (float)(yc_cg[k] * bw[yc_trip[k]]);
-    std::memcpy(&w[k], &c, sizeof(c));
-  }
-  return w;
+void HostTables::yc_list(std::vector<YcCoef>& coef, std::vector<YcGroup>& group) const {
+  coef.clear();
+  group.clear();
+  std::vector<std::vector<YcCoef>> part(2 * kYcOuts);
+  const unsigned* last = nullptr;
+  int last_task = 0, outs = 0;
+  auto flush = [&] {
+    for (int o = 0; o < outs; ++o) {
+      // the output of a half: the same one in (wide) tasks of a single output
+      group.push_back({(int)coef.size(), last_task * kYcOuts + (yc_wide && yc_task[(size_t)last_task * kYcTask + 2] == 1 ? 0 : o)});
+      coef.insert(coef.end(), part[o].begin(), part[o].end());
+      part[o].clear();
+    }
+    outs = 0;
+  };
+  yc_rows([&](int k, const unsigned* head, int, size_t w, int o, int len) {
+    if (head != last) flush();
+    last = head;
+    last_task = k;
+    outs = std::max(outs, o + 1);
+    for (int c = 0; c < len; ++c)
+      if (yc_trip[w + 2 * c] >= 0) part[o].push_back({yc_cg[w + 2 * c], (int)(w + 2 * c), yc_trip[w + 2 * c]});
+  });
+  flush();
+  group.push_back({(int)coef.size(), 0});
 }
 
 std::vector<unsigned> HostTables::yc_fixed(const double* beta) const {

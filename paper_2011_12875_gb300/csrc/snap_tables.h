@@ -113,6 +113,12 @@ struct HostTables {
   std::vector<long> yc_cost;
   bool yc_wide = false;
   void build_classes(bool wide);
+  // frees yc_head, yc_cg and yc_trip (once they are on the device)
+  void drop_stream() {
+    std::vector<unsigned>().swap(yc_head);
+    std::vector<double>().swap(yc_cg);
+    std::vector<int>().swap(yc_trip);
+  }
   // f(task, word, output, rows' elements) over every row of every output: the
   // coefficient of element c is at word + c * stride
   template <typename F>
@@ -134,10 +140,14 @@ struct HostTables {
       }
     }
   }
-  // The stream's words with the coefficients of beta: FP32, or (wide) in 60-bit
-  // fixed point scaled by the power of two above each output's largest sum of
-  // their sizes over a record (kYcNan: not finite, the output is not a number).
-  std::vector<unsigned> yc_stream(const double* beta) const;
+  // The stream's coefficients in the order of their records and outputs (output
+  // after output, row after row), and the groups of a record and an output; a
+  // last group with first = their number ends the list.
+  void yc_list(std::vector<YcCoef>& coef, std::vector<YcGroup>& group) const;
+  // The stream's words of the FP64 path with the coefficients of beta in 60-bit
+  // fixed point, scaled by the power of two above each output's largest sum of
+  // their sizes over a record (kYcNan: not finite, the output is not a number):
+  // what launch_yc_coefs does on the device.
   std::vector<unsigned> yc_fixed(const double* beta) const;
   // The tasks dealt to nbins CTAs of about equal cost, decreasing in each:
   // nbins + 1 offsets, then the tasks
