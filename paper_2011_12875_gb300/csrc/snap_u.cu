@@ -352,10 +352,18 @@ cudaError_t launch_neigh_geom(const NeighArgs& na, const WorkArgs& a, int ncta, 
 // The units (several classes each, or one: HostTables::u_units) and the
 // groups.  The CTAs an SM holds share its pipes, a quarter of them each warp:
 // in multiply-adds a slot a launch lasts about
-//   max(ceil(blocks G / SMs) (cost / G + 4 J) / 4, half the longest unit),
+//   max(ceil(blocks G / SMs) (cost / G + 4 J) / 4, floor),
 // cost = a block's units, 4 J = about the powers that each CTA tabulates; at most
 // kUMaxWarps / 2 units a CTA.  Fewer than four warps would build the tables one
-// chain after the other.
+// chain after the other.  The floor is the longest unit's warp, which has every
+// other slot: about half of the 6 + 6 K of a class of its own (K = J / 2 + 1
+// steps; FP64 runs best with 3 K); units of several classes, 40, by their five
+// classes of one step, whose monomials count for more than their multiply-adds.
+// With the floors of 2J14 for every order, 27 and 30, small FP64 systems waited
+// for CTAs of nine units.  All splits of 143 shapes (FP64 2J4 to 2J14, FP32 2J10 to
+// 2J14, 16 to 16000 atoms): that choice lies 9.2% (FP64) and 4.9% over the best,
+// this one 2.7% and 4.3% (neighbour build and compute_U, 128 atoms: 2J6 55 -> 45 us,
+// 2J8 53 -> 49).
 template <typename R>
 cudaError_t launch_u(const WorkArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
@@ -366,7 +374,7 @@ cudaError_t launch_u(const WorkArgs& a, cudaStream_t s) {
     const int nu = f ? a.u_nfine : a.u_nunits;
     for (int g = (nu + kUMaxWarps / 2 - 1) / (kUMaxWarps / 2); g <= nu; ++g) {
       const double t = std::max((double)((nblk * g + nsm - 1) / nsm) * ((double)a.u_cost / g + 4.0 * a.twojmax) / 4.0,
-                                f ? 27.0 : 30.0);
+                                f ? (sizeof(R) == 8 ? 0.0 : 3.0) + 3.0 * (a.twojmax / 2 + 1) : 40.0);
       if (t < best - 1e-9) {
         best = t;
         G = g;
@@ -375,6 +383,7 @@ cudaError_t launch_u(const WorkArgs& a, cudaStream_t s) {
     }
   }
   const int nu = fine ? a.u_nfine : a.u_nunits, per = (nu + G - 1) / G, nw = std::max(4, 2 * per);
+  G = (nu + per - 1) / per;  // no group without a unit
   const size_t tables = std::max((size_t)2 * u_slots(sizeof(R)) * u_slot_len(a.twojmax), (size_t)per * kUSums);
   const size_t smem = sizeof(rec_ab<R>) * (size_t)a.npair_steps + sizeof(R) * ((size_t)a.K * 160 + tables);
   cudaError_t e = allow_smem(u_kernel<R>, smem);
