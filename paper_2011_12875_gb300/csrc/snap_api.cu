@@ -576,24 +576,26 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
   return a;
 }
 
-// FP32 up to 2J = 9 runs compute_U by the layer recursion, fused with the
-// neighbour build: one launch less, and the closed form gains little there.
-// Neighbour build and compute_U, layers / closed form: 2J8 2000 atoms 36 / 40 us,
-// 16000 atoms 183 / 192; 2J6 1024 atoms 20 / 30; above, 2J11 57 / 50, 2J14 86 / 57.
-bool u_by_layers(const snap_ctx* c) {
-  return c->precision == SNAP_MIXED && c->twojmax >= 1 && c->twojmax <= snap::kUColMax;
-}
+// FP32 up to 2J = 9 and FP64 up to 2J = 5 run compute_U by the layer recursion,
+// fused with the neighbour build: one launch less, and the closed form's slots,
+// one after the other, take their time however few the atoms.  The order alone
+// decides, so that a configuration's U is the same alone and in a batch.
+// Neighbour build and compute_U, layers / closed form:
+// FP32 2J8 2000 atoms 36 / 40 us, 16000 atoms 183 / 192; 2J6 1024 atoms 20 / 30; above,
+// 2J11 57 / 50, 2J14 86 / 57.  FP64, 128 / 2000 atoms: 2J2 18 / 37, 46 / 55; 2J4 24 / 40,
+// 75 / 76; 2J5 28 / 43, 97 / 92; above, 2J6 34 / 45, 153 / 110, 2J8 59 / 49, 278 / 160.
+bool u_by_layers(const snap_ctx* c) { return c->twojmax <= snap::u_col_max(c->rsize()); }
 
 // The neighbour build with the slots' geometry, and compute_U; the launches
 // are added to *launches.
 int launch_neigh_and_u(snap_ctx* c, const snap::NeighArgs& na, const snap::WorkArgs& a, int ncta, cudaStream_t s,
                        int* launches) {
+  const bool mixed = c->precision == SNAP_MIXED;
   if (u_by_layers(c)) {
-    SNAP_CUDA(c, snap::launch_neigh_u(na, a, ncta, s));
+    SNAP_CUDA(c, mixed ? snap::launch_neigh_u<float>(na, a, ncta, s) : snap::launch_neigh_u<double>(na, a, ncta, s));
     *launches += 1;
     return SNAP_OK;
   }
-  const bool mixed = c->precision == SNAP_MIXED;
   SNAP_CUDA(c, mixed ? snap::launch_neigh_geom<float>(na, a, ncta, s) : snap::launch_neigh_geom<double>(na, a, ncta, s));
   SNAP_CUDA(c, mixed ? snap::launch_u<float>(a, s) : snap::launch_u<double>(a, s));
   *launches += 2;
@@ -650,7 +652,7 @@ int enqueue(snap_ctx* c, int n, const double* pos, const double* box, const int*
                      c->d_img, c->d_rij, c->d_key, c->d_flags, s));
     c->launches += 1;
     SNAP_CUDA(c, mark());
-    if (u_by_layers(c)) SNAP_CUDA(c, snap::launch_ui_col(a, s));
+    if (u_by_layers(c)) SNAP_CUDA(c, mixed ? snap::launch_ui_col<float>(a, s) : snap::launch_ui_col<double>(a, s));
     else SNAP_CUDA(c, mixed ? snap::launch_u<float>(a, s) : snap::launch_u<double>(a, s));
     c->launches += 1;
   } else {

@@ -6,23 +6,25 @@
 
 namespace snap {
 
-cudaError_t launch_ui_col(const WorkArgs& a, cudaStream_t s) {
+template <>
+cudaError_t launch_ui_col<float>(const WorkArgs& a, cudaStream_t s) {
   switch (a.twojmax) {
 #define SNAP_CASE(J) \
   case J: return col::launch_ui_col_t<float, J>(a, s);
-    SNAP_CASE(1) SNAP_CASE(2) SNAP_CASE(3) SNAP_CASE(4) SNAP_CASE(5) SNAP_CASE(6) SNAP_CASE(7)
-    SNAP_CASE(8) SNAP_CASE(9)
+    SNAP_CASE(0) SNAP_CASE(1) SNAP_CASE(2) SNAP_CASE(3) SNAP_CASE(4) SNAP_CASE(5) SNAP_CASE(6)
+    SNAP_CASE(7) SNAP_CASE(8) SNAP_CASE(9)
 #undef SNAP_CASE
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_neigh_u(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s) {
+template <>
+cudaError_t launch_neigh_u<float>(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s) {
   switch (a.twojmax) {
 #define SNAP_CASE(J) \
   case J: return col::launch_neigh_u_t<float, J>(na, a, ncta, s);
-    SNAP_CASE(1) SNAP_CASE(2) SNAP_CASE(3) SNAP_CASE(4) SNAP_CASE(5) SNAP_CASE(6) SNAP_CASE(7)
-    SNAP_CASE(8) SNAP_CASE(9)
+    SNAP_CASE(0) SNAP_CASE(1) SNAP_CASE(2) SNAP_CASE(3) SNAP_CASE(4) SNAP_CASE(5) SNAP_CASE(6)
+    SNAP_CASE(7) SNAP_CASE(8) SNAP_CASE(9)
 #undef SNAP_CASE
     default: return cudaErrorInvalidValue;
   }

@@ -1,10 +1,33 @@
-// snap_col_f64.cu -- instances in FP64 working precision, one per 2J: the fused
-// dE and the tangent of Ulisttot along a displacement field.
+// snap_col_f64.cu -- instances in FP64 working precision, one per 2J: compute_U by
+// the layer recursion, the fused dE, the tangent of Ulisttot along a displacement
+// field.
 #include "snap_colkernels.cuh"
 #include "snap_pairs.cuh"
 #include "snap_tables.h"
 
 namespace snap {
+
+template <>
+cudaError_t launch_ui_col<double>(const WorkArgs& a, cudaStream_t s) {
+  switch (a.twojmax) {
+#define SNAP_CASE(J) \
+  case J: return col::launch_ui_col_t<double, J>(a, s);
+    SNAP_CASE(0) SNAP_CASE(1) SNAP_CASE(2) SNAP_CASE(3) SNAP_CASE(4) SNAP_CASE(5)
+#undef SNAP_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <>
+cudaError_t launch_neigh_u<double>(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s) {
+  switch (a.twojmax) {
+#define SNAP_CASE(J) \
+  case J: return col::launch_neigh_u_t<double, J>(na, a, ncta, s);
+    SNAP_CASE(0) SNAP_CASE(1) SNAP_CASE(2) SNAP_CASE(3) SNAP_CASE(4) SNAP_CASE(5)
+#undef SNAP_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
 
 template <>
 cudaError_t launch_de<double>(const WorkArgs& a, cudaStream_t s) {

@@ -353,12 +353,12 @@ BiPlan bi_plan(int rsize, int H, bool deriv, int maxchunks, int maxterms, int la
 // whether the conjugate-plane records can ever be used for this size and H
 bool bi_plane_fits(int rsize, int H);
 
-// FP32 compute_U by the layer recursion (snap_col_f32.cu), 1 <= 2J <= kUColMax:
-// for caller lists, and fused with the neighbour build, one configuration
-// (ncta = 0) or a batch.
-constexpr int kUColMax = 9;
-cudaError_t launch_ui_col(const WorkArgs& a, cudaStream_t s);
-cudaError_t launch_neigh_u(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s);
+// compute_U by the layer recursion (snap_col_*.cu), 2J <= u_col_max: for caller
+// lists, and fused with the neighbour build, one configuration (ncta = 0) or a
+// batch.
+constexpr int u_col_max(size_t rsize) { return rsize == 4 ? 9 : 5; }
+template <typename R> cudaError_t launch_ui_col(const WorkArgs& a, cudaStream_t s);
+template <typename R> cudaError_t launch_neigh_u(const NeighArgs& na, const WorkArgs& a, int ncta, cudaStream_t s);
 // Tangent of Ulisttot along the displacement field g ([N][3], device); 0..14.
 template <typename R>
 cudaError_t launch_tan_col(const WorkArgs& a, const double* g, void* dU, cudaStream_t s);
