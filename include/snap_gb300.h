@@ -223,7 +223,7 @@ int snap_bispectrum_deriv_batch(snap_ctx* ctx, int nconf, const int* natoms, con
  *  col_warps (2, 4 or 8): the fused dE kernel plans its CTA shape (atoms and
  *    warps per CTA) from the system size and the largest neighbour count
  *    seen; a 32-pair batch is shared by four warps when an SM would hold fewer
- *    than 2 col_warps batches;
+ *    than col_warps batches (SNAP_MIXED above 2J = 9: 2 col_warps);
  *  yi_waves (1..8): fineness of the compute_Y split; the CTAs a block of
  *    atoms minimise ceil(CTAs / SMs) * (1/CTAs a block + 0.02/yi_waves);
  *  yi_layout: 0 = compute_Y with a warp of 32 atoms (lanes = atoms, the

@@ -243,7 +243,7 @@ struct WorkArgs {
   const int* half_tmm;
   const void* hscale;  // R [H]: S_t(ma, mb) of the scaled recursion (u = S v)
   int nsm;
-  int col_warps;  // fused dE: an SM with fewer than 2 col_warps batches shares them (tunable)
+  int col_warps;  // fused dE: an SM with few batches shares them (tunable, de_plan)
   int de_maxcnt;  // neighbour count the fused dE launch is planned for (last seen maximum, else K)
   int yi_waves;   // compute_Y waves per SM (tunable)
   int persist;    // tunable: bit 0 persistent compute_Y, bit 1 persistent fused dE (work queues)

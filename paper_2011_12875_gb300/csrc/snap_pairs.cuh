@@ -506,9 +506,13 @@ __global__ void __launch_bounds__(de_max_warps<R>() * 32, 1) de_pair_kernel(Work
 //   ceil(CTAs / SMs) ceil(A maxcnt / 32),
 // plus a tenth of a batch a CTA for its staging (2000 atoms: 143 CTAs of 14
 // atoms, 12 batches, one CTA an SM).  The batch is shared when an SM would hold
-// fewer than 2 col_warps batch-warps (the tunable; default 8, two a scheduler):
-// each FP64 unit and scheduler serves its own warps, so a lone batch-warp would
-// leave three quarters of the SM idle.
+// fewer than col_warps batch-warps (the tunable; default 4, one a scheduler; FP32
+// above 2J = 9 twice as many: its chains are long, and two warps a scheduler hide
+// each other's latency): each FP64 unit and scheduler serves its own warps, so a
+// lone batch-warp would leave three quarters of the SM idle, but sharing costs
+// a barrier a round and empty parts at small orders.  1024 atoms (6 batches an
+// SM), shared / not: FP64 2J1 18 / 12 us, 2J4 31 / 25, 2J8 88 / 76; FP32 2J2 10 / 8, 2J8
+// 13.5 / 12.3, 2J11 15.6 / 17.2.
 // force_A > 0 (SNAP_KNOB_DE_ATOMS): that A, if its shared memory fits.
 struct DePlan {
   int nw, A, split;
@@ -525,7 +529,7 @@ inline DePlan de_plan(int n, int maxcnt, int nsm, int col_warps, int force_A) {
     const long ctas = (n + A - 1) / A, per_sm = (ctas + nsm - 1) / nsm;
     DePlan p;
     p.A = A;
-    p.split = per_sm * batches < 2 * col_warps ? kParts : 1;
+    p.split = per_sm * batches < (sizeof(R) == 4 && J2 > 9 ? 2 : 1) * col_warps ? kParts : 1;
     p.nw = std::min(batches * p.split, de_max_warps<R>());
     p.smem = sizeof(y4<R>) * (size_t)A * NS + sizeof(rec_ab<R>) * NS +
              (p.split > 1 ? sizeof(Sums<R>) * (size_t)p.nw * 32 : 0) + sizeof(int) * (A + 1);
