@@ -206,10 +206,15 @@ __device__ __forceinline__ void cp_async_wait() {
 // 3039; 128 atoms, 2J8 119 -> 28.
 // Chunks of a warp's ring
 __host__ __device__ constexpr int yc_slots(int rsize) { return rsize == 8 ? 2 : 3; }
-// Warps of a CTA, by the longest vector LM: one CTA an SM above 2J = 9 (the
-// block's U fills its shared memory), two up to there, with the registers that
-// FP32 (128 and 64) and fixed point (96) need.
-__host__ __device__ constexpr int yc_warps(int rsize, int LM) { return rsize == 4 ? 16 : LM <= 5 ? 10 : 20; }
+// Warps of a CTA: one CTA an SM above 2J = 9 (the block's U fills its shared
+// memory), two up to there, with the registers that FP32 and fixed point (96)
+// need.  FP32 up to 2J = 8: with sixteen warps the tasks left most of them waiting
+// for the largest, and their rings took half of the shared memory; sixteen /
+// eight, us: 2J4 2000 atoms 14.2 / 10.0, 5488 22.5 / 18.2; 2J6 22.3 / 16.3, 39.0 / 32.4;
+// 2J8 35.1 / 33.8, 75.7 / 71.4, 16000 atoms 178.3 / 178.0; but 2J9 49.1 / 54.5, 113 / 121.
+__host__ __device__ constexpr int yc_warps(int rsize, int H) {
+  return rsize == 4 ? (H <= half_size(8) ? 8 : 16) : H <= half_size(9) ? 10 : 20;
+}
 
 typedef unsigned long long f2;  // two FP32
 
@@ -350,10 +355,10 @@ __device__ __forceinline__ void yc_chunk(const unsigned* __restrict__ p, const c
 
 // The two precisions of the walk below: what a task's outputs are held in, how
 // a chunk adds to them and how they are stored.
-template <int LM>
+template <int LM, int WARPS>
 struct YcSingle {
   static constexpr int kAtoms = 32;  // of a block; a row is their [32] of an element
-  static constexpr int kWarps = yc_warps(4, LM);  // of a CTA
+  static constexpr int kWarps = WARPS;  // of a CTA
   static constexpr int kSlots = yc_slots(4);
   static constexpr int NPM = LM > 5 ? 4 : 2;
   static constexpr bool COMP = LM > 5;
@@ -532,10 +537,11 @@ __device__ __forceinline__ void yf_run(const unsigned* __restrict__& p, YcHead& 
   } while (h.len() == L);
 }
 
-template <int LM>
+constexpr int kYcBad = 1 << 20;
+template <int LM, int WARPS>
 struct YcFixed {
   static constexpr int kAtoms = 16;
-  static constexpr int kWarps = yc_warps(8, LM);
+  static constexpr int kWarps = WARPS;
   static constexpr int kSlots = yc_slots(8);
   Acc96 yr, yi;
   __device__ __forceinline__ void clear() { yr = yi = Acc96{0u, 0u, 0u}; }
@@ -553,8 +559,7 @@ struct YcFixed {
       }
     }
   }
-  // `ex`: the exponent of the lane's atom, or kBad
-  static constexpr int kBad = 1 << 20;
+  // `ex`: the exponent of the lane's atom, or kYcBad
   __device__ __forceinline__ void store(const int* __restrict__ rec, uint4 h, char* Yb, const char* other, int lane,
                                         int ex) const {
     const int o = lane >> 4, nout = __ldg(rec + 2);
@@ -569,7 +574,7 @@ struct YcFixed {
     const int n1 = n >> 1, n2 = n - n1;
     double f1 = __hiloint2double((n1 + 1023) << 20, 0);
     const double f2 = __hiloint2double((n2 + 1023) << 20, 0);
-    if (ex == kBad || ec == kYcNan) f1 = __longlong_as_double(0x7FF8000000000000LL);
+    if (ex == kYcBad || ec == kYcNan) f1 = __longlong_as_double(0x7FF8000000000000LL);
     const int at = __ldg(rec + 4 + o) * 32 + (lane & 15);
     cx<double> v = mk<double>(r.value() * f1 * f2, i.value() * f1 * f2);
     if (other) {
@@ -583,7 +588,7 @@ struct YcFixed {
 };
 
 // The staged block of U, [H][16] complex double, to fixed point in place;
-// returns the exponent of the lane's atom (kBad if its U is not finite).
+// returns the exponent of the lane's atom (kYcBad if its U is not finite).
 __device__ int yf_prepare(unsigned char* su, int H, int* top) {
   // top: [16] in shared memory.  A thread has one atom throughout.
   const int al = threadIdx.x & 15, n = H * 16;
@@ -605,7 +610,7 @@ __device__ int yf_prepare(unsigned char* su, int H, int* top) {
     yc_limbs(v.z, v.w, E, w.z, w.w);
     *x = w;
   }
-  return E == 0x7FF ? YcFixed<8>::kBad : E - 1022;
+  return E == 0x7FF ? kYcBad : E - 1022;
 }
 
 // One warp's share of a CTA's tasks (tl: first chunk and chunks of each),
@@ -1414,7 +1419,7 @@ YiGeometry yi_geometry(int rsize, int H, int n, int nsm, int waves, int ntasks) 
   // The CTAs an SM holds share its pipes, so the launch lasts as long as the
   // SM with the most CTAs.  c = 0.02 / waves (the tunable: more waves, finer
   // splits).
-  const int warps = yc_warps(rsize, H <= half_size(9) ? 5 : 8);
+  const int warps = yc_warps(rsize, H);
   g.threads = warps * 32;
   g.smem = yc_smem(rsize, H, ntasks, warps);
   g.split = yi_split(g.nblk, nsm, 0.02 / std::max(1, waves));
@@ -1468,10 +1473,14 @@ cudaError_t launch_yi(const WorkArgs& a, cudaStream_t s) {
   }
   const YiGeometry g = yi_geometry(sizeof(R), a.H, a.n, a.nsm, a.yi_waves, a.yc_ntask);
   if (g.split != a.yc_split) return cudaErrorInvalidValue;
-  if constexpr (sizeof(R) == 4)
-    return a.twojmax <= 9 ? launch_yc<YcSingle<5>, 5>(g, a, s) : launch_yc<YcSingle<8>, 8>(g, a, s);
+  constexpr int RS = sizeof(R), W8 = yc_warps(RS, half_size(8)), W9 = yc_warps(RS, half_size(9)),
+                W14 = yc_warps(RS, half_size(14));
+  if constexpr (RS == 4)
+    return a.twojmax <= 8   ? launch_yc<YcSingle<5, W8>, 5>(g, a, s)
+           : a.twojmax <= 9 ? launch_yc<YcSingle<5, W9>, 5>(g, a, s)
+                            : launch_yc<YcSingle<8, W14>, 8>(g, a, s);
   else
-    return a.twojmax <= 9 ? launch_yc<YcFixed<5>, 5>(g, a, s) : launch_yc<YcFixed<8>, 8>(g, a, s);
+    return a.twojmax <= 9 ? launch_yc<YcFixed<5, W9>, 5>(g, a, s) : launch_yc<YcFixed<8, W14>, 8>(g, a, s);
 }
 
 template <typename R>
