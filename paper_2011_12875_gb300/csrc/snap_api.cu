@@ -1224,8 +1224,8 @@ int snap_create(int twojmax, double rcut, double rfac0, double rmin0, int switch
   if (!rc) rc = upload_r(c, &c->d_hscale, c->tab.half_scale);
   if (!rc) rc = upload(c, &c->d_pair_idx, c->tab.pair_idx);
   const bool fp64 = precision == SNAP_FP64;
-  if (!rc) rc = upload_r(c, &c->d_pair_scale, c->tab.pair_scales(fp64));  // the weighted Y of the fused dE
-  if (!rc) rc = upload_r(c, &c->d_pair_norm, fp64 ? c->tab.pair_norm_fix : c->tab.pair_norm);
+  if (!rc) rc = upload_r(c, &c->d_pair_scale, c->tab.pair_scales(fp64, true));  // the weighted Y of the fused dE
+  if (!rc) rc = upload_r(c, &c->d_pair_norm, c->tab.pair_scales(fp64, false));
   if (!rc) rc = upload_r(c, &c->d_pair_ab, c->tab.pair_recursion(fp64));
   if (!rc && fp64) {
     const std::vector<int> cls = c->tab.pair_classes();

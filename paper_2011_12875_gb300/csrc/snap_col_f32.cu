@@ -58,7 +58,7 @@ cudaError_t launch_tan_col<float>(const WorkArgs& a, const double* g, void* dU, 
 
 template <>
 int pair_host<float>(const HostTables& tab, int npairs, const double* par, const double* y, double* out) {
-  const std::vector<double> scale = tab.pair_scales(false), ab = tab.pair_recursion(false);
+  const std::vector<double> scale = tab.pair_scales(false, true), ab = tab.pair_recursion(false);
   const std::vector<int> cls = tab.pair_classes();
   switch (tab.twojmax) {
 #define SNAP_CASE(J) \

@@ -57,7 +57,7 @@ cudaError_t launch_tan_col<double>(const WorkArgs& a, const double* g, void* dU,
 
 template <>
 int pair_host<double>(const HostTables& tab, int npairs, const double* par, const double* y, double* out) {
-  const std::vector<double> scale = tab.pair_scales(true), ab = tab.pair_recursion(true);
+  const std::vector<double> scale = tab.pair_scales(true, true), ab = tab.pair_recursion(true);
   const std::vector<int> cls = tab.pair_classes();
   switch (tab.twojmax) {
 #define SNAP_CASE(J) \

@@ -277,8 +277,8 @@ struct WorkArgs {
   const int* ysched;
   // closed-form u of a pair (snap_pairs.cuh, HostTables::pair_*), per step
   const unsigned* pair_idx;
-  const void* pair_scale;  // R: norm x weight
-  const void* pair_norm;   // R
+  const void* pair_scale;  // step_scale<R>: norm x weight
+  const void* pair_norm;   // step_scale<R>
   const void* pair_ab;     // rec_ab<R>
   const double* pair_fix;  // FP64: [step][kPairFix], the polynomials' rounding (HostTables::pair_fix)
   const int* pair_cls;     // FP64: the classes of several steps, first step | steps << 16

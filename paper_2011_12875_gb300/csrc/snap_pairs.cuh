@@ -38,6 +38,7 @@
 #include <cmath>
 #include <vector>
 
+#include "snap_closed.cuh"
 #include "snap_internal.h"
 
 namespace snap {
@@ -45,58 +46,12 @@ namespace pr {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// the arithmetic of a pair is the host walk's too (snap_pair_host)
-#define SNAP_HD __host__ __device__ __forceinline__
-
-template <typename R>
-struct __align__(2 * sizeof(R)) r2 {
-  R x, y;
-};
 // the two elements of (p, q, k): re and im of the b^q one, re and im of the
 // (-conj b)^q one
 template <typename R>
 struct __align__(16) y4 {
   R pr, pi, mr, mi;
 };
-
-// alpha_k, beta_k of a step.  Their rounding is the same for every pair, so its
-// effect adds up over them, where the rest of a pair's rounding averages out.
-// FP64 takes them rounded to FP32 and turns the weighted Y, once an atom, into
-// the coefficients in the polynomials that those give (fix_class).  The error
-// that all pairs share, of the size of S, 2J8 / 2J11 / 2J14, in units of 2^-53:
-// 0.7 each, which is the scales' and Y's own rounding; rounded to FP64 and left
-// so 0.8 / 1.1 / 1.4 (tests/test_pair_closed_form.py).  It takes 1% of a step.
-// FP32: with the part that their rounding leaves off, z and w (rounded and left
-// so, 2J14: 1.3e-7 of the virial's sum of sizes).  Eight 2000-atom cells, mean
-// error of the virial with the rounded ones / now / the layer recursion: 2J10
-// 7.7e-7 / 5.3e-7 / 5.3e-7, 2J14 3.4e-7 / 2.8e-7 / 3.1e-7, for three operations a
-// step (dE 26.6 -> 28.1 us).
-template <typename R>
-struct rec_ab;
-template <>
-struct __align__(16) rec_ab<float> {
-  float x, y, z, w;
-};
-template <>
-struct __align__(16) rec_ab<double> {
-  double x, y;
-};
-
-// x * y + z in one rounding, also where the compiler would split it
-#ifdef __CUDA_ARCH__
-__device__ __forceinline__ float fm(float x, float y, float z) { return __fmaf_rn(x, y, z); }
-__device__ __forceinline__ double fm(double x, double y, double z) { return __fma_rn(x, y, z); }
-#else
-__host__ __device__ inline float fm(float x, float y, float z) { return std::fma(x, y, z); }
-__host__ __device__ inline double fm(double x, double y, double z) { return std::fma(x, y, z); }
-#endif
-
-// alpha x + beta
-SNAP_HD float rec_t(const rec_ab<float>& c, float x) { return fm(c.x, x, c.y) + fm(c.z, x, c.w); }
-SNAP_HD double rec_t(const rec_ab<double>& c, double x) { return fm(c.x, x, c.y); }
-// alpha p + d
-SNAP_HD float rec_d(const rec_ab<float>& c, float p, float d) { return fm(c.x, p, fm(c.z, p, d)); }
-SNAP_HD double rec_d(const rec_ab<double>& c, double p, double d) { return fm(c.x, p, d); }
 
 // steps (p, q, k) of the classes with p' < p: a class of remainder
 // r = 2J - p - q has r / 2 + 1 steps, stored p rising, then r rising
@@ -139,17 +94,17 @@ struct Sums {
 // The weighted, scaled Y of a step (w: HostTables::pair_idx) from the Y of its
 // two elements, at(element) each.
 template <typename R, typename F>
-SNAP_HD y4<R> weighted_y(unsigned w, R sc, F&& at) {
+SNAP_HD y4<R> weighted_y(unsigned w, step_scale<R> sc, F&& at) {
   const r2<R> u = at(w & 1023u);
   y4<R> v;
-  const R sp = (w >> 11) & 1u ? -sc : sc;
-  v.pr = sp * u.x;
-  v.pi = ((w >> 10) & 1u) ? -sp * u.y : sp * u.y;
+  const bool neg = (w >> 11) & 1u, conj = (w >> 10) & 1u;
+  v.pr = scaled(sc, neg ? -u.x : u.x);
+  v.pi = scaled(sc, neg != conj ? -u.y : u.y);
   v.mr = v.mi = R(0);
   if ((w >> 22) & 1u) {
     const r2<R> m = at((w >> 12) & 1023u);
-    v.mr = sc * m.x;
-    v.mi = sc * m.y;
+    v.mr = scaled(sc, m.x);
+    v.mi = scaled(sc, m.y);
   }
   return v;
 }
@@ -204,10 +159,10 @@ SNAP_HD void class_sums(const y4<R>* __restrict__ y, const rec_ab<R>* __restrict
       d = c.x;
     } else if (k == 2) {
       p = fm(t, p1, R(-1));
-      d = fm(t, d1, rec_d(c, p1, R(0)));
+      d = rec_d(c, t, d1, p1, R(0));
     } else {
       p = fm(t, p1, -p0);
-      d = fm(t, d1, rec_d(c, p1, -d0));
+      d = rec_d(c, t, d1, p1, d0);
     }
     p0 = p1;
     p1 = p;
@@ -225,22 +180,6 @@ SNAP_HD void class_sums(const y4<R>* __restrict__ y, const rec_ab<R>* __restrict
       xm.y = k == 1 ? v.mi * d : fm(v.mi, d, xm.y);
     }
   }
-}
-
-// v * b + c (complex)
-template <typename R>
-SNAP_HD r2<R> cfma(r2<R> v, r2<R> b, r2<R> c) {
-  r2<R> o;
-  o.x = fm(-v.y, b.y, fm(v.x, b.x, c.x));
-  o.y = fm(v.y, b.x, fm(v.x, b.y, c.y));
-  return o;
-}
-template <typename R>
-SNAP_HD r2<R> cmul(r2<R> v, r2<R> b) {
-  r2<R> o;
-  o.x = fm(-v.y, b.y, v.x * b.x);
-  o.y = fm(v.y, b.x, v.x * b.y);
-  return o;
 }
 
 // Horner state in q of one p: value, derivative and x-derivative of the two
@@ -402,7 +341,7 @@ __global__ void __launch_bounds__(de_max_warps<R>() * 32, 1) de_pair_kernel(Work
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int H = a.H;
   const rec_ab<R>* abg = reinterpret_cast<const rec_ab<R>*>(a.pair_ab);
-  const R* scg = reinterpret_cast<const R*>(a.pair_scale);
+  const step_scale<R>* scg = reinterpret_cast<const step_scale<R>*>(a.pair_scale);
   for (int st = threadIdx.x; st < NS; st += blockDim.x) abt[st] = abg[st];
   const long nitems = (a.n + A - 1) / A;
   for (long item = blockIdx.x;;) {
@@ -582,9 +521,11 @@ void pair_host_t(const std::vector<unsigned>& idx, const std::vector<double>& sc
   constexpr int NS = steps_total(J2);
   std::vector<y4<R>> Y(NS);
   std::vector<rec_ab<R>> t(NS);
-  constexpr int W = sizeof(rec_ab<R>) / sizeof(R);
+  constexpr int W = sizeof(rec_ab<R>) / sizeof(R), V = sizeof(step_scale<R>) / sizeof(R);
   for (int st = 0; st < NS; ++st) {
-    Y[st] = weighted_y<R>(idx[st], (R)scale[st], [&](unsigned e) { return r2<R>{(R)y[2 * e], (R)y[2 * e + 1]}; });
+    step_scale<R> sc;
+    for (int k = 0; k < V; ++k) (&sc.x)[k] = (R)scale[V * st + k];
+    Y[st] = weighted_y<R>(idx[st], sc, [&](unsigned e) { return r2<R>{(R)y[2 * e], (R)y[2 * e + 1]}; });
     for (int k = 0; k < W; ++k) (&t[st].x)[k] = (R)ab[W * st + k];
   }
   if constexpr (sizeof(R) == 8)

@@ -426,9 +426,13 @@ void HostTables::build(int J2) {
   }
 }
 
-std::vector<double> HostTables::pair_scales(bool fp64) const {
-  std::vector<double> w(fp64 ? pair_norm_fix : pair_norm);
-  for (size_t k = 0; k < w.size(); ++k) w[k] *= pair_weight[k];
+std::vector<double> HostTables::pair_scales(bool fp64, bool weighted) const {
+  std::vector<double> w;
+  for (size_t k = 0; k < pair_norm.size(); ++k) {
+    const double n = (fp64 ? pair_norm_fix[k] : pair_norm[k]) * (weighted ? pair_weight[k] : 1.0);
+    w.push_back(fp64 ? n : (float)n);
+    if (!fp64) w.push_back(n - (float)n);
+  }
   return w;
 }
 

@@ -29,43 +29,20 @@
 #include "snap_geom.cuh"
 #include "snap_internal.h"
 #include "snap_neigh.cuh"
+#include "snap_closed.cuh"
 
 namespace snap {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-template <typename R>
-struct __align__(2 * sizeof(R)) r2 {
-  R x, y;
-};
-
-// alpha_k, beta_k of a step, as in snap_pairs.cuh: in FP32 with what their
-// rounding leaves off, in FP64 rounded to FP32 (the sums are then put right)
-template <typename R>
-struct rec_ab;
-template <>
-struct __align__(16) rec_ab<float> {
-  float x, y, z, w;
-};
-template <>
-struct __align__(16) rec_ab<double> {
-  double x, y;
-};
-
-__device__ __forceinline__ float fm(float x, float y, float z) { return __fmaf_rn(x, y, z); }
-__device__ __forceinline__ double fm(double x, double y, double z) { return __fma_rn(x, y, z); }
-
-__device__ __forceinline__ float rec_t(const rec_ab<float>& c, float x) { return fm(c.x, x, c.y) + fm(c.z, x, c.w); }
-__device__ __forceinline__ double rec_t(const rec_ab<double>& c, double x) { return fm(c.x, x, c.y); }
-
-template <typename R>
-__device__ __forceinline__ r2<R> cmul(r2<R> v, r2<R> b) {
-  r2<R> o;
-  o.x = fm(-v.y, b.y, v.x * b.x);
-  o.y = fm(v.y, b.x, v.x * b.y);
-  return o;
-}
+using pr::cmul;
+using pr::fm;
+using pr::r2;
+using pr::rec_ab;
+using pr::rec_t;
+using pr::scaled;
+using pr::step_scale;
 
 constexpr int kUMaxWarps = 18;  // 112 registers: the longest unit's sums in FP64
 // pair slots of a chunk, by the size of R: two buffers of 2J14 take 61 KB
@@ -242,16 +219,15 @@ __device__ __forceinline__ void u_unit(const WorkArgs& a, const UArgs& u, const 
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const unsigned w = __ldg(a.pair_idx + st[m] + k);
-      const R n = reinterpret_cast<const R*>(a.pair_norm)[st[m] + k];
+      const step_scale<R> n = reinterpret_cast<const step_scale<R>*>(a.pair_norm)[st[m] + k];
       const R odd = (q[m] & 1) ? R(-1) : R(1);
       // (k, k + q): stored, or its mirror (-1)^q conj is
-      r2<R> v = {n * sp[m][k].x, n * sp[m][k].y};
+      r2<R> v = {scaled(n, sp[m][k].x), scaled(n, sp[m][k].y)};
       if (q[m] == 0) v.x += (R)a.wself;
       const r2<R> mir = {odd * v.x, -odd * v.y};
       U[(w & 1023u) * 32] = ((w >> 10) & 1u) ? mir : v;
       if (p[m] > 0 && q[m] > 0) {
-        const R on = odd * n;
-        U[((w >> 12) & 1023u) * 32] = r2<R>{on * sm[m][k].x, on * sm[m][k].y};
+        U[((w >> 12) & 1023u) * 32] = r2<R>{odd * scaled(n, sm[m][k].x), odd * scaled(n, sm[m][k].y)};
         // on the middle column (2 (k + q) = t, p = q) the mirror is stored too
         if (p[m] == q[m]) {
           const int t = p[m] + q[m] + 2 * k, mb = k + q[m];

@@ -145,3 +145,37 @@ def test_value_and_gradient(snapmod, twojmax, precision):
     tol = 40 * (twojmax + 1) * EPS[precision]
     assert np.abs(o[:, 0] - ref).max() <= tol * np.abs(ref).max()
     assert np.abs(along(o, ab, tan) - d).max() <= tol * ((twojmax + 1) * np.abs(ref).max() + np.abs(d).max())
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_no_error_is_shared_by_all_atoms(snapmod, precision):
+    """One element of Y at a time, with many values: the error of its share of S,
+    projected on that share, is the same for every atom only by the tables.  In
+    FP32 these have what their rounding leaves off beside them, which a kernel may
+    round away again; in FP64 the scale's own rounding is left, 0.41 EPS.  3000
+    pairs with rounding errors of up to 4 EPS each leave 4 / sqrt(3000) = 0.07 EPS in a
+    value's projection and the value's own product, 0.41 EPS, sqrt(12) less in the
+    mean of twelve, 0.14 together: twice that is allowed beside the scale's."""
+    twojmax, n = 11, 3000
+    rng = np.random.default_rng(1)
+    ab = sphere(rng, n)
+    if precision == 1:
+        ab = ab.astype(np.float32).astype(np.float64)
+    g = ab.astype(np.longdouble)
+    u, _ = layers(twojmax, g[:, 0] + 1j * g[:, 1], g[:, 2] + 1j * g[:, 3])
+    els = [(t, ma, mb) for t in range(twojmax + 1) for mb in range(t // 2 + 1) for ma in range(t + 1)
+           if not (2 * mb == t and ma > mb)]
+    rng.shuffle(els)
+    gain = []
+    for t, ma, mb in els[:40]:
+        weight, got = 2 if 2 * mb < t or ma < mb else 1, []
+        for _ in range(12):
+            y = np.zeros((snapmod.half_size(twojmax), 2))
+            val = 1.0 + rng.random()
+            val = float(np.float32(val)) if precision == 1 else val
+            y[snapmod.half_index(twojmax, t, ma, mb), 0] = val
+            ref = weight * val * u[t][:, ma, mb].real
+            err = (snapmod.pair_host(twojmax, ab, y, precision=precision)[:, 0] - ref).astype(np.float64)
+            got.append((err * ref).sum() / (ref * ref).sum() / EPS[precision])
+        gain.append(np.mean(got))
+    assert np.sqrt(np.mean(np.square(gain))) <= (0.28 if precision == 1 else (0.41 ** 2 + 0.28 ** 2) ** 0.5)
