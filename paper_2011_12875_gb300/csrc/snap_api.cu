@@ -498,7 +498,6 @@ snap::WorkArgs make_args(snap_ctx* c, int n, int K) {
   a.K = K;
   a.twojmax = c->twojmax;
   a.H = c->tab.H;
-  a.lmax = c->tab.lmax;
   a.rcut = c->rcut;
   a.rfac0 = c->rfac0;
   a.rmin0 = c->rmin0;

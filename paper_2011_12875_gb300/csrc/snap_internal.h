@@ -58,7 +58,10 @@ constexpr int kMaxTwoJ = 14;
 constexpr int kYcChunk = 256;  // words of a compute_Y stream chunk (snap_tables.h)
 constexpr int kYcOuts = 8;     // most outputs of a compute_Y task
 constexpr int kYcTask = 4 + 2 * kYcOuts;
-constexpr long kYcWhole = 1000;  // cost from which a task's sum is split in two
+// Cost from which a task's sum is split in two.  compute_Y, 2000 atoms, us, from 300 /
+// 1000 / 3000 / never: FP32 2J8 34.1 / 33.8 / 32.6 / 36.3, 2J14 388 / 388 / 388 / 491; FP64 2J6
+// 60 / 61 / 70 / 72, 2J8 170 / 170 / 171 / 174.
+constexpr long kYcWhole = 1000;
 constexpr int kPairFix = 8;  // most steps of a class (HostTables::pair_fix)
 constexpr int kUUnit = 8;  // words of a compute_U unit (HostTables::u_units)
 constexpr int kYcNan = 0x7FFF;  // exponent of an output whose coefficients are not finite
@@ -210,7 +213,7 @@ __host__ __device__ constexpr int pair_key(int k, int ix, int iy, int iz, long n
 
 // What a kernel reads stands together: every CTA fetches its lines of it.
 struct WorkArgs {
-  int n, K, twojmax, H, lmax;
+  int n, K, twojmax, H;
   double rcut, rfac0, rmin0, wself, beta0;
   double inv_span;  // 1 / (rcut - rmin0)
   double th_scale;  // rfac0 / (rcut - rmin0): theta0 / pi = th_scale (r - rmin0)

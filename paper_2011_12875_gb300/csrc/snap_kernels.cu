@@ -31,23 +31,12 @@ __device__ __forceinline__ cx<R> mk(R re, R im) {
   c.im = im;
   return c;
 }
-// conj(a) * b
-template <typename R>
-__device__ __forceinline__ cx<R> conj_mul(cx<R> a, cx<R> b) {
-  return mk<R>(a.re * b.re + a.im * b.im, a.re * b.im - a.im * b.re);
-}
 // x * y + z with one rounding (complex multiply-adds are written as chains
 // of these, two a component)
 template <typename R>
 __device__ __forceinline__ R fmr(R x, R y, R z) {
   if constexpr (sizeof(R) == 4) return fmaf(x, y, z);
   else return fma(x, y, z);
-}
-
-// a * b
-template <typename R>
-__device__ __forceinline__ cx<R> mul(cx<R> a, cx<R> b) {
-  return mk<R>(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re);
 }
 
 template <typename R>

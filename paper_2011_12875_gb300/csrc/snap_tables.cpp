@@ -157,7 +157,6 @@ void half_elem(int tt, int xa, int xb, int& idx, int& conj, double& sgn) {
 void HostTables::build(int J2) {
   twojmax = J2;
   H = half_size(J2);
-  lmax = half_layer_size(J2);
   half_tmm.clear();
   for (int t = 0; t <= J2; ++t)
     for (int mb = 0; 2 * mb <= t; ++mb)

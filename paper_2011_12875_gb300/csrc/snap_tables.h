@@ -14,7 +14,7 @@ struct ZTrip {
 };
 
 struct HostTables {
-  int twojmax = 0, H = 0, lmax = 0, ncoeff = 0;
+  int twojmax = 0, H = 0, ncoeff = 0;
   std::vector<int> half_tmm;
   std::vector<ZTrip> ztrip;
   std::vector<double> cg;

@@ -173,7 +173,8 @@ def half_index(twojmax: int, t: int, ma: int, mb: int) -> int:
 
 
 def yi_host(twojmax: int, beta, u_half, precision: int = MIXED) -> np.ndarray:
-    """compute_Y's term list for one atom on the host in FP64 (snap_yi_host):
+    """compute_Y's stream of coefficients walked on the host for one atom
+    (snap_yi_host; MIXED in FP64 arithmetic, FP64 in the kernel's fixed point):
     u_half [H][2] -> Y [H][2], half layout.  No GPU work."""
     H = half_size(twojmax)
     beta = np.ascontiguousarray(beta, dtype=np.float64)
