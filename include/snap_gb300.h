@@ -229,7 +229,8 @@ int snap_bispectrum_deriv_batch(snap_ctx* ctx, int nconf, const int* natoms, con
  *  yi_layout: 0 = compute_Y with a warp of 32 atoms (lanes = atoms, the
  *    block's Ulisttot staged by TMA; the paper's AoSoA layout, Sec. V-B),
  *    1 = a warp per atom (its Ulisttot staged in shared memory, lanes over
- *    output elements), the layout the paper compares it with.
+ *    output elements), the layout the paper compares it with; its list of
+ *    terms is made and uploaded when it is first chosen (synchronous).
  * col_warps and yi_waves change no result bit; yi_layout changes the
  * compute_Y kernel and may change rounding.  snap_autotune times every
  * combination of col_warps in {2, 4, 8} with yi_waves in {1, 2, 4} (layout 0)

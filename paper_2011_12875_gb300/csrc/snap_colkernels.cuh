@@ -1,5 +1,5 @@
-// snap_colkernels.cuh -- compute_U (FP32 up to 2J = 9) and the tangent of
-// Ulisttot with the layer recursion in registers, one lane per half-matrix column.
+// snap_colkernels.cuh -- compute_U (FP32 up to 2J = 9, FP64 up to 5) and the tangent
+// of Ulisttot with the layer recursion in registers, one lane per half-matrix column.
 //
 // Eq. (hysphrecur) of arXiv:2011.12875 builds u_t from u_{t-1}; element
 // (ma, mb) only reads elements (ma, mb) and (ma-1, mb) of the previous layer,

@@ -187,12 +187,12 @@ __device__ __forceinline__ void cp_async_wait() {
 // a load) and the vectors about 0.4.  The dense forms hold 7% of zero
 // coefficients at 2J14.  What bounds it now is issue: a packed FMA (two cycles of
 // its pipe) comes with 1.6 other instructions (unpacking the vectors, heads,
-// loops), on 16 warps an SM (2J14, 2000 atoms: issue slots 53% used, shared
-// memory 42%, FMA pipe 36% of the launch).
-// Measured, list of terms -> now: FP32, 2000 atoms, 2J8 41 -> 35 us, 2J11 199 ->
-// 120, 2J14 845 -> 388; 16000 atoms, 2J8 218 -> 179, 2J14 6005 -> 2809; FP64 (in
-// fixed point, below), 2000 atoms, 2J8 404 -> 170, 2J11 2388 -> 820, 2J14 9335 ->
-// 3039; 128 atoms, 2J8 119 -> 28.
+// loops), on 16 warps an SM (2J14, 2000 atoms: issue slots 62% used, shared
+// memory 59%, FMA pipe 52%).
+// Measured, list of terms -> now: FP32, 2000 atoms, 2J8 41 -> 34 us, 2J11 199 ->
+// 119, 2J14 845 -> 388; 16000 atoms, 2J8 218 -> 178, 2J14 6005 -> 2809; FP64 (in
+// fixed point, below), 2000 atoms, 2J8 404 -> 170, 2J11 2390 -> 821, 2J14 9344 ->
+// 3042; 128 atoms, 2J8 119 -> 28.
 // Chunks of a warp's ring
 __host__ __device__ constexpr int yc_slots(int rsize) { return rsize == 8 ? 2 : 3; }
 // Warps of a CTA: one CTA an SM above 2J = 9 (the block's U fills its shared

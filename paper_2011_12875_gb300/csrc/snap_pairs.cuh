@@ -30,9 +30,9 @@
 // step use the same ones) and of Horner's scheme (24 a class): about 1,450 a
 // pair at 2J8 against 4,030, every lane a pair.  FP64 is bound by the FP64 pipe
 // either way; FP32 by the latency of about three warps a scheduler.  Measured,
-// 2000 atoms of 26 neighbours, before -> now: 2J8 FP64 725 -> 138 us, 2J14 FP64
-// 2850 -> 494, 2J8 FP32 38.1 -> 12.2, 2J14 FP32 137 -> 26.6 (16000 atoms: 1092 ->
-// 178); 128 atoms at 2J8 FP64 74 -> 26.
+// 2000 atoms of 26 neighbours, before -> now: 2J8 FP64 725 -> 141 us, 2J14 FP64
+// 2850 -> 512, 2J8 FP32 37 -> 12.7, 2J14 FP32 137 -> 28.1 (16000 atoms: 1094 ->
+// 197); 128 atoms at 2J8 FP64 74 -> 27.
 #pragma once
 #include <algorithm>
 #include <cmath>

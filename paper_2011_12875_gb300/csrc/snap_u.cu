@@ -20,10 +20,12 @@
 // with a lane a column (31% of the lanes idle).  FP64 is bound by the FP64 pipe
 // (a warp's multiply-add takes 15 cycles of an SM) and by SMs that hold one CTA
 // more than others; FP32 by latency and instruction fetch, which is why the CTAs'
-// warps run the same code and FP32 takes this form only above 2J = 9.  Neighbour
-// build and compute_U together, before -> now, 2000 atoms: FP64 2J8 278 -> 164 us,
-// 2J11 690 -> 274, 2J14 1113 -> 384; FP32 2J11 57 -> 50, 2J14 86 -> 57, 16000 atoms
-// 556 -> 347; 128 atoms FP64 2J8 58 -> 53.
+// warps run the same code.  A block's slots follow one another, so a launch
+// takes 30 us and more in FP64 however few the atoms: FP64 takes this form above
+// 2J = 5 and FP32 above 2J = 9 (u_by_layers).  Neighbour build and compute_U
+// together, before -> now, 2000 atoms: FP64 2J6 153 -> 116 us, 2J8 278 -> 165, 2J11 692
+// -> 278, 2J14 1146 -> 397; FP32 2J11 57 -> 53, 2J14 84 -> 61, 16000 atoms 561 -> 365;
+// 128 atoms FP64 2J8 59 -> 48.
 #include <algorithm>
 
 #include "snap_geom.cuh"
