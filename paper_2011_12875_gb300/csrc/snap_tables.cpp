@@ -454,6 +454,9 @@ std::vector<int> HostTables::pair_classes() const {
       if (steps > 1) cls.push_back(st | steps << 16);
       st += steps;
     }
+  // longest first, those of a length together: a warp takes several, its lanes then
+  // run the same code (fused dE, 128 atoms 2J14: 57 us, in the classes' own order 59)
+  std::stable_sort(cls.begin(), cls.end(), [](int x, int y) { return x >> 16 > y >> 16; });
   return cls;
 }
 

@@ -68,8 +68,8 @@ struct HostTables {
   std::vector<double> pair_norm, pair_norm_fix, pair_weight, pair_ab, pair_fix;
   // What the kernels take of these.  pair_scales: a step's step_scale, norm (x
   // weight), and pair_recursion: its rec_ab (snap_closed.cuh), in FP32 with what
-  // the rounding leaves off; pair_classes: the classes of several steps, first
-  // step | steps << 16.
+  // the rounding leaves off; pair_classes: the classes of several steps, longest
+  // first, first step | steps << 16.
   std::vector<double> pair_scales(bool fp64, bool weighted) const;
   std::vector<double> pair_recursion(bool fp64) const;
   std::vector<int> pair_classes() const;
